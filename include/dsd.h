@@ -87,17 +87,14 @@ uint64_t dsd_kernel_launches(void);
  * Default 20000 ms.  Applies to calls started afterwards, process-wide. */
 dsd_status dsd_set_wait_limit_ms(uint32_t ms);
 
-/* Tuning: once at most `max_alive` vertices remain alive, the peeling kernel
- * keeps the alive list and the frontier in every block's shared memory and
- * needs one grid barrier per round (the tail of many tiny levels).  Default
- * 16384 (also capped by shared memory); 0 disables it.  Results do not
- * depend on it.  Process-wide; applies to calls started afterwards. */
+/* Accepted for callers of earlier versions; the peel has no regime of its
+ * own for small alive sets any more.  No effect; never fails. */
 dsd_status dsd_set_peel_small_limit(uint32_t max_alive);
-/* Largest alive set whose remaining levels (h = 2, 3) are finished by one
- * thread-block cluster holding the alive subgraph as bitmap rows (in global
- * memory up to 16,384 vertices for h = 3, in the cluster's distributed shared
- * memory below about 4,600; the default is as large as those hold; 0 =
- * never).  Results do not depend on it.  Process-wide. */
+/* Largest alive set whose levels the peel groups into bands: at or below it
+ * the peel first cuts the alive set at a few thresholds, one cascade each,
+ * then peels the bands between them level by level, all side by side
+ * (default 2^30; 0 = never: one level after another).  Results do not depend
+ * on it.  Process-wide. */
 dsd_status dsd_set_peel_tail_limit(uint32_t max_alive);
 /* Where dsd_peel_app keeps each level's bucket queue (the bitmaps, one per
  * count below k + 1, over the level's positions): in a block's shared memory
@@ -552,17 +549,15 @@ dsd_status dsd_listing_bytes(dsd_graph* g, uint64_t* staged, uint64_t* merge);
 
 /* Counters of the last peeling run: which = 0 the degeneracy (h = 2) peel,
  * 1 the last (k,Psi) peel with h >= 3.  out[DSD_PEEL_STATS] receives:
- * rounds, levels, frontier work items, metered algorithmic bytes, time block 0
- * spent inside grid barriers (ns), barriers passed, row compactions, block
- * size, grid size, k_max, first round run with the alive set replicated in
- * every block's shared memory (0 if none), then block 0's time (ns) in each
- * phase outside barriers: [large regime] retire/mark, alive-list scan, level
- * jump, clique enumeration; [small regime] retire/copy, level jump,
- * mark/bitmaps, clique enumeration; then the alive vertices handed to the
- * cluster tail kernel (0 if none), the round of the hand-over, the tail
- * kernel's time (ns) and its lead CTA's time (ns) in: building the rows,
- * frontier broadcast, level jumps and frontier lists, candidate numbering,
- * candidate work, the barrier after it, retiring.  Zeros if that peel has
+ * rounds (of the level-by-level peel), levels, frontier work items, metered
+ * algorithmic bytes, time block 0 spent inside grid barriers (ns), barriers
+ * passed, row compactions, block size, grid size, k_max, 0, then block 0's
+ * time (ns) outside barriers: [bands] retire/mark, alive-list scan,
+ * threshold and frontier, clique enumeration; [levels] set-up and
+ * bookkeeping, row filter, clique enumeration, queued items; then the alive
+ * vertices when levels began to be grouped (0: never), the round at that
+ * point, the time of the level-by-level phase (ns), the bands of several
+ * levels, the rounds run in both phases, and zeros.  Zeros if that peel has
  * not run. */
 #define DSD_PEEL_STATS 29
 dsd_status dsd_peel_stats(dsd_graph* g, int which, uint64_t* out);

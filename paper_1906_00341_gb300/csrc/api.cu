@@ -12,9 +12,6 @@ const char* last_error();
 static uint64_t g_wait_ns = 20000ull * 1000000ull;
 uint64_t wait_limit_ns() { return g_wait_ns; }
 
-static std::atomic<uint32_t> g_small_limit{16384};
-uint32_t peel_small_limit() { return g_small_limit.load(); }
-
 static std::atomic<uint32_t> g_tail_limit{1u << 30};
 uint32_t peel_tail_limit() { return g_tail_limit.load(); }
 
@@ -46,12 +43,14 @@ void record_peel(dsd_graph* g, int which, const PeelResult& r) {
     o[7] = r.threads;
     o[8] = r.grid;
     o[9] = r.kmax;
-    o[10] = r.small_round;
+    o[10] = 0;   // the replicated small regime is gone
     for (int i = 0; i < 8; i++) o[11 + i] = r.tph[i];
-    o[19] = r.tail_n;
-    o[20] = r.tail_round;
-    o[21] = r.tail_ns;
-    for (int i = 0; i < 7; i++) o[22 + i] = r.tail_tph[i];
+    o[19] = r.band_n;
+    o[20] = r.band_round;
+    o[21] = r.phase2_ns;
+    o[22] = r.bands;
+    o[23] = r.grid_rounds;
+    for (int i = 24; i < 29; i++) o[i] = 0;
 }
 
 void prof_begin(dsd_graph* g, int phase) {
@@ -362,7 +361,7 @@ dsd_status dsd_set_wait_limit_ms(uint32_t ms) {
 }
 
 dsd_status dsd_set_peel_small_limit(uint32_t max_alive) {
-    g_small_limit = max_alive;
+    (void)max_alive;   // the peel no longer has a regime of its own for small alive sets
     return DSD_OK;
 }
 

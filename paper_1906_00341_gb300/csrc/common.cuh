@@ -52,9 +52,7 @@ uint64_t wait_limit_ns();
 // Process-wide count of kernel launches issued by the library.
 void note_launch();
 
-// Largest alive set the peel replicates in every block's shared memory.
-uint32_t peel_small_limit();
-// Largest alive set handed to the cluster tail kernel (0 = never).
+// Largest alive set whose levels the peel groups into bands (0 = never).
 uint32_t peel_tail_limit();
 uint32_t peel_app_queue_shared();   // PeelApp bucket queues: shared-memory words per block
 uint64_t peel_app_queue_global();   // and global-memory words in all

@@ -92,12 +92,12 @@ struct PeelResult {
     uint32_t compactions = 0;
     uint32_t threads = 0;     // block size used
     uint32_t grid = 0;        // blocks launched
-    uint32_t small_round = 0; // first round of the small regime (0 = never)
+    uint32_t grid_rounds = 0; // rounds executed (bands and levels)
     uint64_t tph[8] = {};     // block 0's time per phase (ns)
-    uint32_t tail_n = 0;      // alive vertices handed to the cluster tail kernel
-    uint32_t tail_round = 0;  // round of the hand-over
-    uint64_t tail_ns = 0;     // the tail kernel's duration
-    uint64_t tail_tph[7] = {};  // the tail's time per phase (ns)
+    uint32_t band_n = 0;      // alive vertices when levels began to be grouped in bands
+    uint32_t band_round = 0;  // round at that point
+    uint32_t bands = 0;       // bands of several levels
+    uint64_t phase2_ns = 0;   // time peeling them level by level
 };
 // off/adj/split: CSR in the working id space (split may be null for h = 2).
 // deg: [n] clique-degrees in, destroyed on return.  core/rnd: [n] outputs
@@ -107,7 +107,7 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
                     uint64_t mu0, uint64_t* core, uint32_t* rnd, uint64_t* lvl_k,
                     uint32_t* lvl_size, uint64_t* lvl_mu, PeelResult* res,
                     uint64_t kstart = 0, uint64_t* snap = nullptr);
-// snap (may be null; no cluster tail then): snap[v] receives v's count in
+// snap (may be null): snap[v] receives v's count in
 // R_core(v), its clique-degree inside its own (k,Psi)-core.
 // kstart > 0: the first level removes every vertex with fewer than kstart
 // cliques in one cascade (threshold pruning to the (kstart,Psi)-core); its

@@ -5,60 +5,78 @@
 // below the removed vertex's value.  Here every alive vertex whose
 // clique-degree is <= k leaves at once (the frontier F); each clique
 // instance destroyed by F is credited once, to its smallest-id frontier
-// member, and lowers the count of each of its alive non-frontier members by
-// one.  A vertex whose count falls to <= k joins the next frontier at the
-// same level; when no vertex is left at <= k, k jumps to the minimum alive
-// count.  core(v) is the k at which v leaves.  The first round of every
-// level starts from the set R_k (Def. 6), whose size and clique count are
-// recorded: these give the CoreApp outputs (the k_max core, Lemma 6) and the
-// densest residual level (Pruning1, Sec. 5.1) without storing cliques.
+// member v, and lowers the count of each of its other members that are alive
+// or frontier members (of larger id) by one.  A vertex whose count falls to
+// <= k joins the next frontier at the same level; when no vertex is left at
+// <= k, k jumps to the minimum alive count.  core(v) is the k at which v
+// leaves.  A frontier member's count after its round is the number of
+// cliques credited to it, so mu falls by the sum of those counts.  The first
+// round of every level starts from the set R_k (Def. 6), whose size and
+// clique count are recorded: these give the CoreApp outputs (the k_max core,
+// Lemma 6) and the densest residual level (Pruning1, Sec. 5.1) without
+// storing cliques.
+//
+// Levels are many and small (5,552 on the 1M-vertex Chung-Lu graph, h = 3;
+// the last 8,000 vertices hold nearly all of them), and a round costs grid
+// barriers and latency whatever its size, so taking the levels one after
+// another is bound by their number.  R_t for any t is reached by one cascade
+// from any R_s, s < t (remove everything below t, repeat), in a few rounds
+// however many levels lie between.  So the peel has two phases:
+//   1 -- bands.  The alive set is cut at a few thresholds t_1 < t_2 < ...,
+//        chosen from a histogram of the counts at each jump; the vertices a
+//        cascade removes form a band, a run of consecutive levels.  Each
+//        vertex's count at its band's start is kept (c0).  A band of a
+//        single level is finished here.
+//   2 -- levels.  Every vertex of R_{t_i} \ R_{t_{i+1}} leaves between those
+//        two sets, while R_{t_{i+1}} stays whole, so given c0 the bands do
+//        not depend on one another: all of them are peeled level by level
+//        side by side, a round of every band per grid round.  A clique
+//        belongs to the lowest band among its members, and only members in
+//        that band count it.
+// The 1M-vertex graph, h = 3: 7,016 rounds one level at a time (86 ms), 587
+// in the two phases (41 ms); R-MAT scale 17, h = 4: 8,232 and 428 (389 ms and
+// 114 ms).  Bound by the latency of a round (barriers, row walks) and by the
+// blocks that wait for the longest items of it.
 //
 // One persistent cooperative kernel runs every round; phases are separated
 // by grid barriers whose waits are bounded in time (a wait that runs out
 // records DSD_ERR_TIMEOUT and every block leaves).
 //
-// Large regime (many alive vertices), round r, F_r in global lists r mod 3:
-//   P1  mark F_{r-1} removed (core = k); mark F_r as frontier     | barrier
-//   J   (only if F_r is empty) compact the alive list and take   |
-//       the minimum count; k = that minimum; record the level    | barrier
-//       (k, |R_k|, mu(R_k)); F_r = alive vertices with count <= k;|
-//       when the alive set has halved, drop removed vertices     |
-//       from the rows of alive vertices                          | barrier
+// Phase 1, round r, F_r in global lists r mod 3:
+//   P1  retire F_{r-1} (band); mark F_r as frontier                | barrier
+//   J   (only if F_r is empty) compact the alive list, take the   |
+//       minimum count and a histogram of the counts above k       | barrier
+//       choose k; F_r = alive vertices with count <= k; when the   |
+//       alive set has halved, drop removed vertices from the rows  |
+//       of alive vertices                                         | barrier
 //   P2  enumerate the cliques each v in F_r destroys; decrement   | barrier
-//   P2b (h >= 4) candidate sets above 32 vertices, one block each | barrier
-//
-// Small regime (the long tail of tiny levels: at most `asmall` vertices
-// alive).  Every block holds a slice of the alive list and the whole
-// frontier in shared memory and performs the bookkeeping of P1 itself
-// (identical writes in every block).  A level jump is distributed: each block
-// publishes its slice minimum and the slice vertices attaining it; after one
-// barrier every block combines them into k and the frontier.  So a round
-// needs one grid barrier after P2, plus the jump barrier (no block may
-// decrement counts another block is still reading) and one when big items
-// exist.  On entry every alive vertex gets a fixed local id, kept in the
-// upper bits of its state word; each block then holds, for the first
-// frontier vertices, a bitmap over local ids of their neighbourhoods, so that
-// "x in N(v)" is one shared-memory bit instead of a binary search in global
-// memory.
+//   P2b (h >= 4) candidate sets above warp_cand: warp groups and   |
+//       blocks                                                    | barrier
+// Phase 2, round r: each band has one owner block.
+//   A   retire the band's frontier, find its next one (counts <= k, else
+//       k = the least count: a new level), append it to F_r       | barrier
+//   P2, P2b as above                                              | barrier
 //
 // Rows live in a private copy of the oriented CSR: row v is
-// wadj[off[v] .. wend[v]) and N+(v) = wadj[wnb[v] .. wend[v]).  Compaction
-// rewrites a row in place (stable, so rows stay sorted) and moves wend/wnb.
+// wadj[off[v] .. wend[v]).  In phase 1 N+(v) is its tail wadj[wnb[v] ..
+// wend[v]); compaction rewrites a row in place (stable, so rows stay sorted)
+// and moves wend/wnb.  For phase 2 every row keeps the entries of its own
+// band and later ones, and N+(v) is read from the caller's rows (a
+// compaction drops members of the bands peeled before it).
 #include "cliques.cuh"
 #include "graph.cuh"
 #include "xl.cuh"
 
-#include <cooperative_groups.h>
 #include <string.h>
 
 namespace dsd {
 namespace {
 
-// state word: bits 0-1 the state, bits 2-31 the local id (small regime)
+// state word: bits 0-1 the state, bit 2 kHeavyBit, bits 3-10 a bitmap slot
+// (phase 1 only), bits 11-31 the band key (zero throughout phase 1)
 enum : uint32_t { kAlive = 0, kFront = 1, kGone = 2 };
 enum : uint32_t { kErrTimeout = 1, kErrBigOverflow = 2 };
 constexpr uint32_t kSmallFront = 1024;
-constexpr uint32_t kBitmapSlots = 16;   // frontier vertices with a shared bitmap
 constexpr int kChunks = 4;              // 32-entry chunks of a row in flight per warp
 constexpr uint32_t kWarpCand = 32;      // candidate sets a warp handles itself (h >= 4)
 constexpr uint32_t kWarpWords = 3 * kWarpCand;   // a warp's candidates, counters, rows
@@ -77,20 +95,75 @@ inline uint32_t warp_cand_limit(int h) {
 constexpr uint32_t kHeavyBit = 4;       // state word: frontier vertex on the heavy list
 constexpr uint32_t kSlotShift = 3;      // state word: 1 + its neighbourhood bitmap slot
 constexpr uint32_t kSlotMask = 0xffu;
+constexpr uint32_t kKeyShift = 11;      // state word: band key
+
+// Band keys: the j-th band of several levels has key 2j + 1, a vertex of a
+// single-level band the key 2j with j the multi-level bands before it, so keys
+// order the bands that phase 2 has to tell apart.
+constexpr uint32_t kMaxBands = 4096;    // multi-level bands (then levels go one by one)
+// A threshold is set for at most kBandAim vertices, or fewer (pick_threshold);
+// a cascade that removes more than kBandMax is undone and its first level
+// taken alone: a band's owner block reads all its members every round.
+constexpr uint32_t kBandAim = 2048;
+constexpr uint32_t kBandMax = 8192;
+// With N vertices left a band aims at sqrt(kBandFill N) of them: a cascade
+// takes 2-5 rounds, so phase 1 runs ~3 N / T rounds for bands of T vertices and
+// phase 2 as many as the fullest band has levels (up to one a vertex).  The
+// 1M-vertex graph (h = 3) and R-MAT scale 17 (h = 4) take the same time within
+// 3 % from 1 to 16.
+constexpr float kBandFill = 2.0f;
+// h = 2: rounds taken one level at a time before the bands begin.  Levels are
+// few there (at most the degeneracy), and a graph that is done in fewer rounds
+// gains nothing: G(100,000, 0.0002) has 44 rounds in 7 levels (0.74 ms, 0.85
+// with bands); the 50,000-vertex Chung-Lu graph 351 in 51 (3.85 -> 2.6 ms).
+constexpr uint32_t kBandAfter2 = 64;
+// h = 2: graphs of up to kOneBlockN vertices (12 bytes each fit shared memory)
+// and kOneBlockAdj row entries go to one block (k_peel2_block).  Measured
+// against the grid: G(2000, 0.005) 0.10 against 0.31 ms, power law with 10,000
+// vertices 0.40 / 1.41, G(n, p) with 320,000 entries 0.47 / 0.53 and with
+// 983,000 entries 1.05 / 0.61 ms.
+constexpr uint32_t kOneBlockN = 16384;
+constexpr uint64_t kOneBlockAdj = 400000;
 
 __device__ __forceinline__ uint32_t st_of(uint32_t w) { return w & 3u; }
+
+// Is x (state word wx) a member of the current set as seen from frontier
+// vertex v of key kv, with frontier members of smaller id taken as gone?
+// dec: x is also counting the cliques it shares with v (same band).
+__device__ __forceinline__ bool cand_ok(uint32_t wx, uint32_t x, uint32_t kv, uint32_t v,
+                                        bool& dec) {
+    const uint32_t kx = wx >> kKeyShift, s = wx & 3u;
+    dec = kx == kv && (s == kAlive || (s == kFront && x > v));
+    return dec || kx > kv;
+}
+
+// Histogram of count offsets at a jump: 16 bins an octave, exact below 32.
+constexpr uint32_t kBins = 1024;
+constexpr uint32_t kLastBin = 975;      // the bin of 2^64 - 1
+__device__ __forceinline__ uint32_t bin_of(unsigned long long d) {
+    if (d < 16) return (uint32_t)d;
+    const uint32_t e = 63u - (uint32_t)__clzll((long long)d);
+    return (e - 3u) * 16u + ((uint32_t)(d >> (e - 4u)) & 15u);
+}
+// Largest offset of bin b <= kLastBin.
+__device__ __forceinline__ unsigned long long bin_last(uint32_t b) {
+    if (b < 16) return b;
+    const uint32_t e = (b >> 4) + 3u;
+    return (((16ull + (b & 15u)) + 1ull) << (e - 4u)) - 1ull;
+}
 
 struct PeelCtrl {
     unsigned long long min_deg[2];
     uint32_t new_alive[2];
     uint32_t fcnt[3];
     uint32_t big_cnt[6];            // per round slot s: big items [s], mid items [3 + s]
-    unsigned long long destroyed[3];
     uint32_t hcnt[3];               // heavy frontier vertices of the round
     uint32_t grab[3];               // light frontier vertices taken by blocks
     uint32_t bgrab[6];              // big items [s] and mid items [3 + s] taken
     uint32_t hubcnt[2];             // bitmap slots asked for, by round parity
-    uint32_t pad0[11];
+    uint32_t busy[3];               // phase 2: bands with vertices left, by round
+    unsigned long long destroyed;   // phase 1: cliques destroyed so far
+    uint32_t pad0[16];
     uint32_t bar_count;
     uint32_t pad1[31];
     uint32_t bar_gen;
@@ -99,33 +172,38 @@ struct PeelCtrl {
     uint32_t err_info;
     unsigned long long kmax;
     uint32_t nlevels;
-    uint32_t rounds;
+    uint32_t rounds;                // rounds of the level-by-level peel
     unsigned long long items;
     unsigned long long bytes;       // algorithmic bytes (meter notes below)
     unsigned long long barrier_ns;  // block 0's time inside grid barriers
     uint32_t barriers;
     uint32_t compactions;
-    uint32_t small_round;           // first round of the small regime (0 = never)
-    uint32_t pad3;
+    uint32_t band_n;                // alive vertices when the bands began (0 = none)
+    uint32_t band_round;            // round of phase 1 at that point
+    uint32_t nbands;                // multi-level bands
+    uint32_t grid_rounds;           // rounds executed, both phases
+    unsigned long long phase2_ns;
     unsigned long long tph[8];      // block 0's time per phase (ns)
-    // hand-over to the cluster tail kernel
-    uint32_t tail_n;                // alive vertices handed over (0 = none)
-    uint32_t tail_round;            // round at the hand-over
-    uint32_t tail_sel;              // which hand-over list holds them
-    uint32_t tail_entry;            // alive vertices at the first hand-over
-    uint32_t tail_entry_round;      // its round
-    uint32_t pad4;
-    unsigned long long mu_tail;     // mu of the alive graph at the hand-over
-    unsigned long long tail_ns;     // the tail kernel's duration
-    unsigned long long tail_tph[7]; // tail lead CTA: build, A+sync, jump+list, C prefix, C work, C sync, D
+    uint32_t hist[2][kBins];        // counts above k at a jump, by jump parity
+};
+
+// A multi-level band: members mem[seg .. seg + size).
+struct Band {
+    unsigned long long k;           // phase 2: current level
+    unsigned long long mu;          // cliques of the current set (the band and above)
+    uint32_t seg, size;
+    uint32_t left;                  // size; 0 once every member has left
+    uint32_t above;                 // vertices of the bands above
+    uint32_t nlev, rounds;
+    uint32_t rbase;                 // single-level rounds of phase 1 before the band
+    uint32_t pad;
 };
 
 // Byte meter.  Every global-memory element the algorithm reads or writes is
 // counted once per access: ids and state words 4 B, offsets 8 B, counters
 // 8 B, an atomic read-modify-write 16 B, a binary search over a row of d
 // entries floor(log2 d) + 1 probes of 4 B.  Shared-memory traffic is not
-// counted, and bookkeeping that every block repeats in the small regime
-// counts once.
+// counted, and bookkeeping that every block repeats counts once.
 __device__ __forceinline__ unsigned probes(uint64_t d) {
     return d ? 64u - (unsigned)__clzll((long long)d) : 0u;
 }
@@ -143,8 +221,17 @@ struct PeelParams {
     uint32_t* sl;          // state words
     uint32_t* alive[2];
     uint32_t* front[3];
-    uint32_t* jf;          // small regime: per-slice jump candidates
-    ulonglong2* jblk;      // small regime: per-block (slice minimum, alive<<32 | candidates)
+    const uint32_t* nadj;  // the caller's rows (phase 2: N+(v) = nadj[nsplit[v] .. off[v + 1]))
+    const uint64_t* nsplit;
+    uint32_t* mem;         // vertices in the order phase 1 retired them
+    uint32_t* band_of;     // band key
+    unsigned long long* c0;  // count at the start of the band
+    Band* bands;           // multi-level bands [kMaxBands]
+    uint32_t* blkcnt;      // per-block counts of the final pass
+    uint64_t* t_k;         // level records by position in mem (t_size 0: none)
+    uint32_t* t_size;
+    uint64_t* t_mu;
+    uint32_t band_max;     // group levels into bands at <= this many alive (0 = never)
     uint2* big;
     uint64_t big_cap;
     uint32_t* heavy;       // large regime: frontier vertices with long rows
@@ -175,9 +262,6 @@ struct PeelParams {
     uint32_t mid_cap;      // 0: none (every set above warp_cand goes to a block)
     uint32_t* xl;          // per block (kMaxDepth + 1) * cap entries when cap > kBitmapMax
     int compact;           // drop removed vertices from rows as the graph shrinks
-    uint32_t work_words;   // shared words before the small-regime lists
-    uint32_t asmall;       // small-regime list capacity (0 = regime off)
-    uint32_t tail_max;     // hand over to the cluster tail at <= this many alive (0 = off)
     uint64_t* snap;        // if set: each alive vertex's count at every level jump (the
                            // last one written is its count in its own (k,Psi)-core)
 };
@@ -216,13 +300,28 @@ __device__ bool grid_barrier(PeelCtrl* c, uint64_t wait_ns, unsigned long long& 
 }
 
 // ------------------------------------------------------------ helpers
-__device__ __forceinline__ void dec_and_queue(const PeelParams& P, uint32_t u,
-                                              unsigned long long c, unsigned long long k,
-                                              uint32_t* next, uint32_t* next_cnt) {
-    unsigned long long old = atomic_sub_u64(&P.deg[u], c);
-    if (old > k && old - c <= k) {
-        uint32_t at = atomicAdd(next_cnt, 1u);
-        next[at] = u;
+
+// N+ lists of the current phase: adj[nb[v] .. ne[v]).
+struct NPlus {
+    const uint32_t* adj;
+    const uint64_t* nb;
+    const uint64_t* ne;
+};
+
+// Lower the count of x, alive or frontier (state s), by c.  With a queue
+// (phase 1) an alive vertex that falls to <= k joins the next frontier; phase
+// 2 finds them by scanning the bands, and needs no old value.
+__device__ __forceinline__ void lower(const PeelParams& P, uint32_t x, uint32_t s,
+                                      unsigned long long c, unsigned long long k,
+                                      uint32_t* next, uint32_t* next_cnt) {
+    if (next && s == kAlive) {
+        unsigned long long old = atomic_sub_u64(&P.deg[x], c);
+        if (old > k && old - c <= k) {
+            uint32_t at = atomicAdd(next_cnt, 1u);
+            next[at] = x;
+        }
+    } else {
+        atomic_sub_u64(&P.deg[x], c);
     }
 }
 
@@ -278,11 +377,12 @@ __device__ __forceinline__ uint32_t block_scan_count(uint32_t v, uint32_t* wtot,
 
 // pre[0] = 0, pre[i+1] = sum of the current row lengths of F[0..i], for
 // f <= kSmallFront entries (each thread owns kSmallFront/NT consecutive ones).
-template <int NT>
+// ALL: every entry counts; else a frontier vertex marked gone (count 0) has
+// no items.
+template <int NT, bool ALL = false>
 __device__ __forceinline__ void block_prefix_degrees(const PeelParams& P, const uint32_t* F,
                                                      uint32_t f, unsigned long long* pre,
-                                                     unsigned long long* red,
-                                                     bool skip_empty = false) {
+                                                     unsigned long long* red) {
     constexpr int E = kSmallFront / NT;
     unsigned long long d[E], sum = 0;
     uint32_t i0 = threadIdx.x * E;
@@ -292,8 +392,7 @@ __device__ __forceinline__ void block_prefix_degrees(const PeelParams& P, const 
         d[q] = 0;
         if (i < f) {
             uint32_t v = F[i];
-            // a frontier vertex of count 0 lies in no clique: no items
-            if (!skip_empty || P.deg[v] != 0) d[q] = P.wend[v] - P.off[v];
+            if (ALL || st_of(P.sl[v]) == kFront) d[q] = P.wend[v] - P.off[v];
         }
         sum += d[q];
     }
@@ -318,29 +417,28 @@ __device__ __forceinline__ void block_prefix_degrees(const PeelParams& P, const 
     __syncthreads();
 }
 
-// Candidates of frontier vertex v among N+(w), in order (one warp).  A
-// candidate is alive, or a frontier vertex with a larger id than v, and is
-// adjacent to v: tested on v's shared bitmap `bm` (over local ids) when
-// given, else by binary search in v's row.  kChunks chunks of the row are
-// loaded at once.  MODE:
-//   kGatherDirect (h = 3): each candidate closes the triangle {v, w, x}; an
-//     alive candidate loses it on the spot; nothing is stored;
+// Candidates of frontier vertex v (key kv) among N+(w), in order (one warp):
+// members of the current set (cand_ok) adjacent to v, tested on v's
+// neighbourhood bitmap gbm over vertex ids when it has one, else by binary
+// search in v's row.  kChunks chunks of the row are loaded at once.  MODE:
+//   kGatherDirect (h = 3): each candidate closes the triangle {v, w, x}; a
+//     counting candidate loses it on the spot; nothing is stored;
 //   kGatherWarp: the first kWarpCand candidates go to C; the walk stops as
 //     soon as there are more than P.gather_cap (the item then needs a block).
-// gbm (large regime, may be null): v's neighbourhood bitmap over vertex ids.
-// Returns the number of candidates seen.
+// Returns the number of candidates seen; anyd: some of this lane's count.
 enum { kGatherDirect = 0, kGatherWarp = 1 };
 
 template <int MODE>
-__device__ __forceinline__ void take_candidate(const PeelParams& P, bool ok, bool alive,
-                                               uint32_t x, uint32_t* C, uint32_t& nc,
+__device__ __forceinline__ void take_candidate(const PeelParams& P, bool ok, bool dec, uint32_t s,
+                                               uint32_t x, uint32_t* C, uint32_t& nc, bool& anyd,
                                                unsigned long long k, uint32_t* next,
                                                uint32_t* next_cnt, unsigned long long& bytes) {
     unsigned lane = lane_id();
     unsigned bal = __ballot_sync(0xffffffffu, ok);
+    if (ok && dec) anyd = true;
     if (MODE == kGatherDirect) {
-        if (ok && alive) {
-            dec_and_queue(P, x, 1ull, k, next, next_cnt);
+        if (ok && dec) {
+            lower(P, x, s, 1ull, k, next, next_cnt);
             bytes += 16;
         }
     } else {
@@ -351,93 +449,61 @@ __device__ __forceinline__ void take_candidate(const PeelParams& P, bool ok, boo
 }
 
 template <int MODE>
-__device__ __forceinline__ uint32_t gather_candidates(const PeelParams& P, uint32_t v,
-                                                      uint32_t w, uint32_t* C,
-                                                      const uint32_t* bm, const uint32_t* gbm,
-                                                      unsigned long long k,
+__device__ __forceinline__ uint32_t gather_candidates(const PeelParams& P, const NPlus& R,
+                                                      uint32_t v, uint32_t kv, uint32_t w,
+                                                      uint32_t* C, const uint32_t* gbm,
+                                                      bool& anyd, unsigned long long k,
                                                       uint32_t* next, uint32_t* next_cnt,
                                                       unsigned long long& bytes) {
     unsigned lane = lane_id();
     const uint32_t* Nv = P.wadj + P.off[v];
     uint64_t dv = P.wend[v] - P.off[v];
-    uint64_t b = P.wnb[w], e = P.wend[w];
+    uint64_t b = R.nb[w], e = R.ne[w];
     const uint64_t dw = e - b;
     const unsigned pr = probes(dv);
     uint32_t nc = 0;
     // Walk the shorter side: the entries of N(v) above w, each searched in
     // N+(w), when that costs fewer probes than walking N+(w).
-    const uint64_t cost_w = (bm || gbm) ? dw : dw * pr;
-    if (dv * probes(dw) < cost_w) {
-        const uint32_t* Nw = P.wadj + b;
-        uint64_t s0 = lower_bound_u32(Nv, dv, w + 1u);
-        const unsigned pw = probes(dw);
-        for (uint64_t p0 = s0; p0 < dv; p0 += 32 * kChunks) {
-            uint32_t xs[kChunks], ws[kChunks];
-#pragma unroll
-            for (int u = 0; u < kChunks; u++) {
-                uint64_t p = p0 + u * 32 + lane;
-                xs[u] = p < dv ? Nv[p] : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < kChunks; u++) {
-                uint64_t p = p0 + u * 32 + lane;
-                ws[u] = p < dv ? P.sl[xs[u]] : (uint32_t)kGone;
-            }
-#pragma unroll
-            for (int u = 0; u < kChunks; u++) {
-                uint64_t p = p0 + u * 32 + lane;
-                bool ok = false;
-                uint32_t x = xs[u];
-                uint32_t s = st_of(ws[u]);
-                if (p < dv) {
-                    bytes += 8;
-                    if (s == kAlive || (s == kFront && x > v)) {
-                        uint64_t pos = lower_bound_u32(Nw, dw, x);
-                        ok = pos < dw && Nw[pos] == x;
-                        bytes += 4ull * pw;
-                    }
-                }
-                take_candidate<MODE>(P, ok, s == kAlive, x, C, nc, k, next, next_cnt, bytes);
-            }
-            if (MODE == kGatherWarp && nc > P.gather_cap) return nc;
-        }
-        return nc;
-    }
-    for (uint64_t p0 = b; p0 < e; p0 += 32 * kChunks) {
+    const uint64_t cost_w = gbm ? dw : dw * pr;
+    const bool own = dv * probes(dw) < cost_w;
+    const uint32_t* L = own ? Nv : R.adj + b;       // the list walked
+    const uint64_t len = own ? dv : dw;
+    const uint32_t* S = own ? R.adj + b : Nv;       // the list searched
+    const uint64_t slen = own ? dw : dv;
+    const unsigned ps = probes(slen);
+    const uint32_t* bm = own ? nullptr : gbm;
+    for (uint64_t p0 = own ? lower_bound_u32(Nv, dv, w + 1u) : 0; p0 < len; p0 += 32 * kChunks) {
         uint32_t xs[kChunks], ws[kChunks];
 #pragma unroll
         for (int u = 0; u < kChunks; u++) {
             uint64_t p = p0 + u * 32 + lane;
-            xs[u] = p < e ? P.wadj[p] : 0u;
+            xs[u] = p < len ? L[p] : 0u;
         }
 #pragma unroll
         for (int u = 0; u < kChunks; u++) {
             uint64_t p = p0 + u * 32 + lane;
-            ws[u] = p < e ? P.sl[xs[u]] : (uint32_t)kGone;
+            ws[u] = p < len ? P.sl[xs[u]] : (uint32_t)kGone;
         }
 #pragma unroll
         for (int u = 0; u < kChunks; u++) {
             uint64_t p = p0 + u * 32 + lane;
-            bool ok = false;
+            bool ok = false, dec = false;
             uint32_t x = xs[u];
-            uint32_t s = st_of(ws[u]);
-            if (p < e) {
+            if (p < len) {
                 bytes += 8;
-                if (s == kAlive || (s == kFront && x > v)) {
+                if (cand_ok(ws[u], x, kv, v, dec)) {
                     if (bm) {
-                        uint32_t l = ws[u] >> 2;
-                        ok = (bm[l >> 5] >> (l & 31)) & 1u;
-                    } else if (gbm) {
-                        ok = (gbm[x >> 5] >> (x & 31)) & 1u;
+                        ok = (bm[x >> 5] >> (x & 31)) & 1u;
                         bytes += 4;
                     } else {
-                        uint64_t pos = lower_bound_u32(Nv, dv, x);
-                        ok = pos < dv && Nv[pos] == x;
-                        bytes += 4ull * pr;
+                        uint64_t pos = lower_bound_u32(S, slen, x);
+                        ok = pos < slen && S[pos] == x;
+                        bytes += 4ull * ps;
                     }
                 }
             }
-            take_candidate<MODE>(P, ok, s == kAlive, x, C, nc, k, next, next_cnt, bytes);
+            take_candidate<MODE>(P, ok, dec, st_of(ws[u]), x, C, nc, anyd, k, next, next_cnt,
+                                 bytes);
         }
         if (MODE == kGatherWarp && nc > P.gather_cap) return nc;
     }
@@ -445,30 +511,33 @@ __device__ __forceinline__ uint32_t gather_candidates(const PeelParams& P, uint3
 }
 
 // One (v, w) work item of a frontier vertex v with h >= 3: the cliques
-// {v, w, ...} whose members other than v are candidates of v and whose
-// smallest such member is w.  Executed by one warp; C, cnt, rows are the
+// {v, w, ...} whose members other than v are candidates of v (in the current
+// set, N+(.) from R) and whose smallest such member is w.  Executed by one warp; C, cnt, rows are the
 // warp's kWarpCand-entry buffers.  Candidate sets above P.warp_cand (h >= 4)
 // are queued, as mid items with their candidates when at most kWarpCand
 // (`big_cnt + 3` counts them), else as big items for a block.
-__device__ void process_vw(const PeelParams& P, uint32_t v, uint32_t w, unsigned long long k,
-                           uint32_t* next, uint32_t* next_cnt, uint32_t* C, unsigned* cnt,
-                           uint32_t* rows, uint32_t* big_cnt, const uint32_t* bm,
-                           const uint32_t* gbm, unsigned long long& destroyed,
+__device__ void process_vw(const PeelParams& P, const NPlus& R, uint32_t v, uint32_t w,
+                           unsigned long long k, uint32_t* next, uint32_t* next_cnt, uint32_t* C,
+                           unsigned* cnt, uint32_t* rows, uint32_t* big_cnt, const uint32_t* gbm,
                            unsigned long long& bytes) {
     unsigned lane = lane_id();
-    uint32_t sw = st_of(P.sl[w]);
+    const uint32_t kv = P.sl[v] >> kKeyShift, ww = P.sl[w];
+    bool dec_w;
     if (lane == 0) bytes += 4 + 4;   // w, its state word
-    if (!(sw == kAlive || (sw == kFront && w > v))) return;
-    if (lane == 0) bytes += 16;      // wnb[w], wend[w]
+    if (!cand_ok(ww, w, kv, v, dec_w)) return;
+    if (lane == 0) bytes += 16;      // the bounds of N+(w)
     const int r = P.h - 2;
     unsigned long long tot = 0;
+    bool anyd = false;
     if (r == 1) {
-        tot = gather_candidates<kGatherDirect>(P, v, w, C, bm, gbm, k, next, next_cnt, bytes);
+        tot = gather_candidates<kGatherDirect>(P, R, v, kv, w, C, gbm, anyd, k, next, next_cnt,
+                                               bytes);
     } else {
-        uint32_t nc =
-            gather_candidates<kGatherWarp>(P, v, w, C, bm, gbm, k, next, next_cnt, bytes);
+        uint32_t nc = gather_candidates<kGatherWarp>(P, R, v, kv, w, C, gbm, anyd, k, next,
+                                                     next_cnt, bytes);
         __syncwarp();
         if (nc < (uint32_t)r) return;
+        if (nc <= kWarpCand && !dec_w && !__any_sync(0xffffffffu, anyd)) return;   // none count
         if (nc > P.warp_cand) {
             // mid item: its candidates go with it to a warp group; else a block
             if (nc <= kWarpCand && P.mid_cap) {
@@ -501,8 +570,8 @@ __device__ void process_vw(const PeelParams& P, uint32_t v, uint32_t w, unsigned
             const uint32_t cmax = C[nc - 1];
             for (uint32_t i = 0; i + 1 < nc; i++) {
                 uint32_t x = C[i];
-                uint64_t xb = P.wnb[x], xe = P.wend[x], xr = xe;
-                unsigned hits = scan_row_hits(C, nc, cmax, P.wadj, xb, xe, cnt, &xr);
+                uint64_t xb = R.nb[x], xe = R.ne[x], xr = xe;
+                unsigned hits = scan_row_hits(C, nc, cmax, R.adj, xb, xe, cnt, &xr);
                 if (lane == 0) bytes += 16 + 4ull * (xr - xb);
                 hits = __reduce_add_sync(0xffffffffu, hits);
                 if (lane == 0 && hits) atomicAdd(&cnt[i], hits);
@@ -511,8 +580,8 @@ __device__ void process_vw(const PeelParams& P, uint32_t v, uint32_t w, unsigned
         } else {
             if (lane == 0)
                 for (uint32_t i = 0; i < nc; i++)
-                    bytes += 16 + 4ull * (P.wend[C[i]] - P.wnb[C[i]]);
-            warp_build_rows32(C, nc, P.wend, P.wadj, P.wnb, rows);
+                    bytes += 16 + 4ull * (R.ne[C[i]] - R.nb[C[i]]);
+            warp_build_rows32(C, nc, R.ne, R.adj, R.nb, rows);
             tot = warp_dfs32(rows, nc, r, cnt);
         }
         __syncwarp();
@@ -520,21 +589,77 @@ __device__ void process_vw(const PeelParams& P, uint32_t v, uint32_t w, unsigned
             for (uint32_t i = lane; i < nc; i += 32) {
                 uint32_t x = C[i];
                 if (cnt[i]) {
+                    bool dec;
+                    const uint32_t wx = P.sl[x];
                     bytes += 4;
-                    if (st_of(P.sl[x]) == kAlive) {
-                        dec_and_queue(P, x, (unsigned long long)cnt[i], k, next, next_cnt);
+                    (void)cand_ok(wx, x, kv, v, dec);
+                    if (dec) {
+                        lower(P, x, st_of(wx), (unsigned long long)cnt[i], k, next, next_cnt);
                         bytes += 16;
                     }
                 }
             }
         __syncwarp();
     }
-    if (tot && lane == 0) {
-        if (sw == kAlive) {
-            dec_and_queue(P, w, tot, k, next, next_cnt);
-            bytes += 16;
+    if (tot && lane == 0 && dec_w) {
+        lower(P, w, st_of(ww), tot, k, next, next_cnt);
+        bytes += 16;
+    }
+}
+
+// h = 3, phase 2: one pair (v, u) of a frontier vertex v and a counting
+// neighbour u of the same band (state word wu): u loses the triangles {v, u,
+// x} with x in the current set.  Rows hold no member of an earlier band, so
+// the members of a later band are never enumerated on their own account:
+// only pairs inside a band cost anything.  One warp; the shorter of the two
+// rows is read and searched for in the longer.
+__device__ __forceinline__ void process_pair(const PeelParams& P, uint32_t v, uint32_t kv,
+                                             uint32_t u, unsigned long long& bytes) {
+    const unsigned lane = lane_id();
+    const uint32_t* A = P.wadj + P.off[v];
+    uint64_t da = P.wend[v] - P.off[v];
+    const uint32_t* B = P.wadj + P.off[u];
+    uint64_t db = P.wend[u] - P.off[u];
+    if (db < da) {
+        const uint32_t* t = A;
+        A = B;
+        B = t;
+        const uint64_t td = da;
+        da = db;
+        db = td;
+    }
+    const unsigned pr = probes(db);
+    unsigned hits = 0;
+    for (uint64_t p0 = 0; p0 < da; p0 += 32 * kChunks) {
+        uint32_t xs[kChunks], ws[kChunks];
+#pragma unroll
+        for (int q = 0; q < kChunks; q++) {
+            uint64_t p = p0 + q * 32 + lane;
+            xs[q] = p < da ? A[p] : 0u;
         }
-        destroyed += tot;
+#pragma unroll
+        for (int q = 0; q < kChunks; q++) {
+            uint64_t p = p0 + q * 32 + lane;
+            ws[q] = p < da ? P.sl[xs[q]] : (uint32_t)kGone;
+        }
+#pragma unroll
+        for (int q = 0; q < kChunks; q++) {
+            uint64_t p = p0 + q * 32 + lane;
+            bool dec;
+            if (p < da) {
+                bytes += 8;
+                if (cand_ok(ws[q], xs[q], kv, v, dec)) {
+                    uint64_t pos = lower_bound_u32(B, db, xs[q]);
+                    hits += pos < db && B[pos] == xs[q];
+                    bytes += 4ull * pr;
+                }
+            }
+        }
+    }
+    hits = __reduce_add_sync(0xffffffffu, hits);
+    if (lane == 0 && hits) {
+        atomic_sub_u64(&P.deg[u], (unsigned long long)hits);
+        bytes += 16 + 16;
     }
 }
 
@@ -543,10 +668,9 @@ __device__ void process_vw(const PeelParams& P, uint32_t v, uint32_t w, unsigned
 // N+(w) holds more than kBitmapMax entries (degeneracy above 1024) the
 // candidates are gathered into the block's global scratch; a set that still
 // exceeds kBitmapMax is split by its next member (xl.cuh).
-__device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigned long long k,
-                            uint32_t* next, uint32_t* next_cnt, uint32_t* smem,
-                            const uint32_t* gbm, unsigned long long& destroyed,
-                            unsigned long long& bytes) {
+__device__ void process_big(const PeelParams& P, const NPlus& R, uint32_t v, uint32_t w,
+                            unsigned long long k, uint32_t* next, uint32_t* next_cnt,
+                            uint32_t* smem, const uint32_t* gbm, unsigned long long& bytes) {
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // bcap
     uint32_t* C = smem + 2 * P.bcap;                                          // bcap
     uint32_t* rows = C + P.bcap;                                              // bcap * W
@@ -556,8 +680,10 @@ __device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigne
     __shared__ uint32_t s_flag[kBitmapMax / 32], s_at[kBitmapMax / 32];
     __shared__ uint32_t s_w[32], s_t2;
     const unsigned lane = lane_id(), nw = blockDim.x >> 5;
-    uint32_t sw = st_of(P.sl[w]);
-    const uint64_t b = P.wnb[w], e = P.wend[w];
+    const uint32_t kv = P.sl[v] >> kKeyShift, ww = P.sl[w];
+    bool dec_w;
+    (void)cand_ok(ww, w, kv, v, dec_w);
+    const uint64_t b = R.nb[w], e = R.ne[w];
     const uint32_t* Nv = P.wadj + P.off[v];
     const uint64_t dv = P.wend[v] - P.off[v];
     const unsigned pr = probes(dv);
@@ -565,10 +691,10 @@ __device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigne
         // oversized N+(w): gather in order into the block's global scratch
         uint32_t* G0 = P.xl + (size_t)blockIdx.x * (kMaxDepth + 1) * P.cap;
         const uint32_t nc = block_filter(
-            P.wadj + b, e - b, G0,
+            R.adj + b, e - b, G0,
             [&](uint32_t x) {
-                const uint32_t st = st_of(P.sl[x]);
-                if (!(st == kAlive || (st == kFront && x > v))) return false;
+                bool dec;
+                if (!cand_ok(P.sl[x], x, kv, v, dec)) return false;
                 if (gbm) return ((gbm[x >> 5] >> (x & 31)) & 1u) != 0u;
                 uint64_t pos = lower_bound_u32(Nv, dv, x);
                 return pos < dv && Nv[pos] == x;
@@ -579,16 +705,17 @@ __device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigne
             if (threadIdx.x == 0) s_tot = 0;
             __syncthreads();
             xl_cliques(
-                G0, nc, P.h - 2, P.wnb, P.wend, P.wadj, G0 + P.cap, P.cap, smem,
+                G0, nc, P.h - 2, R.nb, R.ne, R.adj, G0 + P.cap, P.cap, smem,
                 [&](uint32_t x, unsigned long long c) {
-                    if (st_of(P.sl[x]) == kAlive) dec_and_queue(P, x, c, k, next, next_cnt);
+                    bool dec;
+                    const uint32_t wx = P.sl[x];
+                    (void)cand_ok(wx, x, kv, v, dec);
+                    if (dec) lower(P, x, st_of(wx), c, k, next, next_cnt);
                 },
                 [&](unsigned long long c) { s_tot += c; });
             __syncthreads();
-            if (threadIdx.x == 0 && s_tot) {
-                if (sw == kAlive) dec_and_queue(P, w, s_tot, k, next, next_cnt);
-                destroyed += s_tot;
-            }
+            if (threadIdx.x == 0 && s_tot && dec_w)
+                lower(P, w, st_of(ww), s_tot, k, next, next_cnt);
             __syncthreads();
             return;
         }
@@ -610,10 +737,10 @@ __device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigne
         const uint64_t p = b + (uint64_t)c * 32 + lane;
         bool ok = false;
         if (p < e) {
-            const uint32_t x = P.wadj[p];
-            const uint32_t st = st_of(P.sl[x]);
+            const uint32_t x = R.adj[p];
+            bool dec;
             bytes += 8;
-            if (st == kAlive || (st == kFront && x > v)) {
+            if (cand_ok(P.sl[x], x, kv, v, dec)) {
                 if (gbm) {
                     ok = (gbm[x >> 5] >> (x & 31)) & 1u;
                     bytes += 4;
@@ -652,20 +779,27 @@ __device__ void process_big(const PeelParams& P, uint32_t v, uint32_t w, unsigne
     for (uint32_t c = warp_id(); c < runs; c += nw) {
         const unsigned bal = s_flag[c];
         if ((bal >> lane) & 1u)
-            C[s_at[c] + __popc(bal & ((1u << lane) - 1u))] = P.wadj[b + (uint64_t)c * 32 + lane];
+            C[s_at[c] + __popc(bal & ((1u << lane) - 1u))] = R.adj[b + (uint64_t)c * 32 + lane];
     }
     __syncthreads();
     }
 bitmap:
     uint32_t nc = s_nc;
     uint32_t W = (nc + 31) >> 5;
+    {
+        // nothing to do unless w or some candidate counts these cliques
+        bool any = dec_w;
+        for (uint32_t i = threadIdx.x; i < nc && !any; i += blockDim.x)
+            (void)cand_ok(P.sl[C[i]], C[i], kv, v, any);
+        if (!__syncthreads_or(any)) return;
+    }
     for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) {
         cnt[i] = 0;
-        bytes += 16 + 4ull * (P.wend[C[i]] - P.wnb[C[i]]);
+        bytes += 16 + 4ull * (R.ne[C[i]] - R.nb[C[i]]);
     }
     for (uint32_t i = threadIdx.x; i < nc * W; i += blockDim.x) rows[i] = 0;
     __syncthreads();
-    block_build_rows(C, nc, W, P.wend, P.wadj, P.wnb, rows);
+    block_build_rows(C, nc, W, R.ne, R.adj, R.nb, rows);
     __syncthreads();
     unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next);
     if (mine) atomicAdd(&s_tot, mine);
@@ -674,15 +808,16 @@ bitmap:
     if (tot) {
         for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) {
             uint32_t x = C[i];
-            if (cnt[i] && st_of(P.sl[x]) == kAlive) {
-                dec_and_queue(P, x, cnt[i], k, next, next_cnt);
+            if (!cnt[i]) continue;
+            bool dec;
+            const uint32_t wx = P.sl[x];
+            (void)cand_ok(wx, x, kv, v, dec);
+            if (dec) {
+                lower(P, x, st_of(wx), cnt[i], k, next, next_cnt);
                 bytes += 20;
             }
         }
-        if (threadIdx.x == 0) {
-            if (sw == kAlive) dec_and_queue(P, w, tot, k, next, next_cnt);
-            destroyed += tot;
-        }
+        if (threadIdx.x == 0 && dec_w) lower(P, w, st_of(ww), tot, k, next, next_cnt);
     }
     __syncthreads();
 }
@@ -696,10 +831,10 @@ __device__ __forceinline__ void group_bar(uint32_t id, uint32_t threads) {
 // *grab, several per block at once.  The group's warps build the one-word
 // rows of G[C] side by side (one candidate's list each), its first warp
 // lists the cliques of G[C] (warp_dfs32), and the alive members are lowered.
-// Group g synchronises on named barrier 1 + g.  destroyed: the round's sum.
+// Group g synchronises on named barrier 1 + g.
 template <int NT>
-__device__ void drain_mid(const PeelParams& P, uint32_t nm, uint32_t* grab, unsigned long long k,
-                          uint32_t* next, uint32_t* next_cnt, unsigned long long* destroyed,
+__device__ void drain_mid(const PeelParams& P, const NPlus& R, uint32_t nm, uint32_t* grab,
+                          unsigned long long k, uint32_t* next, uint32_t* next_cnt,
                           unsigned long long& bytes) {
     constexpr int NG = NT / 32 / kGroupWarps;
     struct MidBuf {
@@ -715,7 +850,6 @@ __device__ void drain_mid(const PeelParams& P, uint32_t nm, uint32_t* grab, unsi
     const uint32_t bar = 1u + grp, nth = kGroupWarps * 32u;
     MidBuf& B = s_mb[grp];
     const int r = P.h - 2;
-    unsigned long long dsum = 0;
     for (;;) {
         if (gw == 0 && lane == 0) B.i = atomicAdd(grab, 1u);
         group_bar(bar, nth);
@@ -723,7 +857,7 @@ __device__ void drain_mid(const PeelParams& P, uint32_t nm, uint32_t* grab, unsi
         if (i >= nm) break;
         const uint32_t* rec = P.mid + (size_t)i * kMidWords;
         const uint32_t v = rec[0], w = rec[1], nc = rec[2];
-        (void)v;
+        const uint32_t kv = P.sl[v] >> kKeyShift;
         if (gw == 0) {
             B.C[lane] = lane < nc ? rec[3 + lane] : 0u;
             B.cnt[lane] = 0;
@@ -733,10 +867,10 @@ __device__ void drain_mid(const PeelParams& P, uint32_t nm, uint32_t* grab, unsi
         const uint32_t cmax = B.C[nc - 1];
         for (uint32_t x = gw; x + 1 < nc; x += kGroupWarps) {
             const uint32_t y = B.C[x];
-            const uint32_t bits = warp_row32(B.C, nc, cmax, y, P.wadj, P.wnb[y], P.wend[y]);
+            const uint32_t bits = warp_row32(B.C, nc, cmax, y, R.adj, R.nb[y], R.ne[y]);
             if (lane == 0) {
                 B.rows[x] = bits;
-                bytes += 16 + 4ull * (P.wend[y] - P.wnb[y]);
+                bytes += 16 + 4ull * (R.ne[y] - R.nb[y]);
             }
         }
         group_bar(bar, nth);
@@ -750,23 +884,28 @@ __device__ void drain_mid(const PeelParams& P, uint32_t nm, uint32_t* grab, unsi
             const uint32_t t = gw * 32 + lane;
             if (t < nc && B.cnt[t]) {
                 const uint32_t x = B.C[t];
-                if (st_of(P.sl[x]) == kAlive) {
-                    dec_and_queue(P, x, (unsigned long long)B.cnt[t], k, next, next_cnt);
+                const uint32_t wx = P.sl[x];
+                bool dec;
+                (void)cand_ok(wx, x, kv, v, dec);
+                if (dec) {
+                    lower(P, x, st_of(wx), (unsigned long long)B.cnt[t], k, next, next_cnt);
                     bytes += 20;
                 }
             }
             if (gw == 0 && lane == 0) {
-                if (st_of(P.sl[w]) == kAlive) dec_and_queue(P, w, tot, k, next, next_cnt);
-                dsum += tot;
+                const uint32_t ww = P.sl[w];
+                bool dec;
+                (void)cand_ok(ww, w, kv, v, dec);
+                if (dec) lower(P, w, st_of(ww), tot, k, next, next_cnt);
             }
         }
         group_bar(bar, nth);   // B is rewritten by the next item
     }
-    if (gw == 0 && lane == 0 && dsum) atomicAdd(destroyed, dsum);
 }
 
-// Drop removed vertices from row v in place (one warp); rows stay sorted.
-__device__ __forceinline__ void compact_row(const PeelParams& P, uint32_t v,
+// Drop removed vertices (phase 2, where every key is set: members of earlier
+// bands) from row v in place (one warp); rows stay sorted.
+__device__ __forceinline__ void compact_row(const PeelParams& P, uint32_t v, uint32_t kv,
                                             unsigned long long& bytes) {
     unsigned lane = lane_id();
     uint64_t b = P.off[v], e = P.wend[v];
@@ -778,7 +917,8 @@ __device__ __forceinline__ void compact_row(const PeelParams& P, uint32_t v,
         bool keep = false;
         if (p < e) {
             x = P.wadj[p];
-            keep = st_of(P.sl[x]) != kGone;
+            const uint32_t wx = P.sl[x], kx = wx >> kKeyShift;
+            keep = kx > kv || (kx == kv && st_of(wx) != kGone);
         }
         unsigned bal = __ballot_sync(0xffffffffu, keep);
         unsigned lt = __ballot_sync(0xffffffffu, keep && x < v);
@@ -796,7 +936,7 @@ __device__ __forceinline__ void compact_row(const PeelParams& P, uint32_t v,
     }
 }
 
-// Large regime: the neighbourhood bitmap of frontier vertex v for rounds of
+// Phase 1: the neighbourhood bitmap of frontier vertex v for rounds of
 // parity par, or null if v has none.
 __device__ __forceinline__ const uint32_t* hub_bm_of(const PeelParams& P, uint32_t v,
                                                     uint32_t par) {
@@ -805,12 +945,15 @@ __device__ __forceinline__ const uint32_t* hub_bm_of(const PeelParams& P, uint32
     return slot ? P.hub_bm + ((size_t)par * P.hub_slots + (slot - 1)) * P.hub_words : nullptr;
 }
 
-// Large regime, marking v as a member of frontier F_r: its state word, with
-// kHeavyBit for rows longer than heavy_min and, for rows longer than hub_min
+// Phase 1, marking v as a member of frontier F_r: its state word (gone at
+// once if it lies in no clique of the current set: nothing is enumerated
+// from it), with kHeavyBit for rows longer than heavy_min and, for rows longer than hub_min
 // while slots of this parity last, 1 + its bitmap slot (the owner goes to
 // the parity's hub list).
 __device__ __forceinline__ uint32_t front_word(const PeelParams& P, PeelCtrl* c, uint32_t v,
                                                uint32_t par, bool& hv) {
+    hv = false;
+    if (P.deg[v] == 0) return kGone;
     uint64_t d = P.wend[v] - P.off[v];
     hv = P.heavy_min && d > P.heavy_min;
     uint32_t w = kFront | (hv ? kHeavyBit : 0u);
@@ -833,7 +976,7 @@ __device__ __forceinline__ void hub_bitmaps(const PeelParams& P, uint32_t nhub, 
                                             unsigned long long* s_red,
                                             unsigned long long& bytes) {
     const uint32_t* H = P.hubs + (size_t)par * P.hub_slots;
-    block_prefix_degrees<NT>(P, H, nhub, s_pre, s_red);
+    block_prefix_degrees<NT, true>(P, H, nhub, s_pre, s_red);
     const unsigned long long T = s_pre[nhub];
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t gthreads = (uint64_t)gridDim.x * blockDim.x;
@@ -853,18 +996,15 @@ __device__ __forceinline__ void hub_bitmaps(const PeelParams& P, uint32_t nhub, 
     __syncthreads();   // s_pre is reused afterwards
 }
 
-// P2: the cliques destroyed by frontier F (nf vertices; F in global or
-// shared memory, identical for every block).  Frontier counts do not change
-// during P2 (only alive vertices are lowered), so a frontier vertex of count
-// 0, which lies in no clique of the current set, is skipped.  bm: shared bitmaps of the
-// neighbourhoods of F[0 .. min(nf, kBitmapSlots)) (small regime), or null.
+// P2, phase 1: the cliques destroyed by frontier F (nf vertices, identical
+// for every block).  Frontier vertices marked gone (count 0) have no items.
 template <int NT>
 __device__ __forceinline__ void process_frontier(
-    const PeelParams& P, const uint32_t* F, uint32_t nf, unsigned long long k, uint32_t* Fnext,
-    uint32_t* next_cnt, uint32_t* big_cnt, uint32_t* wC, unsigned* wCnt, uint32_t* wRows,
-    const uint32_t* bm, uint32_t bm_words, unsigned long long* s_pre, unsigned long long* s_red,
-    const uint32_t* hl, uint32_t nh, uint32_t* grab, uint32_t* s_grab, uint32_t par,
-    unsigned long long& destroyed, unsigned long long& items, unsigned long long& bytes) {
+    const PeelParams& P, const NPlus& R, const uint32_t* F, uint32_t nf, unsigned long long k,
+    uint32_t* Fnext, uint32_t* next_cnt, uint32_t* big_cnt, uint32_t* wC, unsigned* wCnt,
+    uint32_t* wRows, unsigned long long* s_pre, unsigned long long* s_red, uint32_t nh,
+    uint32_t* grab, uint32_t* s_grab, uint32_t par, unsigned long long& items,
+    unsigned long long& bytes) {
     constexpr int NW = NT / 32;
     const unsigned lane = lane_id(), wid = warp_id();
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -874,7 +1014,7 @@ __device__ __forceinline__ void process_frontier(
     if (k == 0) return;   // every frontier vertex has count 0
     if (nf <= kSmallFront) {
         // flatten (v, neighbour index) items over the whole grid
-        block_prefix_degrees<NT>(P, F, nf, s_pre, s_red, true);
+        block_prefix_degrees<NT>(P, F, nf, s_pre, s_red);
         unsigned long long T = s_pre[nf];
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             items += T;
@@ -889,14 +1029,13 @@ __device__ __forceinline__ void process_frontier(
                 }
                 uint32_t v = F[lo];
                 uint32_t u = P.wadj[P.off[v] + (t - s_pre[lo])];
-                uint32_t su = st_of(P.sl[u]);
+                const uint32_t wu = P.sl[u];
+                bool dec;
+                (void)cand_ok(wu, u, 0u, v, dec);
                 bytes += 4 + 4;
-                if (su == kAlive) {
-                    dec_and_queue(P, u, 1ull, k, Fnext, next_cnt);
-                    destroyed++;
+                if (dec) {
+                    lower(P, u, st_of(wu), 1ull, k, Fnext, next_cnt);
                     bytes += 16;
-                } else if (su == kFront && u > v) {
-                    destroyed++;
                 }
             }
         } else {
@@ -908,27 +1047,24 @@ __device__ __forceinline__ void process_frontier(
                 }
                 uint32_t v = F[lo];
                 uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
-                const uint32_t* vbm = (bm && lo < kBitmapSlots) ? bm + (size_t)lo * bm_words : nullptr;
-                const uint32_t* gbm = hl ? hub_bm_of(P, v, par) : nullptr;
-                process_vw(P, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt, vbm, gbm,
-                           destroyed, bytes);
+                process_vw(P, R, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
+                           hub_bm_of(P, v, par), bytes);
             }
         }
     } else if (P.h == 2) {
         for (uint64_t i = gwarp; i < nf; i += gwarps) {
             uint32_t v = F[i];
-            if (P.deg[v] == 0) continue;
+            if (st_of(P.sl[v]) != kFront) continue;
             uint64_t b = P.off[v], e = P.wend[v];
             for (uint64_t p = b + lane; p < e; p += 32) {
                 uint32_t u = P.wadj[p];
-                uint32_t su = st_of(P.sl[u]);
+                const uint32_t wu = P.sl[u];
+                bool dec;
+                (void)cand_ok(wu, u, 0u, v, dec);
                 bytes += 4 + 4;
-                if (su == kAlive) {
-                    dec_and_queue(P, u, 1ull, k, Fnext, next_cnt);
-                    destroyed++;
+                if (dec) {
+                    lower(P, u, st_of(wu), 1ull, k, Fnext, next_cnt);
                     bytes += 16;
-                } else if (su == kFront && u > v) {
-                    destroyed++;
                 }
             }
             if (lane == 0) {
@@ -937,98 +1073,200 @@ __device__ __forceinline__ void process_frontier(
             }
         }
     } else {
-        // Large regime: the items of heavy vertices (hl, nh: rows longer than
+        // The items of heavy vertices (P.heavy, nh: rows longer than
         // heavy_min, flagged kHeavyBit) are flattened over every warp of the
         // grid in batches of kSmallFront vertices; every other vertex goes to
-        // one block, blocks taking chunks of the frontier from *grab.  In the
-        // small regime (hl null) blocks take the vertices in a fixed order.
-        if (hl) {
-            for (uint32_t b0 = 0; b0 < nh; b0 += kSmallFront) {
-                const uint32_t nb = nh - b0 < kSmallFront ? nh - b0 : kSmallFront;
-                const uint32_t* H = hl + b0;
-                block_prefix_degrees<NT>(P, H, nb, s_pre, s_red, true);
-                unsigned long long T = s_pre[nb];
-                if (blockIdx.x == 0 && threadIdx.x == 0) {
-                    items += T;
-                    bytes += 20ull * nb;
-                }
-                for (uint64_t t = gwarp; t < T; t += gwarps) {
-                    uint32_t lo = 0, hi = nb;
-                    while (hi - lo > 1) {
-                        uint32_t mid = (lo + hi) >> 1;
-                        if (s_pre[mid] <= t) lo = mid; else hi = mid;
-                    }
-                    uint32_t v = H[lo];
-                    uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
-                    process_vw(P, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt, nullptr,
-                               hub_bm_of(P, v, par), destroyed, bytes);
-                }
-                __syncthreads();   // s_pre is rewritten by the next batch
+        // one block, blocks taking chunks of the frontier from *grab.
+        for (uint32_t b0 = 0; b0 < nh; b0 += kSmallFront) {
+            const uint32_t nb = nh - b0 < kSmallFront ? nh - b0 : kSmallFront;
+            const uint32_t* H = P.heavy + b0;
+            block_prefix_degrees<NT>(P, H, nb, s_pre, s_red);
+            unsigned long long T = s_pre[nb];
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                items += T;
+                bytes += 20ull * nb;
             }
-            const uint32_t ch0 = nf / (4u * gridDim.x);
-            const uint32_t ch = ch0 < 1u ? 1u : (ch0 > 32u ? 32u : ch0);
-            for (;;) {
-                if (threadIdx.x == 0) *s_grab = atomicAdd(grab, ch);
-                __syncthreads();
-                const uint32_t i0 = *s_grab;
-                __syncthreads();
-                if (i0 >= nf) break;
-                const uint32_t i1 = i0 + ch < nf ? i0 + ch : nf;
-                for (uint32_t i = i0; i < i1; i++) {
-                    uint32_t v = F[i];
-                    if ((P.sl[v] & kHeavyBit) || P.deg[v] == 0) continue;   // taken above, or none
-                    uint64_t b = P.off[v], e = P.wend[v];
-                    for (uint64_t p = b + wid; p < e; p += NW)
-                        process_vw(P, v, P.wadj[p], k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
-                                   nullptr, nullptr, destroyed, bytes);
-                    if (threadIdx.x == 0) {
-                        items += e - b;
-                        bytes += 24;
-                    }
+            for (uint64_t t = gwarp; t < T; t += gwarps) {
+                uint32_t lo = 0, hi = nb;
+                while (hi - lo > 1) {
+                    uint32_t mid = (lo + hi) >> 1;
+                    if (s_pre[mid] <= t) lo = mid; else hi = mid;
                 }
+                uint32_t v = H[lo];
+                uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
+                process_vw(P, R, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
+                           hub_bm_of(P, v, par), bytes);
             }
-            return;
+            __syncthreads();   // s_pre is rewritten by the next batch
         }
-        for (uint64_t i = blockIdx.x; i < nf; i += gridDim.x) {
-            uint32_t v = F[i];
-            if (P.deg[v] == 0) continue;
-            uint64_t b = P.off[v], e = P.wend[v];
-            const uint32_t* vbm = (bm && i < kBitmapSlots) ? bm + (size_t)i * bm_words : nullptr;
-            for (uint64_t p = b + wid; p < e; p += NW)
-                process_vw(P, v, P.wadj[p], k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt, vbm,
-                           nullptr, destroyed, bytes);
-            if (threadIdx.x == 0) {
-                items += e - b;
-                bytes += 20;
+        const uint32_t ch0 = nf / (4u * gridDim.x);
+        const uint32_t ch = ch0 < 1u ? 1u : (ch0 > 32u ? 32u : ch0);
+        for (;;) {
+            if (threadIdx.x == 0) *s_grab = atomicAdd(grab, ch);
+            __syncthreads();
+            const uint32_t i0 = *s_grab;
+            __syncthreads();
+            if (i0 >= nf) break;
+            const uint32_t i1 = i0 + ch < nf ? i0 + ch : nf;
+            for (uint32_t i = i0; i < i1; i++) {
+                uint32_t v = F[i];
+                const uint32_t wv = P.sl[v];
+                if ((wv & kHeavyBit) || st_of(wv) != kFront) continue;   // taken above, or none
+                uint64_t b = P.off[v], e = P.wend[v];
+                for (uint64_t p = b + wid; p < e; p += NW)
+                    process_vw(P, R, v, P.wadj[p], k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
+                               nullptr, bytes);
+                if (threadIdx.x == 0) {
+                    items += e - b;
+                    bytes += 24;
+                }
             }
         }
     }
 }
 
-// Shared bitmaps over local ids of the neighbourhoods of F[0..min(nf,
-// kBitmapSlots)), built by every block (small regime).
+// P2, phase 2: the frontiers of all bands together (nf vertices), in batches
+// whose items are flattened over the grid.
 template <int NT>
-__device__ __forceinline__ void build_bitmaps(const PeelParams& P, const uint32_t* F, uint32_t nf,
-                                              uint32_t* bm, uint32_t bm_words) {
-    uint32_t slots = nf < kBitmapSlots ? nf : kBitmapSlots;
-    for (uint32_t i = threadIdx.x; i < slots * bm_words; i += NT) bm[i] = 0;
-    __syncthreads();
-    const unsigned nw = NT / 32;
-    for (uint32_t s = warp_id(); s < slots; s += nw) {
-        uint32_t v = F[s];
-        uint64_t b = P.off[v], e = P.wend[v];
-        uint32_t* row = bm + (size_t)s * bm_words;
-        for (uint64_t p = b + lane_id(); p < e; p += 32) {
-            uint32_t x = P.wadj[p];
-            uint32_t w = P.sl[x];
-            // removed vertices may lack a local id; they are never candidates
-            if (st_of(w) != kGone) {
-                uint32_t l = w >> 2;
-                atomicOr(&row[l >> 5], 1u << (l & 31));
+__device__ __forceinline__ void process_bands(
+    const PeelParams& P, const NPlus& R, const uint32_t* F, uint32_t nf, uint32_t* big_cnt,
+    uint32_t* wC, unsigned* wCnt, uint32_t* wRows, unsigned long long* s_pre,
+    unsigned long long* s_red, unsigned long long& items, unsigned long long& bytes) {
+    const unsigned lane = lane_id();
+    const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t gthreads = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t gwarp = gtid >> 5;
+    const uint64_t gwarps = gthreads >> 5;
+    for (uint32_t b0 = 0; b0 < nf; b0 += kSmallFront) {
+        const uint32_t nb = nf - b0 < kSmallFront ? nf - b0 : kSmallFront;
+        const uint32_t* H = F + b0;
+        block_prefix_degrees<NT>(P, H, nb, s_pre, s_red);
+        const unsigned long long T = s_pre[nb];
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            items += T;
+            bytes += 20ull * nb;
+        }
+        // the frontier vertex of item t: last i with s_pre[i] <= t
+        auto at = [&](uint64_t t) -> uint32_t {
+            uint32_t lo = 0, hi = nb;
+            while (hi - lo > 1) {
+                uint32_t mid = (lo + hi) >> 1;
+                if (s_pre[mid] <= t) lo = mid; else hi = mid;
+            }
+            return lo;
+        };
+        if (P.h == 2) {
+            for (uint64_t t = gtid; t < T; t += gthreads) {
+                const uint32_t i = at(t), v = H[i];
+                const uint32_t u = P.wadj[P.off[v] + (t - s_pre[i])];
+                bool dec;
+                (void)cand_ok(P.sl[u], u, P.sl[v] >> kKeyShift, v, dec);
+                bytes += 4 + 4;
+                if (dec) {
+                    atomic_sub_u64(&P.deg[u], 1ull);
+                    bytes += 16;
+                }
+            }
+        } else if (P.h == 3) {
+            // a warp looks at `cs` consecutive items at once, one a lane, and
+            // takes the pairs among them one by one: most items name a
+            // vertex of a later band and need nothing more
+            uint32_t cs = 1;
+            while (cs < 32 && (uint64_t)cs * gwarps < T) cs <<= 1;
+            for (uint64_t t0 = gwarp * cs; t0 < T; t0 += gwarps * cs) {
+                const uint64_t t = t0 + lane;
+                uint32_t v = 0, u = 0, kv = 0;
+                bool dec = false;
+                if (lane < cs && t < T) {
+                    const uint32_t i = at(t);
+                    v = H[i];
+                    u = P.wadj[P.off[v] + (t - s_pre[i])];
+                    kv = P.sl[v] >> kKeyShift;
+                    (void)cand_ok(P.sl[u], u, kv, v, dec);
+                    bytes += 4 + 4;
+                }
+                unsigned todo = __ballot_sync(0xffffffffu, dec);
+                while (todo) {
+                    const int l = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    process_pair(P, __shfl_sync(0xffffffffu, v, l),
+                                 __shfl_sync(0xffffffffu, kv, l),
+                                 __shfl_sync(0xffffffffu, u, l), bytes);
+                }
+            }
+        } else {
+            for (uint64_t t = gwarp; t < T; t += gwarps) {
+                const uint32_t i = at(t), v = H[i];
+                const uint32_t w = P.wadj[P.off[v] + (t - s_pre[i])];
+                process_vw(P, R, v, w, 0ull, nullptr, nullptr, wC, wCnt, wRows, big_cnt, nullptr,
+                           bytes);
             }
         }
+        __syncthreads();   // s_pre is rewritten by the next batch
+    }
+}
+
+// P2b: the round's mid items (warp groups) and big items (blocks).
+template <int NT>
+__device__ __forceinline__ void process_queued(const PeelParams& P, const NPlus& R, uint32_t slot,
+                                               uint32_t nb, uint32_t nm, unsigned long long k,
+                                               uint32_t* next, uint32_t* next_cnt, uint32_t* smem,
+                                               bool hubs, uint32_t par, uint32_t* s_grab,
+                                               unsigned long long& bytes) {
+    PeelCtrl* c = P.ctrl;
+    if (nb > P.big_cap) nb = (uint32_t)P.big_cap;
+    if (nm > P.mid_cap) nm = P.mid_cap;
+    if (nm) {
+        drain_mid<NT>(P, R, nm, &c->bgrab[3 + slot], k, next, next_cnt, bytes);
+        __syncthreads();
+    }
+    for (;;) {
+        if (threadIdx.x == 0) *s_grab = atomicAdd(&c->bgrab[slot], 1u);
+        __syncthreads();
+        const uint32_t i = *s_grab;
+        __syncthreads();
+        if (i >= nb) break;
+        const uint2 it = P.big[i];
+        process_big(P, R, it.x, it.y, k, next, next_cnt, smem,
+                    hubs ? hub_bm_of(P, it.x, par) : nullptr, bytes);
+    }
+}
+
+// The threshold of a jump (every block alike): the largest count k + 1 + hi
+// such that the alive vertices at or below it number at most `tmax`, or at
+// most kBandAim and span at most `lmax` values.  hist: the alive vertices by bin_of(count - k - 1).
+// Returns k + 1 + hi, or 0 when even the first occupied bin is larger.
+template <int NT>
+__device__ __forceinline__ unsigned long long pick_threshold(const uint32_t* hist,
+                                                             unsigned long long k, uint32_t tmax,
+                                                             uint32_t lmax, uint32_t* s_wtot,
+                                                             uint32_t* s_best) {
+    constexpr uint32_t E = kBins / NT > 0 ? kBins / NT : 1;
+    static_assert(kBins % NT == 0, "a whole number of bins per thread");
+    uint32_t c[E], sum = 0;
+#pragma unroll
+    for (uint32_t q = 0; q < E; q++) {
+        c[q] = hist[threadIdx.x * E + q];
+        sum += c[q];
+    }
+    if (threadIdx.x == 0) *s_best = 0;
+    uint32_t tot;
+    uint32_t run = block_scan_count<NT>(sum, s_wtot, &tot);
+#pragma unroll
+    for (uint32_t q = 0; q < E; q++) {
+        const uint32_t b = threadIdx.x * E + q;
+        run += c[q];
+        // at least one vertex up to here, and few enough of them or of levels
+        if (run && c[q] && (run <= tmax ||
+                            (run <= kBandAim && bin_last(b < kLastBin ? b : kLastBin) < lmax)))
+            atomicMax(s_best, b + 1);
     }
     __syncthreads();
+    const uint32_t b = *s_best;
+    __syncthreads();
+    if (b == 0) return 0;
+    const unsigned long long last = bin_last(b - 1);
+    return last > ~0ull - k - 1 ? ~0ull : k + 1 + last;
 }
 
 // ---------------------------------------------------------------- kernel
@@ -1038,7 +1276,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
     extern __shared__ uint32_t smem[];
     __shared__ unsigned long long s_pre[kSmallFront + 1];
     __shared__ unsigned long long s_red[NW];
+    __shared__ uint32_t s_hist[kBins];
     __shared__ uint32_t s_wtot[NW];
+    __shared__ unsigned long long s_bmin[2][NW], s_bsum[2][NW];
+    __shared__ uint32_t s_bcnt[2][NW], s_bleft[2][NW];
     __shared__ uint32_t s_n;
     __shared__ uint32_t s_grab;
     PeelCtrl* c = P.ctrl;
@@ -1050,23 +1291,23 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
     uint32_t* wC = smem + (size_t)wid * kWarpWords;
     unsigned* wCnt = wC + kWarpCand;
     uint32_t* wRows = wC + 2 * kWarpCand;
-    uint32_t* sA = smem + P.work_words;   // small regime: alive list
-    uint32_t* sF = sA + P.asmall;         // small regime: frontier
-    uint32_t* sBM = sF + P.asmall;        // small regime: neighbourhood bitmaps
-    const uint32_t bm_words = (P.asmall + 31) / 32;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    const NPlus R1{P.wadj, P.wnb, P.wend};
+    const NPlus R2{P.nadj, P.nsplit, P.off + 1};
 
     unsigned long long k = P.k0;           // level floor (threshold pruning when > 0)
-    unsigned long long mu_alive = P.mu0;   // meaningful in block 0
-    uint32_t r = 0, jumps = 0, nlev = 0, nbar = 0, ncompact = 0;
+    unsigned long long klow = k;           // k before the last jump
+    uint32_t r = 0, jumps = 0, nbar = 0, ncompact = 0;
     int ap = 0;
-    uint32_t alive_cnt = P.n;
+    uint32_t alive_cnt = P.n;              // entries of the alive list
     uint32_t compacted_at = P.n;           // alive count at the last row compaction
-    bool small = false;
-    uint32_t na_s = 0, nf_s = 0;           // small regime: alive total, frontier size
-    uint32_t na_entry = 0;                 // alive vertices when the small regime began
-    uint32_t slice_lo = 0, na_loc = 0;     // this block's slice of the alive list
-    uint32_t cmp_loc = 0;                  // slice size at its last row compaction
+    uint32_t retired = 0;                  // vertices in mem
+    uint32_t nb = 0;                       // multi-level bands so far
+    bool multi = false;                    // the current band has several levels
+    uint32_t seg = 0;                      // where it starts in mem
+    uint32_t fails = 0, hold = 0;          // cascades undone in a row; jumps without bands
+    unsigned long long gone0 = 0;          // lead: cliques destroyed before the band
+    uint32_t rs = 0;                       // rounds of single-level bands so far
     unsigned long long items = 0, bytes = 0, waited = 0;
 
     // Block 0's time per phase (thread 0, %globaltimer); the time inside
@@ -1090,437 +1331,467 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
         if (lead) tlast = globaltimer_ns();                \
     } while (0)
 
+    // ============================================================ phase 1
     for (;;) {
-        bool s_jump = false;
-        if (!small) {
-            // ------------------------------------------------------ P1
-            {
-                uint32_t fprev = r ? c->fcnt[(r + 2) % 3] : 0u;
-                const uint32_t* Fprev = P.front[(r + 2) % 3];
-                for (uint64_t i = gtid; i < fprev; i += gthreads) {
-                    uint32_t v = Fprev[i];
-                    P.sl[v] = kGone;
+        // ---------------------------------------------------------- P1
+        const uint32_t fprev = r ? c->fcnt[(r + 2) % 3] : 0u;
+        if (fprev) {
+            const uint32_t* Fprev = P.front[(r + 2) % 3];
+            const uint32_t key = 2u * nb - (multi ? 1u : 0u);
+            unsigned long long gone = 0;
+            for (uint64_t i = gtid; i < fprev; i += gthreads) {
+                uint32_t v = Fprev[i];
+                gone += P.deg[v];
+                P.sl[v] = kGone;
+                P.band_of[v] = key;
+                P.mem[retired + i] = v;
+                if (!multi) {
                     P.core[v] = k;
-                    if (P.rnd) P.rnd[v] = r - 1;
-                    bytes += 4 + 4 + 8 + (P.rnd ? 4 : 0);
+                    if (P.rnd) P.rnd[v] = rs;
                 }
+                bytes += 4 + 4 + 8 + 8 + 4 + (P.rnd ? 4 : 0);
             }
-            uint32_t fcur = c->fcnt[r % 3];
-            uint32_t* Fcur = P.front[r % 3];
-            // the bitmaps of F_{r-1}'s hubs are zeroed for round r+1
-            if (r && P.hub_slots) {
-                uint32_t nhub = c->hubcnt[(r + 1) & 1];
-                if (nhub > P.hub_slots) nhub = P.hub_slots;
-                if (nhub) hub_bitmaps<NT>(P, nhub, (r + 1) & 1, true, s_pre, s_red, bytes);
-            }
-            // mark F_r; rows longer than heavy_min also go to the heavy list
-            for (uint64_t base = gwarp * 32; base < fcur; base += gwarps * 32) {
-                uint64_t i = base + lane;
-                bool hv = false;
-                uint32_t v = 0;
-                if (i < fcur) {
-                    v = Fcur[i];
-                    P.sl[v] = P.heavy_min ? front_word(P, c, v, r & 1, hv) : (uint32_t)kFront;
-                    bytes += 4 + 4 + (P.heavy_min ? 16 : 0);
-                }
-                if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
-            }
-            if (lead) {
-                if (r) {
-                    mu_alive -= c->destroyed[(r + 2) % 3];
-                    c->destroyed[(r + 2) % 3] = 0;
-                    c->big_cnt[(r + 2) % 3] = 0;
-                    c->bgrab[(r + 2) % 3] = 0;
-                    c->big_cnt[3 + (r + 2) % 3] = 0;
-                    c->bgrab[3 + (r + 2) % 3] = 0;
-                }
-                c->fcnt[(r + 1) % 3] = 0;
-                c->hcnt[(r + 1) % 3] = 0;
-                c->grab[(r + 1) % 3] = 0;
-            }
-            BARRIER(0);
-
-            // ------------------------------------------------- level jump
-            if (fcur == 0) {
-                const uint32_t* Ain = P.alive[ap];
-                uint32_t* Aout = P.alive[ap ^ 1];
-                unsigned long long mn = ~0ull;
-                for (uint64_t base = gwarp * 32; base < alive_cnt; base += gwarps * 32) {
-                    uint64_t i = base + lane;
-                    bool keep = false;
-                    uint32_t v = 0;
-                    if (i < alive_cnt) {
-                        v = Ain[i];
-                        bytes += 4 + 4;
-                        if (st_of(P.sl[v]) != kGone) {
-                            keep = true;
-                            unsigned long long d = P.deg[v];
-                            mn = d < mn ? d : mn;
-                            if (P.snap) P.snap[v] = d;
-                            bytes += 8 + 4;
-                        }
-                    }
-                    warp_append(keep, v, &c->new_alive[jumps & 1], Aout);
-                }
-                mn = warp_min_u64(mn);
-                if (lane == 0 && mn != ~0ull) atomicMin(&c->min_deg[jumps & 1], mn);
-                BARRIER(1);
-                uint32_t na = c->new_alive[jumps & 1];
-                if (na == 0) break;
-                ap ^= 1;
-                alive_cnt = na;
-                if (na <= P.asmall) {
-                    // enter the small regime: each block keeps its slice of
-                    // the alive list in shared memory and gives those vertices
-                    // their local id (the position in the list)
-                    na_entry = na;
-                    slice_lo = (uint32_t)((uint64_t)na * blockIdx.x / gridDim.x);
-                    na_loc = (uint32_t)((uint64_t)na * (blockIdx.x + 1) / gridDim.x) - slice_lo;
-                    cmp_loc = na_loc;
-                    for (uint32_t i = threadIdx.x; i < na_loc; i += NT) {
-                        uint32_t v = Aout[slice_lo + i];
-                        sA[i] = v;
-                        P.sl[v] = ((slice_lo + i) << 2) | kAlive;
-                    }
-                    if (lead) {
-                        c->small_round = r;
-                        bytes += 12ull * na;
-                    }
-                    small = true;
-                    na_s = na;
-                    nf_s = 0;
-                    s_jump = true;
-                    __syncthreads();
-                } else {
-                    unsigned long long m2 = c->min_deg[jumps & 1];
-                    k = m2 > k ? m2 : k;
-                    if (lead) {
-                        P.lvl_k[nlev] = k;
-                        P.lvl_size[nlev] = na;
-                        P.lvl_mu[nlev] = mu_alive;
-                        c->min_deg[(jumps + 1) & 1] = ~0ull;
-                        c->new_alive[(jumps + 1) & 1] = 0;
-                    }
-                    nlev++;
-                    jumps++;
-                    // Rows may be compacted in this same phase: compaction keeps
-                    // every vertex that is not removed, whether or not it is
-                    // being marked frontier concurrently.
-                    if (P.compact && 2ull * na <= compacted_at) {
-                        compacted_at = na;
-                        ncompact++;
-                        for (uint64_t i = gwarp; i < na; i += gwarps) compact_row(P, Aout[i], bytes);
-                    }
-                    for (uint64_t base = gwarp * 32; base < na; base += gwarps * 32) {
-                        uint64_t i = base + lane;
-                        bool in = false, hv = false;
-                        uint32_t v = 0;
-                        if (i < na) {
-                            v = Aout[i];
-                            bytes += 4 + 8;
-                            if (P.deg[v] <= k) {
-                                in = true;
-                                P.sl[v] = P.heavy_min ? front_word(P, c, v, r & 1, hv)
-                                                      : (uint32_t)kFront;
-                                bytes += 4 + 4 + (P.heavy_min ? 16 : 0);
-                            }
-                        }
-                        warp_append(in, v, &c->fcnt[r % 3], Fcur);
-                        if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
-                    }
-                    BARRIER(2);
-                    fcur = c->fcnt[r % 3];
-                }
-            }
-            if (!small) {
-                // -------------------------------------------------- P2
-                if (P.hub_slots) {
-                    uint32_t nhub = c->hubcnt[r & 1];
-                    if (nhub > P.hub_slots) nhub = P.hub_slots;
-                    if (lead) c->hubcnt[(r + 1) & 1] = 0;   // read last in this round's P1
-                    if (nhub) {
-                        hub_bitmaps<NT>(P, nhub, r & 1, false, s_pre, s_red, bytes);
-                        BARRIER(3);
-                    }
-                }
-                unsigned long long destroyed = 0;
-                process_frontier<NT>(P, Fcur, fcur, k, P.front[(r + 1) % 3],
-                                     &c->fcnt[(r + 1) % 3], &c->big_cnt[r % 3], wC, wCnt,
-                                     wRows, nullptr, 0, s_pre, s_red,
-                                     P.heavy_min ? P.heavy : nullptr, c->hcnt[r % 3],
-                                     &c->grab[r % 3], &s_grab, r & 1, destroyed, items, bytes);
-                unsigned long long bd = block_sum<NT>(destroyed, s_red);
-                if (threadIdx.x == 0 && bd) atomicAdd(&c->destroyed[r % 3], bd);
-                BARRIER(3);
-                // ------------------------------------------------- P2b
-                if (P.big_cap) {
-                    uint32_t nb = c->big_cnt[r % 3];
-                    uint32_t nm = c->big_cnt[3 + r % 3];
-                    if (nb || nm) {
-                        if (nb > P.big_cap) nb = (uint32_t)P.big_cap;
-                        if (nm > P.mid_cap) nm = P.mid_cap;
-                        if (nm) {
-                            drain_mid<NT>(P, nm, &c->bgrab[3 + r % 3], k, P.front[(r + 1) % 3],
-                                          &c->fcnt[(r + 1) % 3], &c->destroyed[r % 3], bytes);
-                            __syncthreads();
-                        }
-                        unsigned long long d2 = 0;
-                        for (;;) {
-                            if (threadIdx.x == 0) s_grab = atomicAdd(&c->bgrab[r % 3], 1u);
-                            __syncthreads();
-                            const uint32_t i = s_grab;
-                            __syncthreads();
-                            if (i >= nb) break;
-                            uint2 it = P.big[i];
-                            process_big(P, it.x, it.y, k, P.front[(r + 1) % 3],
-                                        &c->fcnt[(r + 1) % 3], smem, hub_bm_of(P, it.x, r & 1),
-                                        d2, bytes);
-                        }
-                        if (threadIdx.x == 0 && d2) atomicAdd(&c->destroyed[r % 3], d2);
-                        BARRIER(3);
-                    }
-                }
-                r++;
-                continue;
-            }
+            gone = warp_sum(gone);
+            if (lane == 0 && gone) atomicAdd(&c->destroyed, gone);
+            retired += fprev;
+            if (!multi) rs++;
         }
-
-        // ========================================================= small
-        if (!s_jump) {
-            // retire F_{r-1}: identical writes in every block
-            for (uint32_t i = threadIdx.x; i < nf_s; i += NT) {
-                uint32_t v = sF[i];
-                P.sl[v] = (P.sl[v] & ~3u) | kGone;
-                P.core[v] = k;
-                if (P.rnd) P.rnd[v] = r - 1;
+        uint32_t fcur = c->fcnt[r % 3];
+        uint32_t* Fcur = P.front[r % 3];
+        const bool undo = multi && retired - seg + fcur > kBandMax;
+        // the bitmaps of F_{r-1}'s hubs are zeroed for round r+1
+        if (r && P.hub_slots) {
+            uint32_t nhub = c->hubcnt[(r + 1) & 1];
+            if (nhub > P.hub_slots) nhub = P.hub_slots;
+            if (nhub) hub_bitmaps<NT>(P, nhub, (r + 1) & 1, true, s_pre, s_red, bytes);
+        }
+        // mark F_r; rows longer than heavy_min also go to the heavy list
+        for (uint64_t base = gwarp * 32; base < fcur && !undo; base += gwarps * 32) {
+            uint64_t i = base + lane;
+            bool hv = false;
+            uint32_t v = 0;
+            if (i < fcur) {
+                v = Fcur[i];
+                P.sl[v] = front_word(P, c, v, r & 1, hv);
+                bytes += 4 + 4 + 8 + (P.heavy_min ? 16 : 0);
             }
-            if (lead) bytes += (20ull + (P.rnd ? 4 : 0)) * nf_s;
-            if (lead) {
-                mu_alive -= c->destroyed[(r + 2) % 3];
-                c->destroyed[(r + 2) % 3] = 0;
+            if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
+        }
+        if (lead) {
+            if (r) {
                 c->big_cnt[(r + 2) % 3] = 0;
                 c->bgrab[(r + 2) % 3] = 0;
                 c->big_cnt[3 + (r + 2) % 3] = 0;
                 c->bgrab[3 + (r + 2) % 3] = 0;
             }
-            uint32_t nf_new = c->fcnt[r % 3];
-            __syncthreads();
-            if (nf_new) {
-                const uint32_t* G = P.front[r % 3];
-                for (uint32_t i = threadIdx.x; i < nf_new; i += NT) sF[i] = G[i];
-                if (lead) bytes += 4ull * nf_new;
-                nf_s = nf_new;
-            } else {
-                s_jump = true;
-            }
+            c->fcnt[(r + 1) % 3] = 0;
+            c->hcnt[(r + 1) % 3] = 0;
+            c->grab[(r + 1) % 3] = 0;
         }
-        // the counter that collects round r+2's appends was last read at the
-        // start of round r-1
-        if (lead) c->fcnt[(r + 2) % 3] = 0;
-        PHASE(4);
-        if (s_jump) {
-            // Level jump over the alive set, distributed: each block compacts
-            // its own slice (kept in shared memory), takes the slice minimum
-            // and the slice vertices attaining it, and publishes them; after
-            // the barrier every block combines the slice minima and gathers the
-            // frontier from the slices that attain the global minimum.
-            uint32_t kept = 0;
-            unsigned long long lmin = ~0ull;
-            {
-                if (threadIdx.x == 0) s_n = 0;
-                __syncthreads();
-                for (uint32_t base = 0; base < na_loc; base += NT) {
-                    uint32_t i = base + threadIdx.x;
-                    uint32_t v = i < na_loc ? sA[i] : 0u;
-                    uint32_t s = i < na_loc ? st_of(P.sl[v]) : (uint32_t)kGone;
-                    unsigned long long d = i < na_loc ? P.deg[v] : ~0ull;
-                    bool keep = s == kAlive;
-                    if (keep) lmin = d < lmin ? d : lmin;
-                    if (keep && P.snap) P.snap[v] = d;
-                    uint32_t tot;
-                    uint32_t at = block_scan_count<NT>(keep ? 1u : 0u, s_wtot, &tot);
-                    uint32_t o = s_n;
-                    __syncthreads();   // every read of this pass precedes any write
-                    if (keep) sA[o + at] = v;
-                    __syncthreads();
-                    if (threadIdx.x == 0) s_n = o + tot;
-                }
-                __syncthreads();
-                kept = s_n;
-                if (lead) bytes += 16ull * na_entry;
+        BARRIER(0);
+        if (undo) {
+            // back to the band's start; its first level goes alone, as do the
+            // levels of the next 2^fails - 1 jumps
+            for (uint64_t i = gtid; i < alive_cnt; i += gthreads) {
+                const uint32_t v = P.alive[ap][i];
+                P.deg[v] = P.c0[v];
+                P.sl[v] = kAlive;
+                bytes += 4 + 16 + 4;
             }
-            lmin = warp_min_u64(lmin);
-            if (lane == 0) s_red[wid] = lmin;
-            __syncthreads();
-            lmin = ~0ull;
-            for (int w = 0; w < NW; w++) lmin = s_red[w] < lmin ? s_red[w] : lmin;
-            __syncthreads();
-            na_loc = kept;
-            // the slice vertices attaining the slice minimum, published in
-            // this block's part of the jump list
-            {
-                if (threadIdx.x == 0) s_n = 0;
-                __syncthreads();
-                for (uint32_t base = 0; base < na_loc; base += NT) {
-                    uint32_t i = base + threadIdx.x;
-                    uint32_t v = i < na_loc ? sA[i] : 0u;
-                    bool in = i < na_loc && P.deg[v] == lmin;
-                    uint32_t tot;
-                    uint32_t at = block_scan_count<NT>(in ? 1u : 0u, s_wtot, &tot);
-                    uint32_t o = s_n;
-                    if (in) P.jf[slice_lo + o + at] = v;
-                    __syncthreads();
-                    if (threadIdx.x == 0) s_n = o + tot;
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    P.jblk[blockIdx.x] = make_ulonglong2(lmin, ((unsigned long long)na_loc << 32) | s_n);
-                }
+            if (lead) {
+                c->fcnt[r % 3] = 0;
+                c->destroyed = gone0;
             }
-            // rows of this slice lose their removed entries once the slice
-            // has halved (no block reads rows during this phase)
-            if (P.compact && 2ull * na_loc <= cmp_loc) {
-                cmp_loc = na_loc;
+            fcur = 0;
+            retired = seg;
+            nb--;
+            multi = false;
+            k = klow;
+            fails = fails < 10 ? fails + 1 : 10;
+            hold = 1u << (fails - 1);
+            BARRIER(0);
+        }
+
+        // ------------------------------------------------------ band jump
+        if (fcur == 0) {
+            const uint32_t left = P.n - retired;
+            if (left == 0) break;
+            if (multi) fails = 0;
+            const bool banding = left <= P.band_max && nb < kMaxBands && hold == 0 &&
+                                 (P.h > 2 || rs >= kBandAfter2);
+            if (hold) hold--;
+            const uint32_t* Ain = P.alive[ap];
+            uint32_t* Aout = P.alive[ap ^ 1];
+            uint32_t* ghist = c->hist[jumps & 1];
+            unsigned long long mn = ~0ull;
+            if (banding) {
+                for (uint32_t i = threadIdx.x; i < kBins; i += NT) s_hist[i] = 0;
+                if (lead && c->band_n == 0) {
+                    c->band_n = left;
+                    c->band_round = r;
+                }
+                __syncthreads();
+            }
+            for (uint64_t base = gwarp * 32; base < alive_cnt; base += gwarps * 32) {
+                uint64_t i = base + lane;
+                bool keep = false;
+                uint32_t v = 0;
+                if (i < alive_cnt) {
+                    v = Ain[i];
+                    bytes += 4 + 4;
+                    if (st_of(P.sl[v]) != kGone) {
+                        keep = true;
+                        unsigned long long d = P.deg[v];
+                        mn = d < mn ? d : mn;
+                        if (P.snap) P.snap[v] = d;
+                        if (banding) {
+                            P.c0[v] = d;
+                            atomicAdd(&s_hist[d > k ? bin_of(d - k - 1) : 0u], 1u);
+                            bytes += 8;
+                        }
+                        bytes += 8 + 4;
+                    }
+                }
+                warp_append(keep, v, &c->new_alive[jumps & 1], Aout);
+            }
+            mn = warp_min_u64(mn);
+            if (lane == 0 && mn != ~0ull) atomicMin(&c->min_deg[jumps & 1], mn);
+            if (banding) {
+                __syncthreads();
+                for (uint32_t i = threadIdx.x; i < kBins; i += NT)
+                    if (s_hist[i]) atomicAdd(&ghist[i], s_hist[i]);
+            }
+            BARRIER(1);
+            ap ^= 1;
+            alive_cnt = left;
+            const unsigned long long m2 = c->min_deg[jumps & 1];
+            const unsigned long long kmin = m2 > k ? m2 : k;
+            multi = false;
+            klow = k;
+            seg = retired;
+            unsigned long long kt = 0;
+            if (banding && m2 > k) {
+                const uint32_t tmax = (uint32_t)sqrtf(kBandFill * (float)left);
+                kt = pick_threshold<NT>(ghist, k, tmax, tmax / 8, s_wtot, &s_n);
+                multi = kt > m2;
+            }
+            if (lead) {
+                gone0 = c->destroyed;
+                const unsigned long long mu = P.mu0 - gone0;
+                if (multi) {
+                    Band& b = P.bands[nb];
+                    b.k = k;
+                    b.mu = mu;
+                    b.seg = retired;
+                    b.rbase = rs;
+                    b.nlev = 0;
+                    b.rounds = 0;
+                } else {
+                    P.t_k[retired] = kmin;
+                    P.t_size[retired] = left;
+                    P.t_mu[retired] = mu;
+                }
+                c->min_deg[(jumps + 1) & 1] = ~0ull;
+                c->new_alive[(jumps + 1) & 1] = 0;
+            }
+            if (blockIdx.x == gridDim.x - 1 && P.band_max)
+                for (uint32_t i = threadIdx.x; i < kBins; i += NT) c->hist[(jumps + 1) & 1][i] = 0;
+            if (multi) nb++;
+            k = multi ? kt : kmin;
+            jumps++;
+            // Rows may be compacted in this same phase: compaction keeps
+            // every vertex that is not removed, whether or not it is being
+            // marked frontier concurrently (a frontier vertex of count 0 is
+            // marked gone, but lies in no clique).
+            if (P.compact && 2ull * left <= compacted_at) {
+                compacted_at = left;
                 ncompact++;
-                for (uint32_t i = wid; i < na_loc; i += NW) compact_row(P, sA[i], bytes);
+                for (uint64_t i = gwarp; i < left; i += gwarps) compact_row(P, Aout[i], 0u, bytes);
             }
-            // Every block must have read the counts for this jump before any
-            // block starts the round's decrements.
-            BARRIER(5);
-            // combine: global minimum, alive count, and the frontier
-            {
-                unsigned long long gm = ~0ull;
-                unsigned long long tot_alive = 0;
-                uint32_t cnt_t = 0;
-                unsigned long long min_t = ~0ull;
-                if (threadIdx.x < gridDim.x) {
-                    ulonglong2 e = P.jblk[threadIdx.x];
-                    min_t = e.x;
-                    tot_alive = e.y >> 32;
-                    cnt_t = (uint32_t)(e.y & 0xffffffffull);
-                    gm = min_t;
-                }
-                gm = warp_min_u64(gm);
-                tot_alive = warp_sum(tot_alive);
-                if (lane == 0) {
-                    s_red[wid] = gm;
-                    s_pre[wid] = tot_alive;
-                }
-                __syncthreads();
-                gm = ~0ull;
-                tot_alive = 0;
-                for (int w = 0; w < NW; w++) {
-                    gm = s_red[w] < gm ? s_red[w] : gm;
-                    tot_alive += s_pre[w];
-                }
-                __syncthreads();
-                if (tot_alive == 0) break;
-                if (tot_alive <= P.tail_max) {
-                    // Hand the rest to the cluster tail kernel: every block
-                    // writes its compacted slice into one list (blocks in
-                    // order) and gives those vertices their tail local ids.
-                    uint32_t before_me = 0;
-                    if (threadIdx.x < gridDim.x && threadIdx.x < blockIdx.x)
-                        before_me = (uint32_t)(P.jblk[threadIdx.x].y >> 32);
-                    uint32_t base;
-                    block_scan_count<NT>(before_me, s_wtot, &base);
-                    for (uint32_t i = threadIdx.x; i < na_loc; i += NT) {
-                        uint32_t v = sA[i];
-                        P.alive[0][base + i] = v;
-                        P.sl[v] = ((base + i) << 2) | kAlive;
+            for (uint64_t base = gwarp * 32; base < left; base += gwarps * 32) {
+                uint64_t i = base + lane;
+                bool in = false, hv = false;
+                uint32_t v = 0;
+                if (i < left) {
+                    v = Aout[i];
+                    bytes += 4 + 8;
+                    if (P.deg[v] <= k) {
+                        in = true;
+                        P.sl[v] = front_word(P, c, v, r & 1, hv);
+                        bytes += 4 + 4 + (P.heavy_min ? 16 : 0);
                     }
-                    if (lead) {
-                        c->tail_n = (uint32_t)tot_alive;
-                        c->tail_round = r;
-                        c->tail_entry = (uint32_t)tot_alive;
-                        c->tail_entry_round = r;
-                        c->mu_tail = mu_alive;
-                        bytes += 12ull * tot_alive;
-                    }
-                    break;
                 }
-                k = gm > k ? gm : k;
-                na_s = (uint32_t)tot_alive;
-                if (lead) {
-                    P.lvl_k[nlev] = k;
-                    P.lvl_size[nlev] = na_s;
-                    P.lvl_mu[nlev] = mu_alive;
-                }
-                nlev++;
-                // frontier = the published vertices of slices whose minimum is gm
-                uint32_t take = (threadIdx.x < gridDim.x && min_t == gm) ? cnt_t : 0u;
-                uint32_t tot;
-                uint32_t at = block_scan_count<NT>(take, s_wtot, &tot);
-                if (threadIdx.x < gridDim.x) {
-                    s_pre[threadIdx.x] = ((unsigned long long)at << 32) | take;
-                }
-                __syncthreads();
-                for (uint32_t t = wid; t < gridDim.x; t += NW) {
-                    unsigned long long e = s_pre[t];
-                    uint32_t ct = (uint32_t)(e & 0xffffffffull), o = (uint32_t)(e >> 32);
-                    uint64_t lo = (uint64_t)na_entry * t / gridDim.x;
-                    for (uint32_t j = lane; j < ct; j += 32) sF[o + j] = P.jf[lo + j];
-                }
-                nf_s = tot;
-                if (lead) bytes += 16ull * gridDim.x + 8ull * nf_s;
-                __syncthreads();
+                warp_append(in, v, &c->fcnt[r % 3], Fcur);
+                if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
+            }
+            BARRIER(2);
+            fcur = c->fcnt[r % 3];
+        }
+        // ---------------------------------------------------------- P2
+        if (P.hub_slots) {
+            uint32_t nhub = c->hubcnt[r & 1];
+            if (nhub > P.hub_slots) nhub = P.hub_slots;
+            if (lead) c->hubcnt[(r + 1) & 1] = 0;   // read last in this round's P1
+            if (nhub) {
+                hub_bitmaps<NT>(P, nhub, r & 1, false, s_pre, s_red, bytes);
+                BARRIER(3);
             }
         }
-        // mark the frontier (identical writes in every block)
-        for (uint32_t i = threadIdx.x; i < nf_s; i += NT) {
-            uint32_t v = sF[i];
-            P.sl[v] = (P.sl[v] & ~3u) | kFront;
-        }
-        if (lead) bytes += 8ull * nf_s;
-        __syncthreads();
-        if (P.h >= 3) build_bitmaps<NT>(P, sF, nf_s, sBM, bm_words);
-        PHASE(6);
-        {
-            unsigned long long destroyed = 0;
-            process_frontier<NT>(P, sF, nf_s, k, P.front[(r + 1) % 3], &c->fcnt[(r + 1) % 3],
-                                 &c->big_cnt[r % 3], wC, wCnt, wRows, P.h >= 3 ? sBM : nullptr,
-                                 bm_words, s_pre, s_red, nullptr, 0, nullptr, nullptr, 0,
-                                 destroyed, items, bytes);
-            unsigned long long bd = block_sum<NT>(destroyed, s_red);
-            if (threadIdx.x == 0 && bd) atomicAdd(&c->destroyed[r % 3], bd);
-            BARRIER(7);
+        // when everything left leaves at once there is no count to lower
+        if (retired + fcur < P.n) {
+            process_frontier<NT>(P, R1, Fcur, fcur, k, P.front[(r + 1) % 3],
+                                 &c->fcnt[(r + 1) % 3], &c->big_cnt[r % 3], wC, wCnt, wRows,
+                                 s_pre, s_red, c->hcnt[r % 3], &c->grab[r % 3], &s_grab, r & 1,
+                                 items, bytes);
+            BARRIER(3);
             if (P.big_cap) {
-                uint32_t nb = c->big_cnt[r % 3];
-                uint32_t nm = c->big_cnt[3 + r % 3];
-                if (nb || nm) {
-                    if (nb > P.big_cap) nb = (uint32_t)P.big_cap;
-                    if (nm > P.mid_cap) nm = P.mid_cap;
-                    if (nm) {
-                        drain_mid<NT>(P, nm, &c->bgrab[3 + r % 3], k, P.front[(r + 1) % 3],
-                                      &c->fcnt[(r + 1) % 3], &c->destroyed[r % 3], bytes);
-                        __syncthreads();
-                    }
-                    unsigned long long d2 = 0;
-                    for (;;) {
-                        if (threadIdx.x == 0) s_grab = atomicAdd(&c->bgrab[r % 3], 1u);
-                        __syncthreads();
-                        const uint32_t i = s_grab;
-                        __syncthreads();
-                        if (i >= nb) break;
-                        uint2 it = P.big[i];
-                        process_big(P, it.x, it.y, k, P.front[(r + 1) % 3],
-                                    &c->fcnt[(r + 1) % 3], smem, nullptr, d2, bytes);
-                    }
-                    if (threadIdx.x == 0 && d2) atomicAdd(&c->destroyed[r % 3], d2);
-                    BARRIER(7);
+                const uint32_t nbig = c->big_cnt[r % 3], nmid = c->big_cnt[3 + r % 3];
+                if (nbig || nmid) {
+                    process_queued<NT>(P, R1, r % 3, nbig, nmid, k, P.front[(r + 1) % 3],
+                                       &c->fcnt[(r + 1) % 3], smem, true, r & 1, &s_grab, bytes);
+                    BARRIER(3);
                 }
             }
         }
         r++;
+    }
+
+    // ============================================================ phase 2
+    if (nb) {
+        const uint64_t t2 = lead ? globaltimer_ns() : 0;
+        // every vertex gets its key; members of multi-level bands are alive
+        // again with their count at the band's start
+        // (earlier vertices keep key 0, below every band's)
+        const uint32_t first = P.bands[0].seg;
+        for (uint64_t i = first + gtid; i < P.n; i += gthreads) {
+            const uint32_t v = P.mem[i], key = P.band_of[v];
+            if (key & 1u) P.deg[v] = P.c0[v];
+            P.sl[v] = (key << kKeyShift) | ((key & 1u) ? kAlive : kGone);
+            bytes += 4 + 4 + 4 + 16;
+        }
+        if (lead) {
+            c->fcnt[0] = c->fcnt[1] = c->fcnt[2] = 0;
+            c->busy[0] = c->busy[1] = c->busy[2] = 0;
+            for (int i = 0; i < 6; i++) c->big_cnt[i] = c->bgrab[i] = 0;
+        }
+        // band sizes: the first position past seg whose key differs
+        for (uint64_t i = first + gtid; i < P.n; i += gthreads) {
+            const uint32_t key = P.band_of[P.mem[i]];
+            if ((key & 1u) && (i + 1 == P.n || P.band_of[P.mem[i + 1]] != key)) {
+                Band& b = P.bands[key >> 1];
+                b.size = b.left = (uint32_t)(i + 1) - b.seg;
+                b.above = P.n - (uint32_t)(i + 1);
+            }
+        }
+        BARRIER(4);
+        // rows of the members without earlier bands
+        for (uint64_t i = first + gwarp; i < P.n; i += gwarps) {
+            const uint32_t v = P.mem[i], key = P.sl[v] >> kKeyShift;
+            if (key & 1u) compact_row(P, v, key, bytes);
+        }
+        BARRIER(5);
+        uint32_t q = 0;   // round
+        uint32_t flip = 0;
+        for (;;) {
+            // ------------------------------------------------------- A
+            uint32_t* F = P.front[q & 1];
+            uint32_t* fcnt = &c->fcnt[q % 3];
+            for (uint32_t bi = blockIdx.x; bi < nb; bi += gridDim.x) {
+                Band& B = P.bands[bi];
+                const uint32_t left = B.left;
+                if (left == 0) continue;
+                const uint32_t seg = B.seg;
+                const unsigned long long bk = B.k;
+                const uint32_t rb = B.rounds;
+                // retire the frontier; least count, members at <= k and
+                // members left
+                unsigned long long mn = ~0ull, sum = 0;
+                uint32_t cnt = 0, al = 0;
+                uint32_t v0 = 0, w0 = kGone;      // this thread's first member
+                unsigned long long d0 = 0;
+                for (uint32_t i = threadIdx.x; i < left; i += NT) {
+                    const uint32_t v = P.mem[seg + i];
+                    uint32_t w = P.sl[v];
+                    unsigned long long d = 0;
+                    if (st_of(w) != kGone) {
+                        d = P.deg[v];
+                        if (st_of(w) == kFront) {
+                            sum += d;
+                            P.core[v] = bk;
+                            if (P.rnd) P.rnd[v] = rb - 1;
+                            w = (w & ~3u) | kGone;
+                            P.sl[v] = w;
+                            bytes += 12;
+                        } else {
+                            al++;
+                            cnt += d <= bk;
+                            mn = d < mn ? d : mn;
+                        }
+                        bytes += 8;
+                    }
+                    bytes += 8;
+                    if (i < NT) {
+                        v0 = v;
+                        w0 = w;
+                        d0 = d;
+                    }
+                }
+                mn = warp_min_u64(mn);
+                sum = warp_sum(sum);
+                cnt = __reduce_add_sync(0xffffffffu, cnt);
+                al = __reduce_add_sync(0xffffffffu, al);
+                if (lane == 0) {
+                    s_bmin[flip][wid] = mn;
+                    s_bsum[flip][wid] = sum;
+                    s_bcnt[flip][wid] = cnt;
+                    s_bleft[flip][wid] = al;
+                }
+                __syncthreads();
+                mn = warp_min_u64(lane < NW ? s_bmin[flip][lane] : ~0ull);
+                sum = warp_sum(lane < NW ? s_bsum[flip][lane] : 0ull);
+                cnt = __reduce_add_sync(0xffffffffu, lane < NW ? s_bcnt[flip][lane] : 0u);
+                al = __reduce_add_sync(0xffffffffu, lane < NW ? s_bleft[flip][lane] : 0u);
+                flip ^= 1;
+                const unsigned long long mu = B.mu - sum;
+                unsigned long long kk = bk;
+                const bool jump = cnt == 0;
+                if (jump && al) {
+                    kk = mn > bk ? mn : bk;
+                    if (P.snap)
+                        for (uint32_t i = threadIdx.x; i < left; i += NT) {
+                            const uint32_t v = P.mem[seg + i];
+                            if (st_of(P.sl[v]) == kAlive) P.snap[v] = P.deg[v];
+                        }
+                }
+                // mark the next frontier; members of count 0 lie in no clique and
+                // have nothing to enumerate
+                for (uint32_t b0 = 0; b0 < left; b0 += NT) {
+                    const uint32_t i = b0 + threadIdx.x;
+                    uint32_t v = v0, w = w0;
+                    unsigned long long d = d0;
+                    if (b0) {
+                        w = kGone;
+                        if (i < left) {
+                            v = P.mem[seg + i];
+                            w = P.sl[v];
+                            d = P.deg[v];
+                        }
+                    }
+                    const bool in = i < left && st_of(w) == kAlive && d <= kk;
+                    if (in) P.sl[v] = (w & ~3u) | kFront;
+                    warp_append(in && d, v, fcnt, F);
+                }
+                __syncthreads();   // every thread has read the band's record
+                if (threadIdx.x == 0) {
+                    B.mu = mu;
+                    if (al) {
+                        atomicAdd(&c->busy[q % 3], 1u);
+                        B.rounds = rb + 1;
+                        if (jump) {
+                            const uint32_t at = seg + B.nlev;
+                            P.t_k[at] = kk;
+                            P.t_size[at] = B.above + al;
+                            P.t_mu[at] = mu;
+                            B.nlev++;
+                            B.k = kk;
+                        }
+                    } else {
+                        B.left = 0;
+                    }
+                }
+            }
+            if (lead) {
+                c->fcnt[(q + 1) % 3] = 0;
+                c->busy[(q + 1) % 3] = 0;
+                if (q) {
+                    c->big_cnt[(q + 2) % 3] = 0;
+                    c->bgrab[(q + 2) % 3] = 0;
+                    c->big_cnt[3 + (q + 2) % 3] = 0;
+                    c->bgrab[3 + (q + 2) % 3] = 0;
+                }
+            }
+            BARRIER(4);
+            if (c->busy[q % 3] == 0) break;
+            // ------------------------------------------------------- P2
+            process_bands<NT>(P, R2, F, *fcnt, &c->big_cnt[q % 3], wC, wCnt, wRows, s_pre, s_red,
+                              items, bytes);
+            BARRIER(6);
+            if (P.big_cap) {
+                const uint32_t nbig = c->big_cnt[q % 3], nmid = c->big_cnt[3 + q % 3];
+                if (nbig || nmid) {
+                    process_queued<NT>(P, R2, q % 3, nbig, nmid, 0ull, nullptr, nullptr, smem,
+                                       false, 0, &s_grab, bytes);
+                    BARRIER(7);
+                }
+            }
+            q++;
+        }
+        if (lead) c->phase2_ns = globaltimer_ns() - t2;
+        r += q;
+    }
+    // ======================================================== final pass
+    // level records in order (their positions ascend), and the removal
+    // rounds: a band's rounds start after those of the bands before it
+    {
+        uint32_t run = 0;
+        for (uint32_t b0 = 0; b0 < nb; b0 += NT) {
+            const uint32_t i = b0 + threadIdx.x;
+            const uint32_t x = i < nb ? P.bands[i].rounds : 0u;
+            uint32_t tot;
+            const uint32_t at = block_scan_count<NT>(x, s_wtot, &tot);
+            if (blockIdx.x == 0 && i < nb) P.bands[i].size = run + at;   // size is free now
+            run += tot;
+        }
+        const uint32_t lo = (uint32_t)((uint64_t)P.n * blockIdx.x / gridDim.x);
+        const uint32_t hi = (uint32_t)((uint64_t)P.n * (blockIdx.x + 1) / gridDim.x);
+        uint32_t mine = 0;
+        for (uint32_t i = lo + threadIdx.x; i < hi; i += NT) mine += P.t_size[i] != 0;
+        uint32_t tot;
+        (void)block_scan_count<NT>(mine, s_wtot, &tot);
+        if (threadIdx.x == 0) P.blkcnt[blockIdx.x] = tot;
+        BARRIER(0);
+        if (P.rnd && nb) {
+            const uint32_t tail = run;
+            for (uint64_t i = gtid; i < P.n; i += gthreads) {
+                const uint32_t key = P.band_of[i], j = key >> 1;
+                uint32_t add = j < nb ? P.bands[j].size : tail;
+                if (key & 1u) add += P.bands[j].rbase;
+                P.rnd[i] += add;
+            }
+        }
+        uint32_t before = 0, all = 0;
+        for (uint32_t t = threadIdx.x; t < gridDim.x; t += NT) {
+            const uint32_t x = P.blkcnt[t];
+            all += x;
+            before += t < blockIdx.x ? x : 0u;
+        }
+        uint32_t base, nlev;
+        (void)block_scan_count<NT>(before, s_wtot, &base);
+        (void)block_scan_count<NT>(all, s_wtot, &nlev);
+        for (uint32_t b0 = lo; b0 < hi; b0 += NT) {
+            const uint32_t i = b0 + threadIdx.x;
+            const uint32_t sz = i < hi ? P.t_size[i] : 0u;
+            const uint32_t at = base + block_scan_count<NT>(sz ? 1u : 0u, s_wtot, &tot);
+            if (sz) {
+                P.lvl_k[at] = P.t_k[i];
+                P.lvl_size[at] = sz;
+                P.lvl_mu[at] = P.t_mu[i];
+                if (at + 1 == nlev) c->kmax = P.t_k[i];
+            }
+            base += tot;
+        }
+        if (lead) {
+            c->nlevels = nlev;
+            c->rounds = rs + run;
+        }
     }
 out:
 #undef BARRIER
 #undef PHASE
     if (lead) {
         for (int i = 0; i < 8; i++) c->tph[i] = tph[i];
-        c->kmax = k;
-        c->nlevels = nlev;
-        c->rounds = r;
+        c->nbands = nb;
+        c->grid_rounds = r;
         c->barrier_ns = waited;
         c->barriers = nbar;
         c->compactions = ncompact;
@@ -1529,6 +1800,155 @@ out:
     bytes = warp_sum(bytes);
     if (lane == 0 && items) atomicAdd(&c->items, items);
     if (lane == 0 && bytes) atomicAdd(&c->bytes, bytes);
+}
+
+// The h = 2 peel of a small graph by one block: every count, row start and
+// state in shared memory, so that a round is a few block barriers and one
+// trip to the rows (L2) instead of grid barriers and global bookkeeping.
+// `order` lists the vertices as they leave: F_r is order[a, b), F_{r+1} is
+// appended behind it.  stamp[v] is the round v leaves in (kStay while alive),
+// so a vertex is a frontier member in that round and gone after it without
+// being marked; the thread whose decrement takes a count to k appends the
+// vertex.  Frontier members of larger id are lowered too: what is left of a
+// frontier member's count is the number of edges credited to it.
+// Bound by the latency of a round (block scan, row load, shared atomics).
+struct Peel2Block {
+    uint32_t n;
+    const uint64_t* off;
+    const uint32_t* adj;
+    uint64_t* core;
+    uint32_t* rnd;
+    uint64_t* lvl_k;
+    uint32_t* lvl_size;
+    uint64_t* lvl_mu;
+    PeelCtrl* ctrl;
+    unsigned long long mu0;
+    uint32_t k0;
+};
+
+constexpr size_t peel2_block_smem(uint32_t n) { return (size_t)n * 12 + 16; }
+
+__global__ void __launch_bounds__(1024, 1) k_peel2_block(Peel2Block P) {
+    constexpr int NT = 1024, NW = NT / 32;
+    constexpr uint32_t kStay = 0xffffu;   // rounds stay below n <= kOneBlockN
+    extern __shared__ uint32_t smem[];
+    uint32_t* deg = smem;                                  // [n]
+    uint32_t* at = deg + P.n;                              // [n + 1] row starts
+    uint16_t* stamp = (uint16_t*)(at + P.n + 1);           // [n]
+    uint16_t* order = stamp + P.n;                         // [n]
+    __shared__ uint32_t s_pre[NT];
+    __shared__ uint32_t s_wtot[NW];
+    __shared__ uint32_t s_min[NW];
+    __shared__ unsigned long long s_sum[NW];
+    __shared__ uint32_t s_end;
+    const uint32_t n = P.n, tid = threadIdx.x;
+    const unsigned lane = lane_id(), wid = warp_id();
+    for (uint32_t v = tid; v <= n; v += NT) at[v] = (uint32_t)P.off[v];
+    __syncthreads();
+    for (uint32_t v = tid; v < n; v += NT) {
+        deg[v] = at[v + 1] - at[v];
+        stamp[v] = (uint16_t)kStay;
+    }
+    if (tid == 0) s_end = 0;
+    __syncthreads();
+    uint32_t a = 0, b = 0;          // F_r = order[a, b)
+    uint32_t r = 0, k = P.k0, nlev = 0;
+    unsigned long long mu = P.mu0, gone = 0;   // gone: this thread's share since the last level
+    unsigned long long items = 0;
+    for (;;) {
+        if (a == b) {
+            // a new level: k = max(k, least count left), recorded before its
+            // first round
+            if (a == n) break;
+            uint32_t mn = 0xffffffffu;
+            for (uint32_t v = tid; v < n; v += NT)
+                if (stamp[v] == kStay) mn = min(mn, deg[v]);
+            mn = __reduce_min_sync(0xffffffffu, mn);
+            gone = warp_sum(gone);
+            if (lane == 0) {
+                s_min[wid] = mn;
+                s_sum[wid] = gone;
+            }
+            gone = 0;
+            __syncthreads();
+            mn = __reduce_min_sync(0xffffffffu, s_min[lane]);
+            mu -= warp_sum(s_sum[lane]);
+            k = mn > k ? mn : k;
+            if (tid == 0) {
+                P.lvl_k[nlev] = k;
+                P.lvl_size[nlev] = n - a;
+                P.lvl_mu[nlev] = mu;
+            }
+            nlev++;
+            for (uint32_t v0 = 0; v0 < n; v0 += NT) {
+                const uint32_t v = v0 + tid;
+                const bool in = v < n && stamp[v] == kStay && deg[v] <= k;
+                const unsigned bal = __ballot_sync(0xffffffffu, in);
+                if (!bal) continue;
+                uint32_t base = 0;
+                if (lane == 0) base = atomicAdd(&s_end, (uint32_t)__popc(bal));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (in) {
+                    order[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)v;
+                    stamp[v] = (uint16_t)r;
+                }
+            }
+            __syncthreads();
+            b = s_end;
+        }
+        // the rows of F_r, flattened over the block, NT frontier vertices at
+        // a time
+        for (uint32_t f0 = a; f0 < b; f0 += NT) {
+            const uint32_t i = f0 + tid;
+            uint32_t d = 0;
+            if (i < b) {
+                const uint32_t v = order[i];
+                d = at[v + 1] - at[v];
+                P.core[v] = k;
+                if (P.rnd) P.rnd[v] = r;
+            }
+            uint32_t T;
+            const uint32_t ex = block_scan_count<NT>(d, s_wtot, &T);
+            s_pre[tid] = ex;   // entries past the frontier hold T
+            __syncthreads();
+            if (tid == 0) items += T;
+            const uint32_t nb = b - f0 < NT ? b - f0 : NT;
+            for (uint32_t t = tid; t < T; t += NT) {
+                uint32_t lo = 0, hi = nb;   // last j with s_pre[j] <= t
+                while (hi - lo > 1) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (s_pre[mid] <= t) lo = mid; else hi = mid;
+                }
+                const uint32_t v = order[f0 + lo];
+                const uint32_t u = P.adj[at[v] + (t - s_pre[lo])];
+                const uint32_t su = stamp[u];
+                if (su > r) {
+                    // alive (perhaps already queued for the next round)
+                    if (atomicSub(&deg[u], 1u) == k + 1u) {
+                        order[atomicAdd(&s_end, 1u)] = (uint16_t)u;
+                        stamp[u] = (uint16_t)(r + 1u);
+                    }
+                } else if (su == r && u > v) {
+                    atomicSub(&deg[u], 1u);
+                }
+            }
+            __syncthreads();
+        }
+        for (uint32_t i = a + tid; i < b; i += NT) gone += deg[order[i]];
+        a = b;
+        b = s_end;
+        r++;
+        __syncthreads();   // every thread has read s_end before it grows again
+    }
+    if (tid == 0) {
+        PeelCtrl* c = P.ctrl;
+        c->kmax = k;
+        c->nlevels = nlev;
+        c->rounds = r;
+        c->grid_rounds = r;
+        c->items = items;
+        c->bytes = items * 4ull + n * 20ull;
+    }
 }
 
 __global__ void k_peel_init(uint32_t n, const uint64_t* off, const uint64_t* split,
@@ -1545,92 +1965,6 @@ __global__ void k_peel_init(uint32_t n, const uint64_t* off, const uint64_t* spl
         c->min_deg[0] = ~0ull;
         c->min_deg[1] = ~0ull;
     }
-}
-
-#include "peel_tail.inc"
-
-// Tail launch shapes: the largest cluster this device co-schedules (16,
-// else 8) and the largest alive set whose per-CTA state fits its shared
-// memory; `grows` selects rows in global memory.
-struct TailShape {
-    uint32_t cs = 0, cap = 0;
-    size_t smem = 0;
-};
-
-TailShape find_tail_shape(bool grows) {
-    TailShape t;
-    const size_t budget = 220 * 1024;
-    const void* fn = grows ? (const void*)k_peel_tail<true> : (const void*)k_peel_tail<false>;
-    for (uint32_t cs : {16u, 8u}) {
-        uint32_t cap = 0;
-        for (uint32_t cc = 32 * cs; cc <= kTailMaxAlive; cc += 32 * cs) {
-            size_t scratch = grows ? SIZE_MAX : (size_t)(cc / cs) * (cc / 32) * 4;
-            if (tail_smem_bytes(grows, cc, cs) <= budget && tail_np(cc) * 4 <= scratch &&
-                (grows || cc <= 8192))
-                cap = cc;
-        }
-        if (!cap) continue;
-        size_t smem = tail_smem_bytes(grows, cap, cs);
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                cudaSuccess ||
-            (cs > 8 &&
-             cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                 cudaSuccess)) {
-            (void)cudaGetLastError();
-            continue;
-        }
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = cs;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(cs);
-        cfg.blockDim = dim3(kTailNT);
-        cfg.dynamicSmemBytes = smem;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) != cudaSuccess) {
-            (void)cudaGetLastError();
-            continue;
-        }
-        if (nc >= 1) {
-            t.cs = cs;
-            t.cap = cap;
-            t.smem = smem;
-            break;
-        }
-    }
-    return t;
-}
-
-const TailShape& tail_shape(bool grows) {
-    static TailShape cached[2];
-    static bool done[2] = {false, false};
-    if (!done[grows]) {
-        cached[grows] = find_tail_shape(grows);
-        done[grows] = true;
-    }
-    return cached[grows];
-}
-
-template <bool GROWS>
-cudaError_t launch_tail(const TailParams& T, const TailShape& sh, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = sh.cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(sh.cs);
-    cfg.blockDim = dim3(kTailNT);
-    cfg.dynamicSmemBytes = sh.smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, k_peel_tail<GROWS>, T);
 }
 
 // Failure detection: the grid barrier of k_peel with one block withheld
@@ -1655,14 +1989,48 @@ cudaError_t launch_peel(PeelParams& P, int sms, size_t smem, cudaStream_t s, uns
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel<NT>, NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-    // one block per SM: the fewest barrier arrivals; every block holds the
-    // small-regime lists in its own shared memory
+    // one block per SM: the fewest barrier arrivals
     unsigned grid = (unsigned)sms;
     *grid_out = grid;
     void* args[] = {&P};
     e = cudaLaunchCooperativeKernel((void*)k_peel<NT>, dim3(grid), dim3(NT), args, smem, s);
     note_launch();
     return e;
+}
+
+dsd_status run_peel2_block(dsd_graph* g, uint32_t n, const uint64_t* off, const uint32_t* adj,
+                           uint64_t mu0, uint64_t* core, uint32_t* rnd, uint64_t* lvl_k,
+                           uint32_t* lvl_size, uint64_t* lvl_mu, PeelResult* res,
+                           uint64_t kstart) {
+    cudaStream_t s = g->stream;
+    PeelCtrl* ctrl = nullptr;
+    DSD_TRY(dalloc(&ctrl, 1, s));
+    Peel2Block P{n, off, adj, core, rnd, lvl_k, lvl_size, lvl_mu, ctrl, mu0,
+                 kstart ? (uint32_t)(kstart - 1) : 0u};
+    const size_t smem = peel2_block_smem(n);
+    PeelCtrl hc;
+    cudaError_t e = cudaMemsetAsync(ctrl, 0, sizeof(PeelCtrl), s);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_peel2_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)peel2_block_smem(kOneBlockN));
+    if (e == cudaSuccess) {
+        k_peel2_block<<<1, 1024, smem, s>>>(P);
+        note_launch();
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctrl, sizeof(hc), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    dev_free(ctrl, s);
+    if (e != cudaSuccess) return cuda_fail(e, "h = 2 peel", __FILE__, __LINE__);
+    res->kmax = hc.kmax;
+    res->nlevels = hc.nlevels;
+    res->rounds = hc.rounds;
+    res->grid_rounds = hc.grid_rounds;
+    res->items = hc.items;
+    res->bytes = hc.bytes;
+    res->threads = 1024;
+    res->grid = 1;
+    return DSD_OK;
 }
 
 }  // namespace
@@ -1675,6 +2043,9 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     cudaStream_t s = g->stream;
     *res = PeelResult();
     if (n == 0) return DSD_OK;
+    if (h == 2 && n <= kOneBlockN && 2 * g->m <= kOneBlockAdj && !snap && kstart < (1u << 31))
+        return run_peel2_block(g, n, off, adj, mu0, core, rnd, lvl_k, lvl_size, lvl_mu, res,
+                               kstart);
     int sms = 152;
     DSD_TRY(num_sms(&sms));
     PeelParams P;
@@ -1697,17 +2068,15 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     P.warp_cand = warp_cand_limit(h);
     P.gather_cap = P.warp_cand;
     P.compact = h >= 3 ? 1 : 0;
-    // Big items (candidate sets above kWarpCand vertices, one block each)
-    // for h >= 4; every candidate set fits 32-word rows.
+    P.band_max = peel_tail_limit();
+    // Big items (candidate sets above warp_cand vertices) for h >= 4; every
+    // candidate set fits 32-word rows.
     const bool big_items = h >= 4;
-    // Shared memory: per-warp candidate buffers (h >= 3) or the big-item
-    // bitmap, then the small-regime alive list, frontier and
-    // neighbourhood bitmaps.
-    const size_t budget = 220 * 1024;
+    // Shared memory: per-warp candidate buffers (h >= 3) or the big-item bitmap
     constexpr int NT = 1024;
     size_t work = h >= 3 ? (size_t)(NT / 32) * kWarpWords : 0;
-    // large-regime frontier vertices with more items than a block's warps
-    // take in four passes have their items spread over the whole grid
+    // phase-1 frontier vertices with more items than a block's warps take in
+    // four passes have their items spread over the whole grid
     P.heavy_min = h >= 3 ? 4u * (NT / 32) : 0u;
     // neighbourhood bitmaps for frontier vertices with rows above 512 (a
     // binary search there takes 10 or more probes): up to 64 per round, two
@@ -1725,59 +2094,35 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
         if (P.cap > kBitmapMax) big = (size_t)3 * kBitmapMax + (size_t)kBitmapMax * 32;
         if (big > work) work = big;
     }
-    size_t room = budget > work * 4 + 12 * 1024 ? budget - work * 4 - 12 * 1024 : 0;
-    // per alive entry: list 4 B + frontier 4 B + one bit per bitmap slot
-    size_t per_entry_bits = 64 + (h >= 3 ? kBitmapSlots : 0);
-    size_t asmall = room * 8 / per_entry_bits;
-    asmall &= ~(size_t)31;
-    if (asmall > 16384) asmall = 16384;
-    if (asmall > peel_small_limit()) asmall = peel_small_limit() & ~31u;
-    if (asmall < 1024) asmall = 0;
-    // the jump combines one entry per block in a single pass over the threads
-    if (sms > NT || sms > 1024) asmall = 0;
-    P.work_words = (uint32_t)work;
-    P.asmall = (uint32_t)asmall;
-    TailShape tsh_d, tsh_g;   // rows in distributed shared memory / in global memory
-    if ((h == 2 || h == 3) && asmall > 0 && peel_tail_limit() > 0 && !snap) {
-        tsh_d = tail_shape(false);
-        // global rows pay for h = 3 only: an h = 2 round is too cheap for the
-        // wider rows (measured on the 1M-vertex Chung-Lu graph)
-        if (tsh_d.cs && h == 3) tsh_g = tail_shape(true);
-        uint32_t tmax = tsh_g.cs && tsh_g.cap > tsh_d.cap ? tsh_g.cap : tsh_d.cap;
-        if (tmax > peel_tail_limit()) tmax = peel_tail_limit();
-        if (tmax <= tsh_d.cap) tsh_g = TailShape();   // the global-row launch is not needed
-        if (tsh_d.cs) P.tail_max = tmax;
-    }
-    size_t bm_words = h >= 3 ? (size_t)kBitmapSlots * (asmall / 32) : 0;
-    size_t smem = (work + 2 * asmall + bm_words) * 4;
+    const size_t smem = work * 4;
 
     uint32_t* sl = nullptr;
     uint32_t* lists = nullptr;
     uint64_t* wmeta = nullptr;
     uint32_t* wadj = nullptr;
     PeelCtrl* ctrl = nullptr;
-    uint32_t* rows_g = nullptr;
+    uint64_t* recs = nullptr;
+    Band* bands = nullptr;
     uint2* big = nullptr;
     uint32_t* mid = nullptr;
     uint32_t* heavy = nullptr;
     uint32_t* xl = nullptr;
     uint32_t* hub_bm = nullptr;
     uint32_t* hubs = nullptr;
-    ulonglong2* jblk = nullptr;
+    uint32_t* blkcnt = nullptr;
     dsd_status st = DSD_OK;
     PeelCtrl hc;
     unsigned grid = 0;
     cudaError_t e = cudaSuccess;
     const uint64_t nadj = 2 * g->m;   // both CSRs of g hold 2m entries
     if ((st = dalloc(&sl, n, s)) != DSD_OK) goto done;
-    if ((st = dalloc(&lists, (size_t)6 * n, s)) != DSD_OK) goto done;
-    if ((st = dalloc(&jblk, 1024, s)) != DSD_OK) goto done;
+    if ((st = dalloc(&lists, (size_t)8 * n, s)) != DSD_OK) goto done;
+    if ((st = dalloc(&blkcnt, (size_t)sms, s)) != DSD_OK) goto done;
     if ((st = dalloc(&wmeta, (size_t)2 * n, s)) != DSD_OK) goto done;
+    if ((st = dalloc(&recs, (size_t)3 * n, s)) != DSD_OK) goto done;
     if ((st = dalloc(&wadj, nadj + 1, s)) != DSD_OK) goto done;
     if ((st = dalloc(&ctrl, 1, s)) != DSD_OK) goto done;
-    if (tsh_g.cs &&
-        (st = dalloc(&rows_g, (size_t)tsh_g.cap * (tsh_g.cap / 32), s)) != DSD_OK)
-        goto done;
+    if (P.band_max && (st = dalloc(&bands, kMaxBands, s)) != DSD_OK) goto done;
     if (big_items) {
         P.big_cap = g->m * 2 + 1;
         if ((st = dalloc(&big, P.big_cap, s)) != DSD_OK) goto done;
@@ -1815,14 +2160,23 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     P.front[0] = lists + 2 * (size_t)n;
     P.front[1] = lists + 3 * (size_t)n;
     P.front[2] = lists + 4 * (size_t)n;
-    P.jf = lists + 5 * (size_t)n;
-    P.jblk = jblk;
+    P.mem = lists + 5 * (size_t)n;
+    P.band_of = lists + 6 * (size_t)n;
+    P.t_size = lists + 7 * (size_t)n;
+    P.blkcnt = blkcnt;
+    P.c0 = reinterpret_cast<unsigned long long*>(recs);
+    P.t_k = recs + n;
+    P.t_mu = recs + 2 * (size_t)n;
+    P.bands = bands;
+    P.nadj = adj;
+    P.nsplit = split ? split : off;
     P.wend = wmeta;
     P.wnb = wmeta + n;
     P.wadj = wadj;
     P.big = big;
     P.ctrl = ctrl;
     e = cudaMemsetAsync(ctrl, 0, sizeof(PeelCtrl), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(P.t_size, 0, (size_t)n * 4, s);
     if (e == cudaSuccess && nadj) e = cudaMemcpyAsync(wadj, adj, nadj * 4, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) {
         k_peel_init<<<sms * 4, 256, 0, s>>>(n, off, h >= 3 ? split : nullptr, sl, P.alive[0],
@@ -1831,41 +2185,6 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = launch_peel<NT>(P, sms, smem, s, &grid);
-    if (e == cudaSuccess && P.tail_max) {
-        // the launches run only if something was handed over (they read tail_n)
-        TailParams T;
-        memset(&T, 0, sizeof(T));
-        T.h = h;
-        T.off = off;
-        T.wend = P.wend;
-        T.wadj = P.wadj;
-        T.sl = P.sl;
-        T.deg = P.deg;
-        T.list[0] = P.alive[0];
-        T.list[1] = P.alive[1];
-        T.core = P.core;
-        T.rnd = P.rnd;
-        T.lvl_k = P.lvl_k;
-        T.lvl_size = P.lvl_size;
-        T.lvl_mu = P.lvl_mu;
-        T.ctrl = ctrl;
-        if (tsh_g.cs) {
-            T.cap = tsh_g.cap;
-            T.rows_cap = tsh_g.cap / tsh_g.cs;
-            T.W = tsh_g.cap / 32;
-            T.pass_below = tsh_d.cap;
-            T.rows_g = rows_g;
-            e = launch_tail<true>(T, tsh_g, s);
-        }
-        if (e == cudaSuccess) {
-            T.cap = tsh_d.cap;
-            T.rows_cap = tsh_d.cap / tsh_d.cs;
-            T.W = tsh_d.cap / 32;
-            T.pass_below = 0;
-            T.rows_g = nullptr;
-            e = launch_tail<false>(T, tsh_d, s);
-        }
-    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctrl, sizeof(PeelCtrl), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
@@ -1893,11 +2212,11 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     res->compactions = hc.compactions;
     res->threads = NT;
     res->grid = grid;
-    res->small_round = hc.small_round;
-    res->tail_n = hc.tail_entry;
-    res->tail_round = hc.tail_entry_round;
-    res->tail_ns = hc.tail_ns;
-    for (int i = 0; i < 7; i++) res->tail_tph[i] = hc.tail_tph[i];
+    res->grid_rounds = hc.grid_rounds;
+    res->band_n = hc.band_n;
+    res->band_round = hc.band_round;
+    res->bands = hc.nbands;
+    res->phase2_ns = hc.phase2_ns;
     for (int i = 0; i < 8; i++) res->tph[i] = hc.tph[i];
 done:
     dev_free(sl, s);
@@ -1905,14 +2224,15 @@ done:
     dev_free(wmeta, s);
     dev_free(wadj, s);
     dev_free(ctrl, s);
-    dev_free(rows_g, s);
+    dev_free(recs, s);
+    dev_free(bands, s);
     dev_free(big, s);
     dev_free(mid, s);
     dev_free(heavy, s);
     dev_free(xl, s);
     dev_free(hub_bm, s);
     dev_free(hubs, s);
-    dev_free(jblk, s);
+    dev_free(blkcnt, s);
     return st;
 }
 

@@ -1,0 +1,98 @@
+"""The peel's bands (levels grouped by one cascade, then peeled side by side)
+and the one-block h = 2 peel, at the sizes where their bookkeeping changes."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1906_00341_gb300 import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1906_00341_gb300 import build as b
+    b.build()
+    from paper_1906_00341_gb300 import _lib
+    _lib.load()
+    return _lib
+
+
+def ring(n, w, drop, seed):
+    """Ring lattice (neighbours at distance <= w) with a share of its edges gone:
+    a cascade that starts at a defect runs around the whole ring."""
+    i = np.arange(n, dtype=np.int64)
+    s = np.concatenate([i] * w)
+    d = np.concatenate([(i + j) % n for j in range(1, w + 1)])
+    keep = np.random.default_rng(seed).random(s.size) >= drop
+    return n, s[keep].astype(np.uint32), d[keep].astype(np.uint32)
+
+
+@pytest.mark.parametrize("limit", [0, 300, 1 << 30])
+@pytest.mark.parametrize("h", [2, 3, 4])
+def test_band_cascades(L, orc, h, limit):
+    """Cascades above the band limit (undone, the level taken alone), bands of
+    every size on a power-law graph, and no bands at all: core numbers, level
+    records and mu equal the oracle's."""
+    graphs = [ring(30000, 4, 0.002, 1),
+              gg.plant(20000, *gg.chung_lu(20000, 160000, 2.1, 900.0, 5)[1:], 70, 0.6, 6)[:3]]
+    L.dsd_set_peel_tail_limit(limit)
+    try:
+        for n, s, d in graphs:
+            og = orc.csr(n, s, d)
+            wcore, wk = orc.core_decompose(og, h)
+            wl = orc.level_stats(og, h, wcore)
+            with L.Graph.from_edges(n, s, d) as g:
+                core, k = g.core_decompose(h)
+                lv = g.level_stats(h)
+            assert k == wk and np.array_equal(core, wcore)
+            for a, b in zip(lv, wl):
+                assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
+    finally:
+        L.dsd_set_peel_tail_limit(1 << 30)
+
+
+def rounds_of(n, s, d):
+    """Core numbers and removal rounds of the level-synchronous h = 2 peel."""
+    lo, hi = np.minimum(s, d).astype(np.int64), np.maximum(s, d).astype(np.int64)
+    key = np.unique((lo * n + hi)[lo != hi])
+    u, v = key // n, key % n
+    src, dst = np.concatenate([u, v]), np.concatenate([v, u])
+    order = np.argsort(src, kind="stable")
+    src, dst = src[order], dst[order]
+    off = np.searchsorted(src, np.arange(n + 1))
+    deg = np.diff(off)
+    core, rnd = np.zeros(n, np.int64), np.zeros(n, np.int64)
+    alive = np.ones(n, bool)
+    k = r = 0
+    while alive.any():
+        k = max(k, int(deg[alive].min()))
+        f = np.nonzero(alive & (deg <= k))[0]
+        while f.size:
+            core[f], rnd[f], alive[f] = k, r, False
+            nb = np.concatenate([dst[off[x]:off[x + 1]] for x in f])
+            np.subtract.at(deg, nb, 1)
+            f = np.nonzero(alive & (deg <= k))[0]
+            r += 1
+    return core, rnd
+
+
+@pytest.mark.parametrize("n,m", [(1, 0), (33, 60), (1025, 5000), (16384, 60000), (16385, 60000),
+                                 (3000, 199900), (3000, 240000)])
+def test_one_block_order(L, n, m):
+    """h = 2 on both sides of the one-block limits: core numbers and the order
+    by (removal round, id)."""
+    if m:
+        n, s, d = gg.chung_lu(n, m, 2.3, 4.0 * n ** 0.5, n)
+    else:
+        s = d = np.zeros(0, np.uint32)
+    core, rnd = rounds_of(n, s, d)
+    rank = np.empty(n, np.int64)
+    rank[np.lexsort((np.arange(n), rnd))] = np.arange(n)
+    with L.Graph.from_edges(n, s, d) as g:
+        c2, rk, _ = g.degeneracy_order()
+    assert np.array_equal(c2, core)
+    assert np.array_equal(rk, rank)
