@@ -96,3 +96,36 @@ def test_one_block_order(L, n, m):
         c2, rk, _ = g.degeneracy_order()
     assert np.array_equal(c2, core)
     assert np.array_equal(rk, rank)
+
+
+@pytest.mark.parametrize("x", [2, 3, 5])
+@pytest.mark.parametrize("graph", ["ring", "power", "dense", "hub"])
+def test_star_bands(L, graph, x):
+    """The x-star peel in bands against the one-level peel (limit 0, itself
+    compared with the oracle in the pattern tests): a cascade around a ring
+    (undone), a power law, one dense block, and a hub whose counts may pass
+    2^62 (x = 5: C(40000, 5) > 2^62, not taken in bands)."""
+    if graph == "ring":
+        n, s, d = ring(20000, 3, 0.003, 2)
+    elif graph == "power":
+        n, s, d = gg.chung_lu(9001, 70000, 2.1, 700.0, 3)
+        s, d = np.concatenate([s, [0, 8999]]).astype(np.uint32), \
+            np.concatenate([d, [9000, 9000]]).astype(np.uint32)
+    elif graph == "dense":
+        n, s, d = gg.er(700, 0.2, 4)
+    else:
+        n, s, d = gg.er(40001, 0.00002, 5)
+        s = np.concatenate([s, np.zeros(40000, np.uint32)])
+        d = np.concatenate([d, np.arange(1, 40001, dtype=np.uint32)])
+    got = []
+    with L.Graph.from_edges(n, s, d) as g:
+        for limit in (0, 500, 1 << 30):
+            L.dsd_set_peel_tail_limit(limit)
+            try:
+                got.append(g.pattern_core_decompose(L.DSD_PATTERN_STAR, x))
+            finally:
+                L.dsd_set_peel_tail_limit(1 << 30)
+    for r in got[1:]:
+        assert r[1] == got[0][1]
+        for a, b in zip(r, got[0]):
+            assert np.array_equal(a, b)
