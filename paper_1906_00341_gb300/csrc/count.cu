@@ -107,10 +107,11 @@ __global__ void __launch_bounds__(kCountThreads) k_count_small(CountArgs A) {
 // Tier M: one block per vertex, |N+(u)| in (32, 1024].
 template <int NT>
 __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // 1024
     uint32_t* C = smem + 2 * kBitmapMax;      // 1024
-    uint32_t* rows = smem + 3 * kBitmapMax;   // up to 1024*32 (only if r >= 3)
+    uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);   // only if r >= 3, as the scratch
+    uint32_t* scratch = rows + kBitmapMax * kRowStrideMax;
     __shared__ unsigned long long s_tot;
     __shared__ uint32_t s_next, s_it;
     uint32_t nM = A.cntML[0];
@@ -127,7 +128,7 @@ __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
         uint32_t W = (d + 31) >> 5;
         for (uint32_t i = threadIdx.x; i < d; i += blockDim.x) { C[i] = A.adj[b + i]; cnt[i] = 0; }
         if (A.r >= 3)
-            for (uint32_t i = threadIdx.x; i < d * W; i += blockDim.x) rows[i] = 0;
+            for (uint32_t i = threadIdx.x; i < d * row_stride(W); i += blockDim.x) rows[i] = 0;
         if (threadIdx.x == 0) {
             s_tot = 0;
             s_next = 0;
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
         } else {
             block_build_rows(C, d, W, A.off + 1, A.adj, A.split, rows);
             __syncthreads();
-            mine = block_dfs(rows, d, W, A.r, cnt, &s_next);
+            mine = block_dfs(rows, d, W, A.r, cnt, &s_next, scratch);
         }
         if (mine) atomicAdd(&s_tot, mine);
         __syncthreads();
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count_large3(CountArgs A) {
 // set is split by its next member until it fits the bitmap tier (xl.cuh).
 // scratch: kMaxDepth * cap entries per block.
 __global__ void __launch_bounds__(1024) k_count_xl(CountArgs A, uint32_t* scratch, uint32_t cap) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_root;
     __shared__ uint32_t s_it;
     uint32_t* mine = scratch + (size_t)blockIdx.x * kMaxDepth * cap;
@@ -366,7 +367,7 @@ dsd_status count_cliques(dsd_graph* g, int h, unsigned long long* deg_new,
                 A.listM = sorted;
             }
         }
-        size_t smemM = (size_t)3 * kBitmapMax * 4 + (h >= 4 ? (size_t)kBitmapMax * 32 * 4 : 0);
+        size_t smemM = h >= 4 ? (size_t)bitmap_words(kBitmapMax, 32) * 4 : (size_t)3 * kBitmapMax * 4;
         if (h >= 4) {
             // one block per SM (the rows fill its shared memory): 32 warps
             cudaFuncSetAttribute(k_count_medium<1024>,

@@ -583,7 +583,8 @@ __device__ void process_big(const PeelParams& P, const NPlus& R, uint32_t v, uin
                             uint32_t* smem, const uint32_t* gbm, unsigned long long& bytes) {
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // bcap
     uint32_t* C = smem + 2 * P.bcap;                                          // bcap
-    uint32_t* rows = C + P.bcap;                                              // bcap * W
+    uint32_t* rows = smem + bitmap_rows_at(P.bcap);                           // bcap rows
+    uint32_t* scratch = rows + P.bcap * row_stride((P.bcap + 31) >> 5);
     __shared__ uint32_t s_nc;
     __shared__ uint32_t s_next;
     __shared__ unsigned long long s_tot;
@@ -707,11 +708,11 @@ bitmap:
         cnt[i] = 0;
         bytes += 16 + 4ull * (R.ne[C[i]] - R.nb[C[i]]);
     }
-    for (uint32_t i = threadIdx.x; i < nc * W; i += blockDim.x) rows[i] = 0;
+    for (uint32_t i = threadIdx.x; i < nc * row_stride(W); i += blockDim.x) rows[i] = 0;
     __syncthreads();
     block_build_rows(C, nc, W, R.ne, R.adj, R.nb, rows);
     __syncthreads();
-    unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next);
+    unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next, scratch);
     if (mine) atomicAdd(&s_tot, mine);
     __syncthreads();
     unsigned long long tot = s_tot;
@@ -1146,7 +1147,7 @@ __device__ __forceinline__ void process_queued(const PeelParams& P, const NPlus&
 template <int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
     constexpr int NW = NT / 32;
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_pre[kSmallFront + 1];
     __shared__ unsigned long long s_red[NW];
     __shared__ uint32_t s_hist[kBins];
@@ -1704,7 +1705,7 @@ constexpr size_t peel2_block_smem(uint32_t n) { return (size_t)n * 12 + 16; }
 __global__ void __launch_bounds__(1024, 1) k_peel2_block(Peel2Block P) {
     constexpr int NT = 1024, NW = NT / 32;
     constexpr uint32_t kStay = 0xffffu;   // rounds stay below n <= kOneBlockN
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     uint32_t* deg = smem;                                  // [n]
     uint32_t* at = deg + P.n;                              // [n + 1] row starts
     uint16_t* stamp = (uint16_t*)(at + P.n + 1);           // [n]
@@ -1961,10 +1962,8 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
         P.hub_min = 4 * P.heavy_min;
     }
     if (big_items) {
-        size_t W = (P.bcap + 31) / 32;
-        size_t big = (size_t)3 * P.bcap + (size_t)P.bcap * W;
-        // the split search of oversized sets uses the full bitmap tier layout
-        if (P.cap > kBitmapMax) big = (size_t)3 * kBitmapMax + (size_t)kBitmapMax * 32;
+        // (cap > kBitmapMax: the split search uses the full-size layout)
+        size_t big = bitmap_words(P.bcap, NT / 32);
         if (big > work) work = big;
     }
     const size_t smem = work * 4;

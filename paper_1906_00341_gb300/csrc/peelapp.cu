@@ -237,7 +237,8 @@ __device__ void app_big(const AppParams& P, const AppQ& Q, uint32_t v, uint32_t 
                         unsigned long long k, uint32_t* smem) {
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);   // bcap
     uint32_t* C = smem + 2 * P.bcap;                                           // bcap
-    uint32_t* rows = C + P.bcap;                                               // bcap * W
+    uint32_t* rows = smem + bitmap_rows_at(P.bcap);                            // bcap rows
+    uint32_t* scratch = rows + P.bcap * row_stride((P.bcap + 31) >> 5);
     __shared__ uint32_t s_nc, s_next, s_w[32], s_t2;
     __shared__ unsigned long long s_tot;
     const uint64_t wb = P.split[w], we = P.off[w + 1];
@@ -285,11 +286,11 @@ __device__ void app_big(const AppParams& P, const AppQ& Q, uint32_t v, uint32_t 
     }
     const uint32_t nc = s_nc, W = (nc + 31) >> 5;
     for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) cnt[i] = 0;
-    for (uint32_t i = threadIdx.x; i < nc * W; i += blockDim.x) rows[i] = 0;
+    for (uint32_t i = threadIdx.x; i < nc * row_stride(W); i += blockDim.x) rows[i] = 0;
     __syncthreads();
     block_build_rows(C, nc, W, P.off + 1, P.adj, P.split, rows);
     __syncthreads();
-    unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next);
+    unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next, scratch);
     if (mine) atomicAdd(&s_tot, mine);
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) lower(P, Q, C[i], k, cnt[i]);
@@ -360,7 +361,7 @@ constexpr uint32_t kPickDone = 0xfffffffeu;   // every member removed
 template <int NT>
 __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
     constexpr int NW = NT / 32;
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     __shared__ unsigned long long s_kd[NW];
     __shared__ uint32_t s_kp[NW];
     __shared__ uint32_t s_lv, s_pick, s_nbig, s_it;
@@ -771,10 +772,8 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
         P.best = best;
         size_t words = (size_t)(kAppNT / 32) * 3 * kAppWarpCand;
         if (h >= 4) {
-            size_t W = (P.bcap + 31) / 32;
-            size_t big = (size_t)3 * P.bcap + (size_t)P.bcap * W;
-            // the split search of oversized sets uses the full bitmap tier layout
-            if (P.cap > kBitmapMax) big = (size_t)3 * kBitmapMax + (size_t)kBitmapMax * 32;
+            // (cap > kBitmapMax: the split search uses the full-size layout)
+            size_t big = bitmap_words(P.bcap, kAppNT / 32);
             if (big > words) words = big;
         }
         // bucket queues: in shared memory after the scratch where they fit

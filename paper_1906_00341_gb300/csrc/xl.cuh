@@ -67,8 +67,7 @@ struct XLLevel {
     uint32_t z;       // member chosen to open this level (not for level 0)
 };
 
-// smem: kBitmapMax u64 counters, kBitmapMax candidates, kBitmapMax * 32 row
-// words (the bitmap tier's buffers).  scratch: kMaxDepth * cap entries.
+// smem: the bitmap tier's buffers, bitmap_words(kBitmapMax, warps) words.  scratch: kMaxDepth * cap entries.
 template <class Cand, class Root>
 __device__ void xl_cliques(const uint32_t* C0, uint32_t n0, int rr0, const uint64_t* nb,
                            const uint64_t* ne, const uint32_t* adj, uint32_t* scratch,
@@ -80,7 +79,8 @@ __device__ void xl_cliques(const uint32_t* C0, uint32_t n0, int rr0, const uint6
     const unsigned lane = lane_id(), wid = warp_id(), nw = blockDim.x >> 5;
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);   // kBitmapMax
     uint32_t* Cs = smem + 2 * kBitmapMax;                                    // kBitmapMax
-    uint32_t* rows = Cs + kBitmapMax;                                        // kBitmapMax * 32
+    uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);
+    uint32_t* wscratch = rows + kBitmapMax * kRowStrideMax;
     if (threadIdx.x == 0) {
         s_lv[0] = XLLevel{C0, n0, rr0, 0u, 0u};
         s_t = 0;
@@ -133,12 +133,12 @@ __device__ void xl_cliques(const uint32_t* C0, uint32_t n0, int rr0, const uint6
                     Cs[i] = L.C[i];
                     cnt[i] = 0;
                 }
-                for (uint32_t i = threadIdx.x; i < n * W; i += blockDim.x) rows[i] = 0;
+                for (uint32_t i = threadIdx.x; i < n * row_stride(W); i += blockDim.x) rows[i] = 0;
                 if (threadIdx.x == 0) s_next = 0;
                 __syncthreads();
                 block_build_rows(Cs, n, W, ne, adj, nb, rows);
                 __syncthreads();
-                mine = block_dfs(rows, n, W, L.rr, cnt, &s_next);
+                mine = block_dfs(rows, n, W, L.rr, cnt, &s_next, wscratch);
                 __syncthreads();
                 for (uint32_t i = threadIdx.x; i < n; i += blockDim.x)
                     if (cnt[i]) cand(Cs[i], cnt[i]);

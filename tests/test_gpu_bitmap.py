@@ -1,0 +1,50 @@
+"""The block-level bitmap search at the sizes where its layout changes: word
+and stride boundaries, node sets above the list buffer, 32- and 64-bit
+counters.  Closed forms on K_n and the oracle on random graphs."""
+from __future__ import annotations
+
+import math
+
+import numpy as np
+import pytest
+
+from paper_1906_00341_gb300 import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1906_00341_gb300 import build as b
+    b.build()
+    from paper_1906_00341_gb300 import _lib
+    _lib.load()
+    return _lib
+
+
+@pytest.mark.parametrize("n,hs", [(34, (4, 5, 8)), (66, (4, 5, 6)), (130, (4, 5, 6)),
+                                  (258, (4, 5)), (300, (4, 5)), (1024, (4,)), (1025, (4,))])
+def test_complete_graphs(L, n, hs):
+    s, d = np.triu_indices(n, 1)
+    with L.Graph.from_edges(n, s.astype(np.uint32), d.astype(np.uint32)) as g:
+        for h in hs:
+            deg, mu = g.clique_degrees(h)
+            assert mu == math.comb(n, h)
+            assert np.all(deg == math.comb(n - 1, h - 1))
+
+
+@pytest.mark.parametrize("n,p,h", [(97, 0.6, 7), (200, 0.5, 6), (330, 0.4, 5), (520, 0.3, 4),
+                                   (700, 0.15, 4)])
+def test_random_dense(L, orc, n, p, h):
+    n, s, d = gg.er(n, p, seed=n + h)
+    og = orc.csr(n, s, d)
+    wdeg, wmu = orc.clique_degrees(og, h)
+    with L.Graph.from_edges(n, s, d) as g:
+        deg, mu = g.clique_degrees(h)
+        core, k = g.core_decompose(h) if n <= 330 and h <= 5 else (None, None)
+    assert mu == wmu and np.array_equal(deg, wdeg)
+    if core is not None:
+        wcore, wk = orc.core_decompose(og, h)
+        assert k == wk and np.array_equal(core, wcore)
