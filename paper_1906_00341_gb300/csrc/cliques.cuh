@@ -269,29 +269,97 @@ __host__ __device__ constexpr uint32_t row_stride(uint32_t W) {
     return ((W + 3u) / 4u | 1u) * 4u;
 }
 constexpr uint32_t kRowStrideMax = row_stride(kBitmapMax / 32);   // 36
+constexpr uint32_t kWindow = 8192;                                 // see block_window
+constexpr uint32_t kWindowWords = kWindow / 2;
 // A warp's scratch: its node's words and the positions of its set bits.
 constexpr uint32_t kLeafList = 256;
 constexpr uint32_t kWarpScratch = kRowStrideMax + kLeafList / 2;  // words
 // Shared words of a bitmap problem of at most bcap candidates (64-bit
-// counters, candidates, rows, scratch of nw warps); the rows start at word
-// bitmap_rows_at(bcap).
+// counters, candidates, rows, window, scratch of nw warps); the rows start at
+// word bitmap_rows_at(bcap), the scratch at bitmap_scratch_at(bcap) and the
+// window before it.
 __host__ __device__ constexpr uint32_t bitmap_rows_at(uint32_t bcap) {
     return (3u * bcap + 3u) & ~3u;
 }
 __host__ __device__ constexpr uint32_t bitmap_words(uint32_t bcap, uint32_t nw) {
-    return bitmap_rows_at(bcap) + bcap * row_stride((bcap + 31u) / 32u) + nw * kWarpScratch;
+    return bitmap_rows_at(bcap) + bcap * row_stride((bcap + 31u) / 32u) + kWindowWords +
+           nw * kWarpScratch;
+}
+__host__ __device__ constexpr uint32_t bitmap_scratch_at(uint32_t bcap) {
+    return bitmap_rows_at(bcap) + bcap * row_stride((bcap + 31u) / 32u) + kWindowWords;
 }
 
-// rows: nc * row_stride(W) words, zeroed by the caller.
+// Positions in C by id for the kWindow largest ids (16-bit, in shared memory):
+// candidates crowd at the high ranks, and there a look-up replaces the ten
+// dependent shared loads of a binary search.
+__device__ __forceinline__ uint32_t window_base(uint32_t cmax) {
+    return cmax >= kWindow ? cmax - (kWindow - 1u) : 0u;
+}
+// Every thread of the block calls it; the caller synchronises after it.  It
+// clears the table, synchronises and enters C (win: 16-byte aligned).
+__device__ __forceinline__ void block_window(const uint32_t* C, uint32_t nc, uint32_t* win) {
+    for (uint32_t i = threadIdx.x; i < kWindowWords / 4; i += blockDim.x)
+        reinterpret_cast<uint4*>(win)[i] = make_uint4(kNone, kNone, kNone, kNone);
+    __syncthreads();
+    if (nc == 0) return;
+    const uint32_t w0 = window_base(C[nc - 1]);
+    for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x)
+        if (C[i] >= w0) reinterpret_cast<uint16_t*>(win)[C[i] - w0] = (uint16_t)i;
+}
+// The position of y <= cmax in C, or kNone.
+__device__ __forceinline__ uint32_t find_pos(const uint32_t* C, uint32_t nc, const uint32_t* win,
+                                             uint32_t w0, uint32_t y) {
+    if (y >= w0) {
+        const uint32_t p = reinterpret_cast<const uint16_t*>(win)[y - w0];
+        return p == 0xffffu ? kNone : p;
+    }
+    const uint32_t p = (uint32_t)lower_bound_u32(C, nc, y);
+    return p < nc && C[p] == y ? p : kNone;
+}
+
+// Hits of adj[b, e) in C as scan_row_hits, found through the window: cnt[2 pos]
+// += 1 (the low words of 64-bit counters).
+__device__ __forceinline__ unsigned scan_row_window(const uint32_t* C, uint32_t nc, uint32_t cmax,
+                                                    const uint32_t* win, uint32_t w0,
+                                                    const uint32_t* adj, uint64_t b, uint64_t e,
+                                                    unsigned* cnt) {
+    const unsigned lane = lane_id();
+    unsigned hits = 0;
+    for (uint64_t p0 = b; p0 < e; p0 += 32 * kScanChunks) {
+        uint32_t ys[kScanChunks];
+#pragma unroll
+        for (int u = 0; u < kScanChunks; u++) {
+            uint64_t p = p0 + u * 32 + lane;
+            ys[u] = p < e ? adj[p] : 0xffffffffu;
+        }
+#pragma unroll
+        for (int u = 0; u < kScanChunks; u++) {
+            if (ys[u] <= cmax) {
+                const uint32_t pos = find_pos(C, nc, win, w0, ys[u]);
+                if (pos != kNone) {
+                    atomicAdd(&cnt[2 * pos], 1u);
+                    hits++;
+                }
+            }
+        }
+        if (__shfl_sync(0xffffffffu, ys[kScanChunks - 1], 31) > cmax) break;
+    }
+    return hits;
+}
+
+// rows: nc * row_stride(W) words, zeroed by the caller; win: C's window
+// (block_window).  num (may be null): the row number of each candidate.
 template <class OFF>
 __device__ __forceinline__ void block_build_rows(const uint32_t* C, uint32_t nc, uint32_t W,
                                                  const OFF* ne, const uint32_t* adj,
-                                                 const OFF* nb, uint32_t* rows) {
+                                                 const OFF* nb, uint32_t* rows,
+                                                 const uint32_t* win,
+                                                 const uint16_t* num = nullptr) {
     const unsigned lane = lane_id();
     const unsigned nw = blockDim.x >> 5;
     if (nc == 0) return;
     const uint32_t Ws = row_stride(W);
-    const uint32_t cmax = C[nc - 1];
+    const uint32_t cmax = C[nc - 1], w0 = window_base(cmax);
     for (uint32_t i = warp_id(); i + 1 < nc; i += nw) {
         const uint32_t x = C[i];
         const uint64_t b = nb[x], e = ne[x];
@@ -306,10 +374,11 @@ __device__ __forceinline__ void block_build_rows(const uint32_t* C, uint32_t nc,
             for (int u = 0; u < kScanChunks; u++) {
                 const uint32_t y = ys[u];
                 if (y > x && y <= cmax) {
-                    uint32_t pos = (uint32_t)lower_bound_u32(C, nc, y);
-                    if (pos < nc && C[pos] == y && pos > i) {
-                        atomicOr(&rows[i * Ws + (pos >> 5)], 1u << (pos & 31));
-                        atomicOr(&rows[pos * Ws + (i >> 5)], 1u << (i & 31));
+                    const uint32_t pos = find_pos(C, nc, win, w0, y);
+                    if (pos != kNone) {
+                        const uint32_t a = num ? num[i] : i, c = num ? num[pos] : pos;
+                        atomicOr(&rows[a * Ws + (c >> 5)], 1u << (c & 31));
+                        atomicOr(&rows[c * Ws + (a >> 5)], 1u << (a & 31));
                     }
                 }
             }
@@ -328,7 +397,9 @@ struct BitmapWarp {
     uint32_t* sP;          // [Ws]
     uint16_t* list;        // [kLeafList]
     bool small;
+    uint32_t nd;           // only candidates below nd are credited
     __device__ __forceinline__ void credit(uint32_t j, unsigned long long v) const {
+        if (j >= nd) return;
         if (small) atomicAdd(reinterpret_cast<unsigned*>(cnt + j), (unsigned)v);
         else atomicAdd(cnt + j, v);
     }
@@ -338,9 +409,8 @@ struct BitmapWarp {
     }
 };
 
-// Edges of G[P] (this lane's word of P given; all lanes get the result);
-// CREDIT: each end gets its degree.
-template <bool CREDIT>
+// Edges of G[P] (this lane's word of P given; all lanes get the result); each
+// end is credited with its degree.
 __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, uint32_t Pw) {
     const unsigned full = 0xffffffffu, lane = lane_id();
     const unsigned nz = __ballot_sync(full, Pw != 0);
@@ -377,7 +447,7 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
                 s += __popc(a.x & p.x) + __popc(a.y & p.y);
                 s += __popc(a.z & p.z) + __popc(a.w & p.w);
             }
-            if (CREDIT && s) B.credit(j, s);
+            if (s) B.credit(j, s);
             sum += s;
         }
         __syncwarp();
@@ -385,11 +455,11 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
     return __reduce_add_sync(full, sum) >> 1;   // sum <= 1024 * 1023
 }
 
-// RR-cliques of G[P], RR >= 2; CREDIT: each member gets the cliques it is in.
-template <int RR, bool CREDIT>
+// RR-cliques of G[P], RR >= 2; each member is credited with those it is in.
+template <int RR>
 __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
     if constexpr (RR == 2) {
-        return warp_edges<CREDIT>(B, Pw);
+        return warp_edges(B, Pw);
     } else {
         const unsigned full = 0xffffffffu, lane = lane_id();
         unsigned long long acc = 0;
@@ -405,13 +475,13 @@ __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
             const uint32_t pn = rem & B.row_word(j);
             unsigned long long sub;
             if constexpr (RR == 3) {
-                sub = warp_edges<CREDIT>(B, pn);
+                sub = warp_edges(B, pn);
             } else {
                 if (__reduce_add_sync(full, (unsigned)__popc(pn)) < RR - 1) continue;
-                sub = warp_cliques<RR - 1, CREDIT>(B, pn);
+                sub = warp_cliques<RR - 1>(B, pn);
             }
             if (sub) {
-                if (CREDIT && lane == 0) B.credit(j, sub);
+                if (lane == 0) B.credit(j, sub);
                 acc += sub;
             }
         }
@@ -419,20 +489,20 @@ __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
     }
 }
 
-template <bool CREDIT>
 __device__ __forceinline__ unsigned long long warp_cliques_of(const BitmapWarp& B, uint32_t Pw,
                                                              int rr) {
     switch (rr) {
-        case 2: return warp_cliques<2, CREDIT>(B, Pw);
-        case 3: return warp_cliques<3, CREDIT>(B, Pw);
-        case 4: return warp_cliques<4, CREDIT>(B, Pw);
-        case 5: return warp_cliques<5, CREDIT>(B, Pw);
-        default: return warp_cliques<6, CREDIT>(B, Pw);   // r <= DSD_MAX_H - 1 = 7
+        case 2: return warp_cliques<2>(B, Pw);
+        case 3: return warp_cliques<3>(B, Pw);
+        case 4: return warp_cliques<4>(B, Pw);
+        case 5: return warp_cliques<5>(B, Pw);
+        default: return warp_cliques<6>(B, Pw);   // r <= DSD_MAX_H - 1 = 7
     }
 }
 
 __device__ __forceinline__ BitmapWarp bitmap_warp(const uint32_t* rows, uint32_t W, int r,
-                                                  unsigned long long* cnt, uint32_t* scratch) {
+                                                  unsigned long long* cnt, uint32_t* scratch,
+                                                  uint32_t nd) {
     BitmapWarp B;
     B.rows = rows;
     B.W = W;
@@ -441,6 +511,7 @@ __device__ __forceinline__ BitmapWarp bitmap_warp(const uint32_t* rows, uint32_t
     B.sP = scratch + warp_id() * kWarpScratch;
     B.list = reinterpret_cast<uint16_t*>(B.sP + kRowStrideMax);
     B.small = r <= 4;
+    B.nd = nd;
     // words past the lanes' 32 (a full-width stride) stay zero
     if (lane_id() < kRowStrideMax - 32) B.sP[32 + lane_id()] = 0;
     __syncwarp();
@@ -450,12 +521,15 @@ __device__ __forceinline__ BitmapWarp bitmap_warp(const uint32_t* rows, uint32_t
 // r-cliques of G[C], r >= 2, with every member's count added to cnt (zeroed
 // by the caller).  Warps take first members i from the shared counter *next_i
 // (zero on entry; the early candidates, with the largest searches above them,
-// go first).  scratch: kWarpScratch words a warp, 16-byte aligned.  Returns
-// this thread's share of the total (sum over the block = total).
+// go first); r >= 3: only those of start, start + step, ... below nd, and
+// only candidates below nd are credited.  scratch: kWarpScratch words a warp, 16-byte aligned.  Returns this
+// thread's share of the total (sum over the block = total).
 __device__ __forceinline__ unsigned long long block_dfs(const uint32_t* rows, uint32_t nc,
                                                        uint32_t W, int r,
                                                        unsigned long long* cnt,
-                                                       uint32_t* next_i, uint32_t* scratch) {
+                                                       uint32_t* next_i, uint32_t* scratch,
+                                                       uint32_t start = 0, uint32_t step = 1,
+                                                       uint32_t nd = kNone) {
     const unsigned full = 0xffffffffu, lane = lane_id();
     unsigned long long total = 0;
     if (r == 2) {
@@ -474,18 +548,19 @@ __device__ __forceinline__ unsigned long long block_dfs(const uint32_t* rows, ui
         }
         return total;
     }
-    const BitmapWarp B = bitmap_warp(rows, W, r, cnt, scratch);
+    if (nd > nc) nd = nc;
+    const BitmapWarp B = bitmap_warp(rows, W, r, cnt, scratch, nd);
     for (;;) {
         uint32_t i = 0;
         if (lane == 0) i = atomicAdd(next_i, 1u);
-        i = __shfl_sync(full, i, 0);
-        if (i >= nc) break;
+        i = start + step * __shfl_sync(full, i, 0);
+        if (i >= nd) break;
         uint32_t P = B.row_word(i);
         const uint32_t iw = i >> 5;
         if (lane < iw) P = 0;
         else if (lane == iw) P &= (i & 31u) == 31u ? 0u : 0xffffffffu << ((i & 31u) + 1u);
         if ((int)__reduce_add_sync(full, (unsigned)__popc(P)) < r - 1) continue;
-        const unsigned long long c = warp_cliques_of<true>(B, P, r - 1);
+        const unsigned long long c = warp_cliques_of(B, P, r - 1);
         if (c) {
             if (lane == 0) B.credit(i, c);
             total += c;

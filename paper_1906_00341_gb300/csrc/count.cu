@@ -111,7 +111,8 @@ __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // 1024
     uint32_t* C = smem + 2 * kBitmapMax;      // 1024
     uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);   // only if r >= 3, as the scratch
-    uint32_t* scratch = rows + kBitmapMax * kRowStrideMax;
+    uint32_t* scratch = smem + bitmap_scratch_at(kBitmapMax);
+    uint32_t* win = A.r >= 3 ? scratch - kWindowWords : smem + 3 * kBitmapMax;
     __shared__ unsigned long long s_tot;
     __shared__ uint32_t s_next, s_it;
     uint32_t nM = A.cntML[0];
@@ -134,19 +135,23 @@ __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
             s_next = 0;
         }
         __syncthreads();
+        block_window(C, d, win);
+        __syncthreads();
         unsigned long long mine = 0;
         if (A.r == 2) {
             unsigned lane = lane_id(), nw = blockDim.x >> 5;
-            const uint32_t cmax = C[d - 1];
+            const uint32_t cmax = C[d - 1], w0 = window_base(cmax);
+            unsigned* cnt32 = reinterpret_cast<unsigned*>(cnt);   // low words: counts < 2^20
             for (uint32_t i = warp_id(); i + 1 < d; i += nw) {
                 uint32_t x = C[i];
-                unsigned hits = scan_row_hits(C, d, cmax, A.adj, A.split[x], A.off[x + 1], cnt);
+                unsigned hits = scan_row_window(C, d, cmax, win, w0, A.adj, A.split[x],
+                                                A.off[x + 1], cnt32);
                 hits = __reduce_add_sync(0xffffffffu, hits);
-                if (lane == 0 && hits) atomicAdd(&cnt[i], (unsigned long long)hits);
+                if (lane == 0 && hits) atomicAdd(&cnt32[2 * i], hits);
                 if (lane == 0) mine += hits;
             }
         } else {
-            block_build_rows(C, d, W, A.off + 1, A.adj, A.split, rows);
+            block_build_rows(C, d, W, A.off + 1, A.adj, A.split, rows, win);
             __syncthreads();
             mine = block_dfs(rows, d, W, A.r, cnt, &s_next, scratch);
         }
@@ -367,7 +372,8 @@ dsd_status count_cliques(dsd_graph* g, int h, unsigned long long* deg_new,
                 A.listM = sorted;
             }
         }
-        size_t smemM = h >= 4 ? (size_t)bitmap_words(kBitmapMax, 32) * 4 : (size_t)3 * kBitmapMax * 4;
+        size_t smemM = h >= 4 ? (size_t)bitmap_words(kBitmapMax, 32) * 4
+                             : (size_t)(3 * kBitmapMax + kWindowWords) * 4;
         if (h >= 4) {
             // one block per SM (the rows fill its shared memory): 32 warps
             cudaFuncSetAttribute(k_count_medium<1024>,

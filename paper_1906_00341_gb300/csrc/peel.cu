@@ -73,7 +73,7 @@
 namespace dsd {
 namespace {
 
-// state word: bits 0-1 the state, bit 2 kHeavyBit, bits 3-10 a bitmap slot
+// state word: bits 0-1 the state, bit 2 kListedBit, bits 3-10 a bitmap slot
 // (phase 1 only), bits 11-31 the band key (zero throughout phase 1)
 enum : uint32_t { kAlive = 0, kFront = 1, kGone = 2 };
 enum : uint32_t { kErrTimeout = 1, kErrBigOverflow = 2 };
@@ -81,6 +81,20 @@ constexpr uint32_t kSmallFront = 1024;
 constexpr int kChunks = 4;              // 32-entry chunks of a row in flight per warp
 constexpr uint32_t kWarpCand = 32;      // candidate sets a warp handles itself (h >= 4)
 constexpr uint32_t kWarpWords = 3 * kWarpCand;   // a warp's candidates, counters, rows
+// h = 4: a frontier vertex whose row holds at most kTinyRow entries goes to a
+// warp, one of up to kBitmapMax to a block (or a few), which list the cliques
+// of its whole neighbourhood at once; longer rows are taken one (vertex,
+// neighbour) item at a time.
+constexpr uint32_t kTinyRow = 32;
+constexpr uint32_t kMaxSlices = 8;      // blocks sharing one such vertex
+// Other h: the items of all frontier vertices are spread over the grid.  At h
+// = 3 an item is one row walk (1M-vertex graph: 14 ms of phase 1 against 41 ms
+// with a group of warps a vertex); at h = 5 the search inside an item has the
+// short rows of a common neighbourhood (R-MAT scale 15: peel 22 ms against 28
+// with whole rows).  In frontiers above kSmallFront only rows above kLongRow
+// are spread, and those above kHubRow get bitmaps.
+constexpr uint32_t kLongRow = 128;
+constexpr uint32_t kHubRow = 512;
 constexpr uint32_t kMidWords = 3 + kWarpCand;    // a mid item: v, w, |C|, C
 constexpr int kGroupWarps = 8;                    // warps of a group taking one mid item
 // h >= 4: a warp lists the cliques of a candidate set of at most this many
@@ -93,7 +107,7 @@ inline uint32_t warp_cand_limit(int h) {
     uint32_t w = peel_item_warp_limit();
     return h >= 4 ? (w < kWarpCand ? w : kWarpCand) : kWarpCand;
 }
-constexpr uint32_t kHeavyBit = 4;       // state word: frontier vertex on the heavy list
+constexpr uint32_t kListedBit = 4;      // state word: frontier vertex on the row or heavy list
 constexpr uint32_t kSlotShift = 3;      // state word: 1 + its neighbourhood bitmap slot
 constexpr uint32_t kSlotMask = 0xffu;
 constexpr uint32_t kKeyShift = 11;      // state word: band key
@@ -131,13 +145,15 @@ struct PeelCtrl {
     uint32_t new_alive[2];
     uint32_t fcnt[3];
     uint32_t big_cnt[6];            // per round slot s: big items [s], mid items [3 + s]
-    uint32_t hcnt[3];               // heavy frontier vertices of the round
-    uint32_t grab[3];               // light frontier vertices taken by blocks
+    uint32_t hcnt[3];               // frontier vertices whose items are spread,
+    uint32_t vcnt[3];               //   and whose rows are taken whole
+    uint32_t vgrab[3];              // those (phase 2: frontier vertices) taken
+    uint32_t grab[3];               // frontier vertices taken by warps
     uint32_t bgrab[6];              // big items [s] and mid items [3 + s] taken
     uint32_t hubcnt[2];             // bitmap slots asked for, by round parity
     uint32_t busy[3];               // phase 2: bands with vertices left, by round
     unsigned long long destroyed;   // phase 1: cliques destroyed so far
-    uint32_t pad0[16];
+    uint32_t pad0[10];
     uint32_t bar_count;
     uint32_t pad1[31];
     uint32_t bar_gen;
@@ -196,18 +212,16 @@ struct PeelParams {
     uint32_t band_max;     // group levels into bands at <= this many alive (0 = never)
     uint2* big;
     uint64_t big_cap;
-    uint32_t* heavy;       // large regime: frontier vertices with long rows
-    uint32_t heavy_min;    // rows longer than this are heavy (0 = no heavy list)
-    // Large regime: frontier vertices with rows longer than hub_min get (up
-    // to hub_slots per round) a bitmap of their neighbourhood over vertex
-    // ids, so that "x in N(v)" is one probe instead of a binary search.  Two
+    uint32_t* heavy;       // phase 1, h >= 3: frontier vertices whose items are spread
+    uint32_t* vlist;       //   (h = 4) or whose rows blocks take whole
+    // Phase 1: frontier vertices with the longest rows get (up to hub_slots
+    // per round) a bitmap of their neighbourhood over vertex ids, so that "x in N(v)" is one probe instead of a binary search.  Two
     // sets of hub_slots bitmaps of hub_words words, by round parity; hubs
     // lists the owners (2 x hub_slots).
     uint32_t* hub_bm;
     uint32_t* hubs;
     uint64_t hub_words;
     uint32_t hub_slots;    // 0 = no bitmaps
-    uint32_t hub_min;
     uint64_t* lvl_k;
     uint32_t* lvl_size;
     uint64_t* lvl_mu;
@@ -216,7 +230,6 @@ struct PeelParams {
     unsigned long long mu0;
     unsigned long long k0; // initial level: kstart - 1, or 0
     uint32_t cap;          // candidate sets are at most this (>= max |N+|, >= 32)
-    uint32_t bcap;         // a big item's shared buffers: min(cap, kBitmapMax)
     uint32_t warp_cand;    // h >= 4: candidate sets a warp handles (<= kWarpCand); larger
                            // ones go to a warp group (mid items) or a block
     uint32_t gather_cap;   // a warp's candidate walk stops past this many
@@ -288,11 +301,11 @@ __device__ __forceinline__ void lower(const PeelParams& P, uint32_t x, uint32_t 
 }
 
 // ALL: every entry counts; else a frontier vertex marked gone (count 0) has
-// no items.
+// no items.  Rows of at most `skip` entries count as empty.
 template <int NT, bool ALL = false>
 __device__ __forceinline__ void block_prefix_degrees(const PeelParams& P, const uint32_t* F,
                                                      uint32_t f, unsigned long long* pre,
-                                                     unsigned long long* red) {
+                                                     unsigned long long* red, uint32_t skip = 0) {
     constexpr int E = kSmallFront / NT;
     unsigned long long d[E], sum = 0;
     uint32_t i0 = threadIdx.x * E;
@@ -303,6 +316,7 @@ __device__ __forceinline__ void block_prefix_degrees(const PeelParams& P, const 
         if (i < f) {
             uint32_t v = F[i];
             if (ALL || st_of(P.sl[v]) == kFront) d[q] = P.wend[v] - P.off[v];
+            if (d[q] <= skip) d[q] = 0;
         }
         sum += d[q];
     }
@@ -426,6 +440,7 @@ __device__ __forceinline__ uint32_t gather_candidates(const PeelParams& P, const
 // warp's kWarpCand-entry buffers.  Candidate sets above P.warp_cand (h >= 4)
 // are queued, as mid items with their candidates when at most kWarpCand
 // (`big_cnt + 3` counts them), else as big items for a block.
+template <int HC>
 __device__ void process_vw(const PeelParams& P, const NPlus& R, uint32_t v, uint32_t w,
                            unsigned long long k, uint32_t* next, uint32_t* next_cnt, uint32_t* C,
                            unsigned* cnt, uint32_t* rows, uint32_t* big_cnt, const uint32_t* gbm,
@@ -436,7 +451,7 @@ __device__ void process_vw(const PeelParams& P, const NPlus& R, uint32_t v, uint
     if (lane == 0) bytes += 4 + 4;   // w, its state word
     if (!cand_ok(ww, w, kv, v, dec_w)) return;
     if (lane == 0) bytes += 16;      // the bounds of N+(w)
-    const int r = P.h - 2;
+    const int r = HC == 3 ? 1 : P.h - 2;
     unsigned long long tot = 0;
     bool anyd = false;
     if (r == 1) {
@@ -581,10 +596,10 @@ __device__ __forceinline__ void process_pair(const PeelParams& P, uint32_t v, ui
 __device__ void process_big(const PeelParams& P, const NPlus& R, uint32_t v, uint32_t w,
                             unsigned long long k, uint32_t* next, uint32_t* next_cnt,
                             uint32_t* smem, const uint32_t* gbm, unsigned long long& bytes) {
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // bcap
-    uint32_t* C = smem + 2 * P.bcap;                                          // bcap
-    uint32_t* rows = smem + bitmap_rows_at(P.bcap);                           // bcap rows
-    uint32_t* scratch = rows + P.bcap * row_stride((P.bcap + 31) >> 5);
+    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);
+    uint32_t* C = smem + 2 * kBitmapMax;
+    uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);
+    uint32_t* scratch = smem + bitmap_scratch_at(kBitmapMax);
     __shared__ uint32_t s_nc;
     __shared__ uint32_t s_next;
     __shared__ unsigned long long s_tot;
@@ -710,7 +725,9 @@ bitmap:
     }
     for (uint32_t i = threadIdx.x; i < nc * row_stride(W); i += blockDim.x) rows[i] = 0;
     __syncthreads();
-    block_build_rows(C, nc, W, R.ne, R.adj, R.nb, rows);
+    block_window(C, nc, scratch - kWindowWords);
+    __syncthreads();
+    block_build_rows(C, nc, W, R.ne, R.adj, R.nb, rows, scratch - kWindowWords);
     __syncthreads();
     unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next, scratch);
     if (mine) atomicAdd(&s_tot, mine);
@@ -858,17 +875,21 @@ __device__ __forceinline__ const uint32_t* hub_bm_of(const PeelParams& P, uint32
 
 // Phase 1, marking v as a member of frontier F_r: its state word (gone at
 // once if it lies in no clique of the current set: nothing is enumerated
-// from it), with kHeavyBit for rows longer than heavy_min and, for rows longer than hub_min
-// while slots of this parity last, 1 + its bitmap slot (the owner goes to
-// the parity's hub list).
+// from it).  h >= 3: cls = 1 for rows that blocks take whole, 2 for rows whose
+// items are spread, both kListedBit; the longest of the latter get, while
+// slots of this parity last, 1 + a bitmap slot (the owner goes to the
+// parity's hub list).
+template <int HC>
 __device__ __forceinline__ uint32_t front_word(const PeelParams& P, PeelCtrl* c, uint32_t v,
-                                               uint32_t par, bool& hv) {
-    hv = false;
+                                               uint32_t par, uint32_t& cls) {
+    cls = 0;
     if (P.deg[v] == 0) return kGone;
-    uint64_t d = P.wend[v] - P.off[v];
-    hv = P.heavy_min && d > P.heavy_min;
-    uint32_t w = kFront | (hv ? kHeavyBit : 0u);
-    if (hv && P.hub_slots && d > P.hub_min) {
+    if (HC == 2) return kFront;
+    const uint64_t d = P.wend[v] - P.off[v];
+    if (HC != 4) cls = d > kLongRow ? 2u : 0u;
+    else cls = d > kBitmapMax ? 2u : (d > kTinyRow ? 1u : 0u);
+    uint32_t w = kFront | (cls ? kListedBit : 0u);
+    if (P.hub_slots && d > (HC == 4 ? kBitmapMax : kHubRow)) {
         uint32_t at = atomicAdd(&c->hubcnt[par], 1u);
         if (at < P.hub_slots) {
             P.hubs[par * P.hub_slots + at] = v;
@@ -907,23 +928,186 @@ __device__ __forceinline__ void hub_bitmaps(const PeelParams& P, uint32_t nhub, 
     __syncthreads();   // s_pre is reused afterwards
 }
 
+// Every clique through frontier vertex v of a short row (at most kTinyRow
+// entries), by one warp: the members of the current set among its neighbours
+// and the (h-1)-cliques they span; C, cnt, rows are the warp's buffers.
+template <int HC>
+__device__ void process_tiny(const PeelParams& P, const NPlus& R, uint32_t v,
+                             unsigned long long k, uint32_t* next, uint32_t* next_cnt,
+                             uint32_t* C, unsigned* cnt, uint32_t* rows,
+                             unsigned long long& bytes) {
+    const unsigned lane = lane_id();
+    const uint32_t kv = P.sl[v] >> kKeyShift;
+    const uint64_t b = P.off[v];
+    const uint32_t len = (uint32_t)(P.wend[v] - b);
+    const int r = HC == 3 ? 2 : P.h - 1;
+    uint32_t x = 0, wx = 0;
+    bool ok = false, dec = false;
+    if (lane < len) {
+        x = P.wadj[b + lane];
+        wx = P.sl[x];
+        ok = cand_ok(wx, x, kv, v, dec);
+        bytes += 8;
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, ok);
+    const uint32_t nc = __popc(bal), at = __popc(bal & ((1u << lane) - 1u));
+    if (nc < (uint32_t)r || !__any_sync(0xffffffffu, ok && dec)) return;
+    if (ok) C[at] = x;
+    cnt[lane] = 0;
+    __syncwarp();
+    if (lane < nc) bytes += 16 + 4ull * (R.ne[C[lane]] - R.nb[C[lane]]);
+    if (r == 2) {
+        const uint32_t cmax = C[nc - 1];
+        for (uint32_t i = 0; i + 1 < nc; i++) {
+            const uint32_t y = C[i];
+            unsigned hits = scan_row_hits(C, nc, cmax, R.adj, R.nb[y], R.ne[y], cnt);
+            hits = __reduce_add_sync(0xffffffffu, hits);
+            if (lane == 0 && hits) atomicAdd(&cnt[i], hits);
+        }
+    } else {
+        warp_build_rows32(C, nc, R.ne, R.adj, R.nb, rows);
+        (void)warp_dfs32(rows, nc, r, cnt);
+    }
+    __syncwarp();
+    if (ok && dec && cnt[at]) {
+        lower(P, x, st_of(wx), (unsigned long long)cnt[at], k, next, next_cnt);
+        bytes += 16;
+    }
+    __syncwarp();
+}
+
+// h = 4: the cliques through frontier vertex v (a row of at most kBitmapMax
+// entries), by a block: bitmap rows of its whole neighbourhood once, instead
+// of once for each (v, w) item, then the (h-1)-cliques in it.  Rows are
+// numbered with the nd neighbours that count these cliques first (phase 2:
+// those of v's band), and only they are first members, so that a clique whose
+// other members all lie in later bands is never listed.  Slice s of S: the
+// first members s, s + S, ... (several blocks share one vertex when there are
+// few).  smem: bitmap_words(kBitmapMax, warps) words and kBitmapMax 16-bit
+// row numbers.  R-MAT scale 17: peel 93 -> 22 ms.
+__device__ void process_row(const PeelParams& P, const NPlus& R, uint32_t v, uint32_t s,
+                            uint32_t S, unsigned long long k, uint32_t* next, uint32_t* next_cnt,
+                            uint32_t* smem, unsigned long long& bytes) {
+    __shared__ uint32_t s_flag[kBitmapMax / 32], s_dec[kBitmapMax / 32];
+    __shared__ uint32_t s_next;
+    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);
+    uint32_t* C = smem + 2 * kBitmapMax;
+    uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);
+    uint32_t* scratch = smem + bitmap_scratch_at(kBitmapMax);
+    const unsigned lane = lane_id(), nw = blockDim.x >> 5;
+    const uint32_t kv = P.sl[v] >> kKeyShift;
+    const uint64_t b = P.off[v];
+    const uint32_t len = (uint32_t)(P.wend[v] - b), runs = (len + 31) >> 5;
+    const int r = P.h - 1;
+    for (uint32_t c = warp_id(); c < runs; c += nw) {
+        const uint32_t p = c * 32 + lane;
+        bool ok = false, dec = false;
+        if (p < len) {
+            const uint32_t x = P.wadj[b + p];
+            ok = cand_ok(P.sl[x], x, kv, v, dec);
+            bytes += 8;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        const unsigned bad = __ballot_sync(0xffffffffu, ok && dec);
+        if (lane == 0) {
+            s_flag[c] = bal;
+            s_dec[c] = bad;
+        }
+    }
+    if (threadIdx.x == 0) s_next = 0;
+    __syncthreads();
+    const uint32_t f = lane < runs ? s_flag[lane] : 0u, g = lane < runs ? s_dec[lane] : 0u;
+    uint32_t inc = __popc(f), dinc = __popc(g);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        uint32_t z = __shfl_up_sync(0xffffffffu, dinc, o);
+        if ((int)lane >= o) {
+            inc += y;
+            dinc += z;
+        }
+    }
+    const uint32_t ex = inc - __popc(f), nc = __shfl_sync(0xffffffffu, inc, 31);
+    const uint32_t dex = dinc - __popc(g), nd = __shfl_sync(0xffffffffu, dinc, 31);
+    if (nc < (uint32_t)r || nd == 0) {
+        __syncthreads();   // s_flag is rewritten by the next vertex
+        return;
+    }
+    uint16_t* num = reinterpret_cast<uint16_t*>(scratch + nw * kWarpScratch);
+    const uint32_t W = (nc + 31) >> 5, Ws = row_stride(W);
+    for (uint32_t c = warp_id(); c < runs; c += nw) {
+        const uint32_t m = __shfl_sync(0xffffffffu, f, c), dm = __shfl_sync(0xffffffffu, g, c);
+        const uint32_t below = (1u << lane) - 1u;
+        const uint32_t at = __shfl_sync(0xffffffffu, ex, c) + __popc(m & below);
+        const uint32_t dat = __shfl_sync(0xffffffffu, dex, c) + __popc(dm & below);
+        if ((m >> lane) & 1u) {
+            C[at] = P.wadj[b + c * 32 + lane];
+            cnt[at] = 0;
+            num[at] = (uint16_t)(((dm >> lane) & 1u) ? dat : nd + at - dat);
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < nc * Ws; i += blockDim.x) rows[i] = 0;
+    __syncthreads();
+    if (threadIdx.x < nc) bytes += 16 + 4ull * (R.ne[C[threadIdx.x]] - R.nb[C[threadIdx.x]]);
+    block_window(C, nc, scratch - kWindowWords);
+    __syncthreads();
+    block_build_rows(C, nc, W, R.ne, R.adj, R.nb, rows, scratch - kWindowWords, num);
+    __syncthreads();
+    (void)block_dfs(rows, nc, W, r, cnt, &s_next, scratch, s, S, nd);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) {
+        const uint32_t j = num[i];
+        if (j >= nd || !cnt[j]) continue;
+        const uint32_t x = C[i];
+        lower(P, x, st_of(P.sl[x]), cnt[j], k, next, next_cnt);
+        bytes += 20;
+    }
+    __syncthreads();
+}
+
+// h = 4: the vertices list[0, nv), blocks taking (vertex, slice) units.
+// ANY: rows of other lengths are among them and passed over (phase 1 lists
+// its vertices by length; a compaction in the same pass may shorten one).
+template <bool ANY>
+__device__ __forceinline__ void drain_rows(const PeelParams& P, const NPlus& R,
+                                           const uint32_t* list, uint32_t nv, uint32_t* grab,
+                                           unsigned long long k, uint32_t* next,
+                                           uint32_t* next_cnt, uint32_t* smem, uint32_t* s_grab,
+                                           unsigned long long& items, unsigned long long& bytes) {
+    if (nv == 0) return;
+    // as many units as blocks: a slice repeats the row building
+    uint32_t S = gridDim.x / nv;
+    S = S < 1u ? 1u : (S > kMaxSlices ? kMaxSlices : S);
+    for (;;) {
+        if (threadIdx.x == 0) *s_grab = atomicAdd(grab, 1u);
+        __syncthreads();
+        const uint32_t u = *s_grab;
+        __syncthreads();
+        if (u >= nv * S) break;
+        const uint32_t v = list[u / S];
+        const uint64_t d = P.wend[v] - P.off[v];
+        if (ANY && (d <= kTinyRow || d > kBitmapMax)) continue;
+        process_row(P, R, v, u % S, S, k, next, next_cnt, smem, bytes);
+        if (threadIdx.x == 0 && u % S == 0) items += d;
+    }
+}
+
 // P2, phase 1: the cliques destroyed by frontier F (nf vertices, identical
 // for every block).  Frontier vertices marked gone (count 0) have no items.
-template <int NT>
+template <int NT, int HC>
 __device__ __forceinline__ void process_frontier(
     const PeelParams& P, const NPlus& R, const uint32_t* F, uint32_t nf, unsigned long long k,
-    uint32_t* Fnext, uint32_t* next_cnt, uint32_t* big_cnt, uint32_t* wC, unsigned* wCnt,
-    uint32_t* wRows, unsigned long long* s_pre, unsigned long long* s_red, uint32_t nh,
-    uint32_t* grab, uint32_t* s_grab, uint32_t par, unsigned long long& items,
-    unsigned long long& bytes) {
-    constexpr int NW = NT / 32;
-    const unsigned lane = lane_id(), wid = warp_id();
+    uint32_t* Fnext, uint32_t* next_cnt, uint32_t slot, uint32_t* smem, uint32_t* wC,
+    unsigned* wCnt, uint32_t* wRows, unsigned long long* s_pre, unsigned long long* s_red,
+    uint32_t* s_grab, uint32_t par, unsigned long long& items, unsigned long long& bytes) {
+    const unsigned lane = lane_id();
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t gthreads = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t gwarp = gtid >> 5;
     const uint64_t gwarps = gthreads >> 5;
+    PeelCtrl* c = P.ctrl;
     if (k == 0) return;   // every frontier vertex has count 0
-    if (nf <= kSmallFront) {
+    if (HC == 2 && nf <= kSmallFront) {
         // flatten (v, neighbour index) items over the whole grid
         block_prefix_degrees<NT>(P, F, nf, s_pre, s_red);
         unsigned long long T = s_pre[nf];
@@ -931,38 +1115,26 @@ __device__ __forceinline__ void process_frontier(
             items += T;
             bytes += 20ull * nf;   // frontier ids and their row bounds
         }
-        if (P.h == 2) {
-            for (uint64_t t = gtid; t < T; t += gthreads) {
-                uint32_t lo = 0, hi = nf;  // last i with s_pre[i] <= t
-                while (hi - lo > 1) {
-                    uint32_t mid = (lo + hi) >> 1;
-                    if (s_pre[mid] <= t) lo = mid; else hi = mid;
-                }
-                uint32_t v = F[lo];
-                uint32_t u = P.wadj[P.off[v] + (t - s_pre[lo])];
-                const uint32_t wu = P.sl[u];
-                bool dec;
-                (void)cand_ok(wu, u, 0u, v, dec);
-                bytes += 4 + 4;
-                if (dec) {
-                    lower(P, u, st_of(wu), 1ull, k, Fnext, next_cnt);
-                    bytes += 16;
-                }
+        for (uint64_t t = gtid; t < T; t += gthreads) {
+            uint32_t lo = 0, hi = nf;  // last i with s_pre[i] <= t
+            while (hi - lo > 1) {
+                uint32_t mid = (lo + hi) >> 1;
+                if (s_pre[mid] <= t) lo = mid; else hi = mid;
             }
-        } else {
-            for (uint64_t t = gwarp; t < T; t += gwarps) {
-                uint32_t lo = 0, hi = nf;
-                while (hi - lo > 1) {
-                    uint32_t mid = (lo + hi) >> 1;
-                    if (s_pre[mid] <= t) lo = mid; else hi = mid;
-                }
-                uint32_t v = F[lo];
-                uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
-                process_vw(P, R, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
-                           hub_bm_of(P, v, par), bytes);
+            uint32_t v = F[lo];
+            uint32_t u = P.wadj[P.off[v] + (t - s_pre[lo])];
+            const uint32_t wu = P.sl[u];
+            bool dec;
+            (void)cand_ok(wu, u, 0u, v, dec);
+            bytes += 4 + 4;
+            if (dec) {
+                lower(P, u, st_of(wu), 1ull, k, Fnext, next_cnt);
+                bytes += 16;
             }
         }
-    } else if (P.h == 2) {
+        return;
+    }
+    if (HC == 2) {
         for (uint64_t i = gwarp; i < nf; i += gwarps) {
             uint32_t v = F[i];
             if (st_of(P.sl[v]) != kFront) continue;
@@ -983,54 +1155,95 @@ __device__ __forceinline__ void process_frontier(
                 bytes += 20;
             }
         }
-    } else {
-        // The items of heavy vertices (P.heavy, nh: rows longer than
-        // heavy_min, flagged kHeavyBit) are flattened over every warp of the
-        // grid in batches of kSmallFront vertices; every other vertex goes to
-        // one block, blocks taking chunks of the frontier from *grab.
-        for (uint32_t b0 = 0; b0 < nh; b0 += kSmallFront) {
-            const uint32_t nb = nh - b0 < kSmallFront ? nh - b0 : kSmallFront;
-            const uint32_t* H = P.heavy + b0;
-            block_prefix_degrees<NT>(P, H, nb, s_pre, s_red);
-            unsigned long long T = s_pre[nb];
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                items += T;
-                bytes += 20ull * nb;
-            }
-            for (uint64_t t = gwarp; t < T; t += gwarps) {
-                uint32_t lo = 0, hi = nb;
-                while (hi - lo > 1) {
-                    uint32_t mid = (lo + hi) >> 1;
-                    if (s_pre[mid] <= t) lo = mid; else hi = mid;
-                }
-                uint32_t v = H[lo];
-                uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
-                process_vw(P, R, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
-                           hub_bm_of(P, v, par), bytes);
-            }
-            __syncthreads();   // s_pre is rewritten by the next batch
+        return;
+    }
+    // items spread over every warp of the grid, in batches of kSmallFront
+    // vertices: the whole of a small frontier (h = 3, >= 5) or the listed rows
+    const bool whole = HC != 4 && nf <= kSmallFront;
+    const uint32_t* L = whole ? F : P.heavy;
+    const uint32_t nh = whole ? nf : c->hcnt[slot];
+    for (uint32_t b0 = 0; b0 < nh; b0 += kSmallFront) {
+        const uint32_t nb = nh - b0 < kSmallFront ? nh - b0 : kSmallFront;
+        const uint32_t* H = L + b0;
+        block_prefix_degrees<NT>(P, H, nb, s_pre, s_red);
+        unsigned long long T = s_pre[nb];
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            items += T;
+            bytes += 20ull * nb;
         }
+        for (uint64_t t = gwarp; t < T; t += gwarps) {
+            uint32_t lo = 0, hi = nb;
+            while (hi - lo > 1) {
+                uint32_t mid = (lo + hi) >> 1;
+                if (s_pre[mid] <= t) lo = mid; else hi = mid;
+            }
+            uint32_t v = H[lo];
+            uint32_t w = P.wadj[P.off[v] + (t - s_pre[lo])];
+            process_vw<HC>(P, R, v, w, k, Fnext, next_cnt, wC, wCnt, wRows, &c->big_cnt[slot],
+                       hub_bm_of(P, v, par), bytes);
+        }
+        __syncthreads();   // s_pre is rewritten by the next batch
+    }
+    if (whole) return;
+    if (HC != 4) {
+        // the other vertices: blocks take chunks; in full chunks a warp takes
+        // each short row, the block's warps the neighbours of the others
         const uint32_t ch0 = nf / (4u * gridDim.x);
         const uint32_t ch = ch0 < 1u ? 1u : (ch0 > 32u ? 32u : ch0);
+        const uint32_t tiny = ch == 32u ? kTinyRow : 0u;
         for (;;) {
-            if (threadIdx.x == 0) *s_grab = atomicAdd(grab, ch);
+            if (threadIdx.x == 0) *s_grab = atomicAdd(&c->grab[slot], ch);
             __syncthreads();
             const uint32_t i0 = *s_grab;
             __syncthreads();
             if (i0 >= nf) break;
             const uint32_t i1 = i0 + ch < nf ? i0 + ch : nf;
+            for (uint32_t i = i0 + warp_id(); i < i1; i += NT / 32) {
+                const uint32_t v = F[i], wv = P.sl[v];
+                if ((wv & kListedBit) || st_of(wv) != kFront) continue;
+                const uint64_t d = P.wend[v] - P.off[v];
+                if (d > tiny) continue;
+                process_tiny<HC>(P, R, v, k, Fnext, next_cnt, wC, wCnt, wRows, bytes);
+                if (lane == 0) {
+                    items += d;
+                    bytes += 24;
+                }
+            }
             for (uint32_t i = i0; i < i1; i++) {
-                uint32_t v = F[i];
-                const uint32_t wv = P.sl[v];
-                if ((wv & kHeavyBit) || st_of(wv) != kFront) continue;   // taken above, or none
-                uint64_t b = P.off[v], e = P.wend[v];
-                for (uint64_t p = b + wid; p < e; p += NW)
-                    process_vw(P, R, v, P.wadj[p], k, Fnext, next_cnt, wC, wCnt, wRows, big_cnt,
-                               nullptr, bytes);
+                const uint32_t v = F[i], wv = P.sl[v];
+                if ((wv & kListedBit) || st_of(wv) != kFront) continue;
+                const uint64_t b = P.off[v], e = P.wend[v];
+                if (e - b <= tiny) continue;
+                for (uint64_t p = b + warp_id(); p < e; p += NT / 32)
+                    process_vw<HC>(P, R, v, P.wadj[p], k, Fnext, next_cnt, wC, wCnt, wRows,
+                               &c->big_cnt[slot], nullptr, bytes);
                 if (threadIdx.x == 0) {
                     items += e - b;
                     bytes += 24;
                 }
+            }
+        }
+        return;
+    }
+    // whole neighbourhoods: longer rows first, then the short ones
+    drain_rows<false>(P, R, P.vlist, c->vcnt[slot], &c->vgrab[slot], k, Fnext, next_cnt, smem,
+                      s_grab, items, bytes);
+    __syncthreads();   // the warps' buffers overlap the block's
+    const uint32_t ch0 = nf / (8u * (uint32_t)gwarps);
+    const uint32_t ch = ch0 < 1u ? 1u : (ch0 > 32u ? 32u : ch0);
+    for (;;) {
+        uint32_t i0 = 0;
+        if (lane == 0) i0 = atomicAdd(&c->grab[slot], ch);
+        i0 = __shfl_sync(0xffffffffu, i0, 0);
+        if (i0 >= nf) break;
+        const uint32_t i1 = i0 + ch < nf ? i0 + ch : nf;
+        for (uint32_t i = i0; i < i1; i++) {
+            const uint32_t v = F[i], wv = P.sl[v];
+            if ((wv & kListedBit) || st_of(wv) != kFront) continue;   // taken above, or none
+            process_tiny<HC>(P, R, v, k, Fnext, next_cnt, wC, wCnt, wRows, bytes);
+            if (lane == 0) {
+                items += P.wend[v] - P.off[v];
+                bytes += 24;
             }
         }
     }
@@ -1038,11 +1251,13 @@ __device__ __forceinline__ void process_frontier(
 
 // P2, phase 2: the frontiers of all bands together (nf vertices), in batches
 // whose items are flattened over the grid.
-template <int NT>
+template <int NT, int HC>
 __device__ __forceinline__ void process_bands(
-    const PeelParams& P, const NPlus& R, const uint32_t* F, uint32_t nf, uint32_t* big_cnt,
-    uint32_t* wC, unsigned* wCnt, uint32_t* wRows, unsigned long long* s_pre,
-    unsigned long long* s_red, unsigned long long& items, unsigned long long& bytes) {
+    const PeelParams& P, const NPlus& R, const uint32_t* F, uint32_t nf, uint32_t slot,
+    uint32_t* smem, uint32_t* wC, unsigned* wCnt, uint32_t* wRows, unsigned long long* s_pre,
+    unsigned long long* s_red, uint32_t* s_grab, unsigned long long& items,
+    unsigned long long& bytes) {
+    PeelCtrl* c = P.ctrl;
     const unsigned lane = lane_id();
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t gthreads = (uint64_t)gridDim.x * blockDim.x;
@@ -1051,7 +1266,8 @@ __device__ __forceinline__ void process_bands(
     for (uint32_t b0 = 0; b0 < nf; b0 += kSmallFront) {
         const uint32_t nb = nf - b0 < kSmallFront ? nf - b0 : kSmallFront;
         const uint32_t* H = F + b0;
-        block_prefix_degrees<NT>(P, H, nb, s_pre, s_red);
+        // h = 4: only the rows that are not taken whole below
+        block_prefix_degrees<NT>(P, H, nb, s_pre, s_red, HC == 4 ? kBitmapMax : 0u);
         const unsigned long long T = s_pre[nb];
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             items += T;
@@ -1066,7 +1282,7 @@ __device__ __forceinline__ void process_bands(
             }
             return lo;
         };
-        if (P.h == 2) {
+        if (HC == 2) {
             for (uint64_t t = gtid; t < T; t += gthreads) {
                 const uint32_t i = at(t), v = H[i];
                 const uint32_t u = P.wadj[P.off[v] + (t - s_pre[i])];
@@ -1078,7 +1294,7 @@ __device__ __forceinline__ void process_bands(
                     bytes += 16;
                 }
             }
-        } else if (P.h == 3) {
+        } else if (HC == 3) {
             // a warp looks at `cs` consecutive items at once, one a lane, and
             // takes the pairs among them one by one: most items name a
             // vertex of a later band and need nothing more
@@ -1109,11 +1325,22 @@ __device__ __forceinline__ void process_bands(
             for (uint64_t t = gwarp; t < T; t += gwarps) {
                 const uint32_t i = at(t), v = H[i];
                 const uint32_t w = P.wadj[P.off[v] + (t - s_pre[i])];
-                process_vw(P, R, v, w, 0ull, nullptr, nullptr, wC, wCnt, wRows, big_cnt, nullptr,
-                           bytes);
+                process_vw<HC>(P, R, v, w, 0ull, nullptr, nullptr, wC, wCnt, wRows,
+                           &c->big_cnt[slot], nullptr, bytes);
             }
         }
         __syncthreads();   // s_pre is rewritten by the next batch
+    }
+    if (HC != 4) return;
+    drain_rows<true>(P, R, F, nf, &c->vgrab[slot], 0ull, nullptr, nullptr, smem, s_grab, items,
+                     bytes);
+    __syncthreads();   // the warps' buffers overlap the block's
+    for (uint64_t i = gwarp; i < nf; i += gwarps) {
+        const uint32_t v = F[i];
+        const uint64_t d = P.wend[v] - P.off[v];
+        if (d > kTinyRow) continue;
+        process_tiny<HC>(P, R, v, 0ull, nullptr, nullptr, wC, wCnt, wRows, bytes);
+        if (lane == 0) items += d;
     }
 }
 
@@ -1144,7 +1371,8 @@ __device__ __forceinline__ void process_queued(const PeelParams& P, const NPlus&
 }
 
 // ---------------------------------------------------------------- kernel
-template <int NT>
+// HC: the clique size, 5 for all from 5 on (P.h): each has its own registers.
+template <int NT, int HC>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) uint32_t smem[];
@@ -1239,17 +1467,19 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             if (nhub > P.hub_slots) nhub = P.hub_slots;
             if (nhub) hub_bitmaps<NT>(P, nhub, (r + 1) & 1, true, s_pre, s_red, bytes);
         }
-        // mark F_r; rows longer than heavy_min also go to the heavy list
+        // mark F_r; all but the short rows are also listed
         for (uint64_t base = gwarp * 32; base < fcur && !undo; base += gwarps * 32) {
             uint64_t i = base + lane;
-            bool hv = false;
-            uint32_t v = 0;
+            uint32_t v = 0, cls = 0;
             if (i < fcur) {
                 v = Fcur[i];
-                P.sl[v] = front_word(P, c, v, r & 1, hv);
-                bytes += 4 + 4 + 8 + (P.heavy_min ? 16 : 0);
+                P.sl[v] = front_word<HC>(P, c, v, r & 1, cls);
+                bytes += 4 + 4 + 8 + (HC > 2 ? 16 : 0);
             }
-            if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
+            if (HC > 2) {
+                warp_append(cls == 2, v, &c->hcnt[r % 3], P.heavy);
+                warp_append(cls == 1, v, &c->vcnt[r % 3], P.vlist);
+            }
         }
         if (lead) {
             if (r) {
@@ -1260,6 +1490,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             }
             c->fcnt[(r + 1) % 3] = 0;
             c->hcnt[(r + 1) % 3] = 0;
+            c->vcnt[(r + 1) % 3] = 0;
+            c->vgrab[(r + 1) % 3] = 0;
             c->grab[(r + 1) % 3] = 0;
         }
         BARRIER(0);
@@ -1292,7 +1524,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             if (left == 0) break;
             if (multi) fails = 0;
             const bool banding = left <= P.band_max && nb < kMaxBands && hold == 0 &&
-                                 (P.h > 2 || rs >= kBandAfter2);
+                                 (HC > 2 || rs >= kBandAfter2);
             if (hold) hold--;
             const uint32_t* Ain = P.alive[ap];
             uint32_t* Aout = P.alive[ap ^ 1];
@@ -1384,19 +1616,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             }
             for (uint64_t base = gwarp * 32; base < left; base += gwarps * 32) {
                 uint64_t i = base + lane;
-                bool in = false, hv = false;
-                uint32_t v = 0;
+                bool in = false;
+                uint32_t v = 0, cls = 0;
                 if (i < left) {
                     v = Aout[i];
                     bytes += 4 + 8;
                     if (P.deg[v] <= k) {
                         in = true;
-                        P.sl[v] = front_word(P, c, v, r & 1, hv);
-                        bytes += 4 + 4 + (P.heavy_min ? 16 : 0);
+                        P.sl[v] = front_word<HC>(P, c, v, r & 1, cls);
+                        bytes += 4 + 4 + (HC > 2 ? 16 : 0);
                     }
                 }
                 warp_append(in, v, &c->fcnt[r % 3], Fcur);
-                if (P.heavy_min) warp_append(hv, v, &c->hcnt[r % 3], P.heavy);
+                if (HC > 2) {
+                    warp_append(cls == 2, v, &c->hcnt[r % 3], P.heavy);
+                    warp_append(cls == 1, v, &c->vcnt[r % 3], P.vlist);
+                }
             }
             BARRIER(2);
             fcur = c->fcnt[r % 3];
@@ -1413,12 +1648,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
         }
         // when everything left leaves at once there is no count to lower
         if (retired + fcur < P.n) {
-            process_frontier<NT>(P, R1, Fcur, fcur, k, P.front[(r + 1) % 3],
-                                 &c->fcnt[(r + 1) % 3], &c->big_cnt[r % 3], wC, wCnt, wRows,
-                                 s_pre, s_red, c->hcnt[r % 3], &c->grab[r % 3], &s_grab, r & 1,
-                                 items, bytes);
+            process_frontier<NT, HC>(P, R1, Fcur, fcur, k, P.front[(r + 1) % 3],
+                                 &c->fcnt[(r + 1) % 3], r % 3, smem, wC, wCnt, wRows, s_pre,
+                                 s_red, &s_grab, r & 1, items, bytes);
             BARRIER(3);
-            if (P.big_cap) {
+            if (HC >= 4 && P.big_cap) {
                 const uint32_t nbig = c->big_cnt[r % 3], nmid = c->big_cnt[3 + r % 3];
                 if (nbig || nmid) {
                     process_queued<NT>(P, R1, r % 3, nbig, nmid, k, P.front[(r + 1) % 3],
@@ -1446,6 +1680,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
         if (lead) {
             c->fcnt[0] = c->fcnt[1] = c->fcnt[2] = 0;
             c->busy[0] = c->busy[1] = c->busy[2] = 0;
+            c->vgrab[0] = c->vgrab[1] = c->vgrab[2] = 0;
             for (int i = 0; i < 6; i++) c->big_cnt[i] = c->bgrab[i] = 0;
         }
         // band sizes: the first position past seg whose key differs
@@ -1577,6 +1812,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             if (lead) {
                 c->fcnt[(q + 1) % 3] = 0;
                 c->busy[(q + 1) % 3] = 0;
+                c->vgrab[(q + 1) % 3] = 0;
                 if (q) {
                     c->big_cnt[(q + 2) % 3] = 0;
                     c->bgrab[(q + 2) % 3] = 0;
@@ -1587,10 +1823,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             BARRIER(4);
             if (c->busy[q % 3] == 0) break;
             // ------------------------------------------------------- P2
-            process_bands<NT>(P, R2, F, *fcnt, &c->big_cnt[q % 3], wC, wCnt, wRows, s_pre, s_red,
-                              items, bytes);
+            process_bands<NT, HC>(P, R2, F, *fcnt, q % 3, smem, wC, wCnt, wRows, s_pre, s_red,
+                              &s_grab, items, bytes);
             BARRIER(6);
-            if (P.big_cap) {
+            if (HC >= 4 && P.big_cap) {
                 const uint32_t nbig = c->big_cnt[q % 3], nmid = c->big_cnt[3 + q % 3];
                 if (nbig || nmid) {
                     process_queued<NT>(P, R2, q % 3, nbig, nmid, 0ull, nullptr, nullptr, smem,
@@ -1852,22 +2088,22 @@ __global__ void k_barrier_probe(PeelCtrl* c, uint64_t wait_ns, int absent) {
     if (blockIdx.x == 0 && threadIdx.x == 0) c->barriers = 4;
 }
 
-template <int NT>
+template <int NT, int HC>
 cudaError_t launch_peel(PeelParams& P, int sms, size_t smem, cudaStream_t s, unsigned* grid_out) {
     // opt in for every launch: the 48 KB default bounds static + dynamic
     // shared memory together, and the attribute persists across calls
-    cudaError_t e = cudaFuncSetAttribute(k_peel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute((k_peel<NT, HC>), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_peel<NT>, NT, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (k_peel<NT, HC>), NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
     // one block per SM: the fewest barrier arrivals
     unsigned grid = (unsigned)sms;
     *grid_out = grid;
     void* args[] = {&P};
-    e = cudaLaunchCooperativeKernel((void*)k_peel<NT>, dim3(grid), dim3(NT), args, smem, s);
+    e = cudaLaunchCooperativeKernel((void*)k_peel<NT, HC>, dim3(grid), dim3(NT), args, smem, s);
     note_launch();
     return e;
 }
@@ -1938,7 +2174,6 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     P.k0 = kstart ? kstart - 1 : 0;
     P.snap = snap;
     P.cap = maxdplus < 32 ? 32 : maxdplus;
-    P.bcap = P.cap < kBitmapMax ? P.cap : kBitmapMax;
     P.warp_cand = warp_cand_limit(h);
     P.gather_cap = P.warp_cand;
     P.compact = h >= 3 ? 1 : 0;
@@ -1946,25 +2181,18 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
     // Big items (candidate sets above warp_cand vertices) for h >= 4; every
     // candidate set fits 32-word rows.
     const bool big_items = h >= 4;
-    // Shared memory: per-warp candidate buffers (h >= 3) or the big-item bitmap
+    // Shared memory: per-warp candidate buffers (h >= 3), which share the
+    // space of the bitmap search's (h >= 4)
     constexpr int NT = 1024;
     size_t work = h >= 3 ? (size_t)(NT / 32) * kWarpWords : 0;
-    // phase-1 frontier vertices with more items than a block's warps take in
-    // four passes have their items spread over the whole grid
-    P.heavy_min = h >= 3 ? 4u * (NT / 32) : 0u;
-    // neighbourhood bitmaps for frontier vertices with rows above 512 (a
+    if (h >= 4) work = bitmap_words(kBitmapMax, NT / 32) + (h == 4 ? kBitmapMax / 2 : 0);
+    // neighbourhood bitmaps for frontier vertices with the longest rows (a
     // binary search there takes 10 or more probes): up to 64 per round, two
     // sets, within 64 MiB
     if (h >= 3) {
         P.hub_words = ((uint64_t)n + 31) / 32;
         uint64_t slots = (64ull << 20) / (2 * 4 * P.hub_words);
         P.hub_slots = (uint32_t)(slots > 64 ? 64 : (slots < 4 ? 0 : slots));
-        P.hub_min = 4 * P.heavy_min;
-    }
-    if (big_items) {
-        // (cap > kBitmapMax: the split search uses the full-size layout)
-        size_t big = bitmap_words(P.bcap, NT / 32);
-        if (big > work) work = big;
     }
     const size_t smem = work * 4;
 
@@ -2009,8 +2237,9 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
             P.gather_cap = kWarpCand;
         }
     }
-    if (P.heavy_min && (st = dalloc(&heavy, n, s)) != DSD_OK) goto done;
+    if (h >= 3 && (st = dalloc(&heavy, (size_t)2 * n, s)) != DSD_OK) goto done;
     P.heavy = heavy;
+    P.vlist = heavy + n;
     if (big_items && P.cap > kBitmapMax &&
         (st = dalloc(&xl, (size_t)sms * (kMaxDepth + 1) * P.cap, s)) != DSD_OK)
         goto done;
@@ -2056,7 +2285,11 @@ dsd_status run_peel(dsd_graph* g, int h, uint32_t n, const uint64_t* off, const 
         note_launch();
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = launch_peel<NT>(P, sms, smem, s, &grid);
+    if (e == cudaSuccess)
+        e = h == 2   ? launch_peel<NT, 2>(P, sms, smem, s, &grid)
+            : h == 3 ? launch_peel<NT, 3>(P, sms, smem, s, &grid)
+            : h == 4 ? launch_peel<NT, 4>(P, sms, smem, s, &grid)
+                     : launch_peel<NT, 5>(P, sms, smem, s, &grid);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctrl, sizeof(PeelCtrl), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {

@@ -238,7 +238,7 @@ __device__ void app_big(const AppParams& P, const AppQ& Q, uint32_t v, uint32_t 
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);   // bcap
     uint32_t* C = smem + 2 * P.bcap;                                           // bcap
     uint32_t* rows = smem + bitmap_rows_at(P.bcap);                            // bcap rows
-    uint32_t* scratch = rows + P.bcap * row_stride((P.bcap + 31) >> 5);
+    uint32_t* scratch = smem + bitmap_scratch_at(P.bcap);
     __shared__ uint32_t s_nc, s_next, s_w[32], s_t2;
     __shared__ unsigned long long s_tot;
     const uint64_t wb = P.split[w], we = P.off[w + 1];
@@ -288,7 +288,9 @@ __device__ void app_big(const AppParams& P, const AppQ& Q, uint32_t v, uint32_t 
     for (uint32_t i = threadIdx.x; i < nc; i += blockDim.x) cnt[i] = 0;
     for (uint32_t i = threadIdx.x; i < nc * row_stride(W); i += blockDim.x) rows[i] = 0;
     __syncthreads();
-    block_build_rows(C, nc, W, P.off + 1, P.adj, P.split, rows);
+    block_window(C, nc, scratch - kWindowWords);
+    __syncthreads();
+    block_build_rows(C, nc, W, P.off + 1, P.adj, P.split, rows, scratch - kWindowWords);
     __syncthreads();
     unsigned long long mine = block_dfs(rows, nc, W, P.h - 2, cnt, &s_next, scratch);
     if (mine) atomicAdd(&s_tot, mine);

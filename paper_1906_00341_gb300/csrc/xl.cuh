@@ -80,7 +80,7 @@ __device__ void xl_cliques(const uint32_t* C0, uint32_t n0, int rr0, const uint6
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);   // kBitmapMax
     uint32_t* Cs = smem + 2 * kBitmapMax;                                    // kBitmapMax
     uint32_t* rows = smem + bitmap_rows_at(kBitmapMax);
-    uint32_t* wscratch = rows + kBitmapMax * kRowStrideMax;
+    uint32_t* wscratch = smem + bitmap_scratch_at(kBitmapMax);
     if (threadIdx.x == 0) {
         s_lv[0] = XLLevel{C0, n0, rr0, 0u, 0u};
         s_t = 0;
@@ -136,7 +136,9 @@ __device__ void xl_cliques(const uint32_t* C0, uint32_t n0, int rr0, const uint6
                 for (uint32_t i = threadIdx.x; i < n * row_stride(W); i += blockDim.x) rows[i] = 0;
                 if (threadIdx.x == 0) s_next = 0;
                 __syncthreads();
-                block_build_rows(Cs, n, W, ne, adj, nb, rows);
+                block_window(Cs, n, wscratch - kWindowWords);
+                __syncthreads();
+                block_build_rows(Cs, n, W, ne, adj, nb, rows, wscratch - kWindowWords);
                 __syncthreads();
                 mine = block_dfs(rows, n, W, L.rr, cnt, &s_next, wscratch);
                 __syncthreads();
