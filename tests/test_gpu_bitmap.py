@@ -48,3 +48,28 @@ def test_random_dense(L, orc, n, p, h):
     if core is not None:
         wcore, wk = orc.core_decompose(og, h)
         assert k == wk and np.array_equal(core, wcore)
+
+
+@pytest.mark.parametrize("d", [31, 32, 33, 63, 64, 1024, 1025, 12288, 12289])
+def test_noalloc_row_tiers(L, d):
+    """dsd_triangle_degrees_noalloc on both sides of its row tiers: a hub of
+    exactly d higher-id neighbours, which carry edges of their own."""
+    import torch
+    rng = np.random.default_rng(d)
+    n = d + 40
+    ring = np.arange(1, d + 1)
+    a = rng.integers(1, n, 6 * n)
+    b = rng.integers(1, n, 6 * n)
+    near = np.minimum(ring + rng.integers(1, 9, d), n - 1)
+    s = np.concatenate([np.zeros(d, np.int64), ring, a]).astype(np.uint32)
+    t = np.concatenate([ring, near, b]).astype(np.uint32)
+    with L.Graph.from_edges(n, s, t) as g:
+        want, wmu = g.clique_degrees(3)
+        off, adj = g.csr(mem="device")
+    deg = torch.full((n,), -1, dtype=torch.int64, device="cuda")
+    mu = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    L.dsd_triangle_degrees_noalloc(n, off.data_ptr(), adj.data_ptr(), deg.data_ptr(),
+                                   mu.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert int(mu.item()) == wmu
+    assert np.array_equal(deg.cpu().numpy().astype(np.uint64), want)
