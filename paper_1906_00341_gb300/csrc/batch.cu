@@ -190,13 +190,11 @@ __device__ void block_radix_sort(uint32_t* a, uint32_t* b, uint32_t cnt, int bit
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < cnt; i += NT) atomicAdd(&S.base[(src[i] >> shift) & 255u], 1u);
         __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t run = 0;
-            for (int d = 0; d < 256; d++) {
-                uint32_t t = S.base[d];
-                S.base[d] = run;
-                run += t;
-            }
+        {
+            uint32_t all;
+            const uint32_t ex =
+                bscan<NT>(threadIdx.x < 256 ? S.base[threadIdx.x] : 0u, S.ured, &all);
+            if (threadIdx.x < 256) S.base[threadIdx.x] = ex;
         }
         __syncthreads();
         for (uint32_t t0 = 0; t0 < cnt; t0 += TILE) {
@@ -257,47 +255,116 @@ __device__ void block_radix_sort(uint32_t* a, uint32_t* b, uint32_t cnt, int bit
     __syncthreads();
 }
 
-__device__ __forceinline__ uint32_t key_bits(uint64_t maxkey) {
-    uint32_t b = 0;
-    while (b < 32 && (maxkey >> b)) b += 8;
-    return b ? b : 8;
+// Exclusive prefix sums of a[0..n) into out[0..n] by one CTA; returns the total.
+template <int NT>
+__device__ uint32_t block_prefix(const uint32_t* a, uint32_t n, uint32_t* out, Smem<NT>& S) {
+    uint32_t run = 0;
+    for (uint32_t t0 = 0; t0 < n; t0 += NT) {
+        const uint32_t i = t0 + threadIdx.x;
+        uint32_t tot;
+        const uint32_t ex = bscan<NT>(i < n ? a[i] : 0u, S.ured, &tot);
+        if (i < n) out[i] = run + ex;
+        run += tot;
+    }
+    if (threadIdx.x == 0) out[n] = run;
+    __syncthreads();
+    return run;
 }
 
-// Sorted keys u * n + v (deduplicated in place) -> CSR off[0..n], adj.
-// Returns the number of entries.
+// Sorts the rows vals[pos[v] .. pos[v] + len[v]) ascending in place, dropping
+// repeats; len[v] becomes the unique length.  A warp a row: a bitonic network
+// in registers up to 32 entries, in its own buffer up to kWarpSortMax; longer
+// rows (listed in `longs`) by the whole CTA.  One radix sort over all (row,
+// entry) keys took 8 passes over the edges and block barriers for each tile:
+// the largest graph of a batch (50,000 vertices, 546,000 edges, h = 4) spent
+// some 18 of 46 ms there.
+constexpr uint32_t kWarpSortMax = 512;
 template <int NT>
-__device__ uint32_t keys_to_csr(uint32_t* keys, uint32_t cnt, uint32_t n, uint32_t* off,
-                                uint32_t* adj, Smem<NT>& S) {
-    // unique (ordered compaction; each pass reads its tile before writing)
-    if (threadIdx.x == 0) S.cnt1 = 0;
+__device__ void block_sort_rows(uint32_t* vals, uint32_t* scratch, const uint32_t* pos,
+                                uint32_t* len, uint32_t n, uint32_t* longs, Smem<NT>& S) {
+    constexpr int NW = NT / 32;
+    const unsigned lane = lane_id(), wid = warp_id();
+    if (threadIdx.x == 0) S.cnt2 = 0;
     __syncthreads();
-    for (uint32_t t0 = 0; t0 < cnt; t0 += NT) {
-        uint32_t i = t0 + threadIdx.x;
-        uint32_t k = i < cnt ? keys[i] : 0u;
-        bool keep = i < cnt && (i == 0 || keys[i - 1] != k);
-        uint32_t tot;
-        uint32_t at = bscan<NT>(keep ? 1u : 0u, S.ured, &tot);
-        uint32_t o = S.cnt1;
-        __syncthreads();
-        if (keep) keys[o + at] = k;
-        __syncthreads();
-        if (threadIdx.x == 0) S.cnt1 = o + tot;
-        __syncthreads();
-    }
-    uint32_t u = S.cnt1;
-    for (uint32_t i = threadIdx.x; i < u; i += NT) adj[i] = keys[i] % n;
-    for (uint32_t v = threadIdx.x; v <= n; v += NT) {
-        uint32_t target = v * n;  // first key of row v (v < n; v == n gives u)
-        uint32_t lo = 0, hi = u;
-        if (v == n) lo = u;
-        while (lo < hi) {
-            uint32_t mid = (lo + hi) >> 1;
-            if (keys[mid] < target) lo = mid + 1; else hi = mid;
+    uint32_t* sw = S.wbuf[wid];
+    for (uint32_t v = wid; v < n; v += NW) {
+        const uint32_t l = len[v];
+        uint32_t* row = vals + pos[v];
+        if (l <= 32) {
+            uint32_t x = lane < l ? row[lane] : kNone;
+#pragma unroll
+            for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+                for (int j = k >> 1; j > 0; j >>= 1) {
+                    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+                    const bool asc = (lane & k) == 0, lower = (lane & j) == 0;
+                    x = (lower == asc) ? min(x, y) : max(x, y);
+                }
+            }
+            const uint32_t prev = __shfl_up_sync(0xffffffffu, x, 1);
+            const bool keep = lane < l && (lane == 0 || x != prev);
+            const unsigned b = __ballot_sync(0xffffffffu, keep);
+            if (keep) row[__popc(b & ((1u << lane) - 1u))] = x;
+            if (lane == 0) len[v] = __popc(b);
+            continue;
         }
-        off[v] = lo;
+        if (l > kWarpSortMax) {
+            if (lane == 0) longs[atomicAdd(&S.cnt2, 1u)] = v;
+            continue;
+        }
+        uint32_t N = 64;
+        while (N < l) N <<= 1;
+        for (uint32_t j = lane; j < N; j += 32) sw[j] = j < l ? row[j] : kNone;
+        __syncwarp();
+        for (uint32_t k = 2; k <= N; k <<= 1) {
+            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+                for (uint32_t x = lane; x < N; x += 32) {
+                    const uint32_t y = x ^ j;
+                    if (y > x) {
+                        const bool asc = (x & k) == 0;
+                        const uint32_t a = sw[x], b = sw[y];
+                        if ((a > b) == asc) {
+                            sw[x] = b;
+                            sw[y] = a;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+        }
+        uint32_t out = 0;
+        for (uint32_t b0 = 0; b0 < l; b0 += 32) {
+            const uint32_t x = b0 + lane;
+            const uint32_t val = x < l ? sw[x] : 0u;
+            const bool keep = x < l && (x == 0 || val != sw[x - 1]);
+            const unsigned bal = __ballot_sync(0xffffffffu, keep);
+            if (keep) row[out + __popc(bal & ((1u << lane) - 1u))] = val;
+            out += __popc(bal);
+        }
+        if (lane == 0) len[v] = out;
+        __syncwarp();
     }
     __syncthreads();
-    return u;
+    const uint32_t nl = S.cnt2;
+    for (uint32_t i = 0; i < nl; i++) {
+        const uint32_t v = longs[i], l = len[v];
+        uint32_t* row = vals + pos[v];
+        block_radix_sort<NT>(row, scratch, l, 16, S);   // ids below 2^16
+        uint32_t out = 0;
+        for (uint32_t t0 = 0; t0 < l; t0 += NT) {
+            const uint32_t x = t0 + threadIdx.x;
+            const uint32_t val = x < l ? row[x] : 0u;
+            const bool keep = x < l && (x == 0 || row[x - 1] != val);
+            uint32_t tot;
+            const uint32_t at = bscan<NT>(keep ? 1u : 0u, S.ured, &tot);
+            if (keep) scratch[out + at] = val;
+            out += tot;
+        }
+        __syncthreads();
+        for (uint32_t x = threadIdx.x; x < out; x += NT) row[x] = scratch[x];
+        if (threadIdx.x == 0) len[v] = out;
+        __syncthreads();
+    }
 }
 
 // ------------------------------------------------------------ peeling
@@ -418,37 +485,44 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
     }
     __syncthreads();
     unsigned long long k = 0;
-    uint32_t na = n, nlev = 0, r = 0;
+    uint32_t na = n, left = n, nlev = 0, r = 0;   // list entries, alive vertices
     uint32_t* F = B.fa;
     uint32_t* G = B.fb;
     uint32_t nf = 0;
     for (;;) {
         if (nf == 0) {
-            // level jump: compact the alive list, minimum count, frontier
-            if (threadIdx.x == 0) S.cnt2 = 0;
-            __syncthreads();
+            // level jump: minimum count and frontier; the alive list is
+            // compacted when it has halved (a block scan per NT entries,
+            // several barriers each; a plain pass needs none)
             unsigned long long mn = ~0ull;
-            for (uint32_t t0 = 0; t0 < na; t0 += NT) {
-                uint32_t i = t0 + threadIdx.x;
-                uint32_t v = i < na ? B.alive[i] : 0u;
-                bool keep = i < na && B.st[v] == kAl;
-                if (keep) mn = B.deg[v] < mn ? B.deg[v] : mn;
-                uint32_t tot;
-                uint32_t at = bscan<NT>(keep ? 1u : 0u, S.ured, &tot);
-                uint32_t o = S.cnt2;
+            if (2 * left <= na) {
+                if (threadIdx.x == 0) S.cnt2 = 0;
                 __syncthreads();
-                if (keep) B.alive[o + at] = v;
-                __syncthreads();
-                if (threadIdx.x == 0) S.cnt2 = o + tot;
-                __syncthreads();
+                for (uint32_t t0 = 0; t0 < na; t0 += NT) {
+                    uint32_t i = t0 + threadIdx.x;
+                    uint32_t v = i < na ? B.alive[i] : 0u;
+                    bool keep = i < na && B.st[v] == kAl;
+                    uint32_t tot;
+                    uint32_t at = bscan<NT>(keep ? 1u : 0u, S.ured, &tot);
+                    uint32_t o = S.cnt2;
+                    __syncthreads();
+                    if (keep) B.alive[o + at] = v;
+                    __syncthreads();
+                    if (threadIdx.x == 0) S.cnt2 = o + tot;
+                    __syncthreads();
+                }
+                na = left;
             }
-            na = S.cnt2;
+            if (left == 0) break;
+            for (uint32_t i = threadIdx.x; i < na; i += NT) {
+                const uint32_t v = B.alive[i];
+                if (B.st[v] == kAl) mn = B.deg[v] < mn ? B.deg[v] : mn;
+            }
             mn = bmin<NT>(mn, S.red);
-            if (na == 0) break;
             k = mn > k ? mn : k;
             if (threadIdx.x == 0) {
                 B.lk[nlev] = k;
-                B.ls[nlev] = na;
+                B.ls[nlev] = left;
                 B.lm[nlev] = S.mu_alive;
                 S.cnt1 = 0;
             }
@@ -456,7 +530,7 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
             __syncthreads();
             for (uint32_t i = threadIdx.x; i < na; i += NT) {
                 uint32_t v = B.alive[i];
-                if (B.deg[v] <= k) F[atomicAdd(&S.cnt1, 1u)] = v;
+                if (B.st[v] == kAl && B.deg[v] <= k) F[atomicAdd(&S.cnt1, 1u)] = v;
             }
             __syncthreads();
             nf = S.cnt1;
@@ -465,9 +539,14 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
         if (threadIdx.x == 0) S.cnt2 = 0;   // next frontier size
         __syncthreads();
         unsigned long long destroyed = 0;
-        if (B.h == 2) {
+        // a frontier vertex of count 0 lies in no clique of the current set:
+        // nothing to enumerate (frontier counts do not change here), and at
+        // level 0 that is every one of them
+        if (k == 0) {
+        } else if (B.h == 2) {
             for (uint32_t i = wid; i < nf; i += NW) {
                 uint32_t v = F[i];
+                if (B.deg[v] == 0) continue;
                 for (uint32_t p = B.off[v] + lane; p < B.off[v + 1]; p += 32) {
                     uint32_t u = B.adj[p];
                     uint32_t s = B.st[u];
@@ -482,9 +561,14 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
         } else {
             uint32_t* C = S.wbuf[wid];
             uint32_t* cnt = C + kBatchMaxDplus;
-            for (uint32_t i = 0; i < nf; i++) {
+            // many frontier vertices: a warp each; few: the block's warps share
+            // the neighbours of one after another
+            const bool each = nf >= 2 * NW;
+            for (uint32_t i = each ? wid : 0; i < nf; i += each ? NW : 1) {
                 uint32_t v = F[i];
-                for (uint32_t p = B.off[v] + wid; p < B.off[v + 1]; p += NW) {
+                if (B.deg[v] == 0) continue;
+                for (uint32_t p = B.off[v] + (each ? 0 : wid); p < B.off[v + 1];
+                     p += each ? 1 : NW) {
                     unsigned long long t = bitem<LPR>(B, v, B.adj[p], k, G, &S.cnt2, C, cnt);
                     if (lane == 0) destroyed += t;
                 }
@@ -499,6 +583,7 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
         }
         if (threadIdx.x == 0) S.mu_alive -= destroyed;
         __syncthreads();
+        left -= nf;
         nf = S.cnt2;
         uint32_t* t = F;
         F = G;
@@ -517,13 +602,118 @@ __device__ __forceinline__ bool bratio_ge(unsigned long long a, unsigned long lo
     return lhi > rhi || (lhi == rhi && llo >= rlo);
 }
 
+// A warp's buffer for candidate sets of 33 .. kBatchWarpRows: ids, 64-bit
+// counts, rows of row_stride(4) words, scratch of the node search.
+constexpr uint32_t kBatchWarpRows = 128;
+static_assert(3 * kBatchWarpRows + kBatchWarpRows * row_stride(4) + kWarpScratch <=
+                  2 * kBatchMaxDplus + 64,
+              "the warp's buffer holds the rows");
+__device__ __forceinline__ unsigned long long* warp_counts64(uint32_t* buf) {
+    return reinterpret_cast<unsigned long long*>(buf + kBatchWarpRows);
+}
+
+// warp_build_rows32 with the bounds of all lists loaded by a lane each and four
+// lists' first entries in flight: a CTA's 32 warps alone do not hide the two
+// dependent loads a list takes otherwise.
+__device__ void warp_rows32_ahead(const uint32_t* C, uint32_t nc, const uint32_t* off,
+                                  const uint32_t* adj, const uint32_t* nb, uint32_t* rows) {
+    const unsigned full = 0xffffffffu, lane = lane_id();
+    const uint32_t cmax = C[nc - 1], m = nc - 1;
+    uint32_t lb = 0, le = 0;
+    if (lane < m) {
+        lb = nb[C[lane]];
+        le = off[C[lane] + 1];
+    }
+    for (uint32_t i0 = 0; i0 < m; i0 += 4) {
+        uint32_t b[4], e[4], y[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t i = i0 + q < m ? i0 + q : m - 1;
+            b[q] = __shfl_sync(full, lb, i);
+            e[q] = __shfl_sync(full, le, i);
+            y[q] = b[q] + lane < e[q] ? adj[b[q] + lane] : kNone;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t i = i0 + q;
+            if (i >= m) break;
+            uint32_t bits = 0;
+            for (uint32_t p = b[q];;) {
+                if (y[q] <= cmax) {
+                    const uint32_t pos = (uint32_t)lower_bound_u32(C, nc, y[q]);
+                    if (pos < nc && C[pos] == y[q]) bits |= 1u << pos;
+                }
+                p += 32;
+                if (p >= e[q] || __shfl_sync(full, y[q], 31) > cmax) break;
+                y[q] = p + lane < e[q] ? adj[p + lane] : kNone;
+            }
+            bits = __reduce_or_sync(full, bits);
+            if (lane == 0) rows[i] = bits;
+        }
+    }
+    if (lane == 0) rows[m] = 0;
+    __syncwarp();
+}
+
+// Triangles of G[C], 32 < nc <= kBatchWarpRows, by one warp: the total; each
+// candidate's count in warp_counts64(buf).  C is buf's start.
+__device__ unsigned long long warp_triangles(const uint32_t* C, uint32_t nc, const uint32_t* off,
+                                             const uint32_t* adj, const uint32_t* nb,
+                                             uint32_t* buf) {
+    const unsigned lane = lane_id();
+    unsigned long long* c64 = warp_counts64(buf);
+    uint32_t* rows = buf + 3 * kBatchWarpRows;
+    const uint32_t W = (nc + 31) >> 5, Ws = row_stride(W);
+    for (uint32_t i = lane; i < nc; i += 32) c64[i] = 0;
+    for (uint32_t i = lane; i < nc * Ws; i += 32) rows[i] = 0;
+    __syncwarp();
+    const uint32_t cmax = C[nc - 1];
+    for (uint32_t i = 0; i + 1 < nc; i++) {
+        const uint32_t x = C[i];
+        const uint32_t b = nb[x], e = off[x + 1];
+        for (uint32_t p0 = b; p0 < e; p0 += 32) {
+            const uint32_t p = p0 + lane;
+            const uint32_t y = p < e ? adj[p] : kNone;
+            if (y <= cmax) {
+                const uint32_t pos = (uint32_t)lower_bound_u32(C, nc, y);
+                if (pos < nc && C[pos] == y) {
+                    atomicOr(&rows[i * Ws + (pos >> 5)], 1u << (pos & 31));
+                    atomicOr(&rows[pos * Ws + (i >> 5)], 1u << (i & 31));
+                }
+            }
+        }
+    }
+    __syncwarp();
+    BitmapWarp B;
+    B.rows = rows;
+    B.W = W;
+    B.Ws = Ws;
+    B.cnt = c64;
+    B.sP = rows + kBatchWarpRows * row_stride(4);
+    B.list = reinterpret_cast<uint16_t*>(B.sP + kRowStrideMax);
+    B.small = true;
+    B.nd = nc;
+    unsigned long long total = 0;
+    for (uint32_t i = 0; i + 2 < nc; i++) {
+        uint32_t P = B.row_word(i);
+        const uint32_t iw = i >> 5;
+        if (lane < iw) P = 0;
+        else if (lane == iw) P &= (i & 31u) == 31u ? 0u : 0xffffffffu << ((i & 31u) + 1u);
+        const unsigned long long c = warp_edges(B, P);
+        if (c && lane == 0) B.credit(i, c);
+        total += c;
+    }
+    __syncwarp();
+    return total;
+}
+
 // ------------------------------------------------------------ the kernel
 // LPR: lanes per row scan (the intersection tile; 32 / LPR rows at once per
 // warp in the triangle listing and the h = 4 edge counts).
 template <int NT, int LPR>
 __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
     constexpr int NW = NT / 32;
-    extern __shared__ uint8_t smem_raw[];
+    extern __shared__ __align__(16) uint8_t smem_raw[];
     Smem<NT>& S = *reinterpret_cast<Smem<NT>*>(smem_raw);
     __shared__ uint32_t s_gi;
     const unsigned lane = lane_id(), wid = warp_id();
@@ -547,22 +737,19 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
             __syncthreads();
             continue;
         }
-        // ---- CSR: keys u*n+v for both orientations, loops dropped
-        if (threadIdx.x == 0) {
-            S.cnt1 = 0;
-            S.flag = 0;
-        }
+        // ---- CSR: endpoint counts, scatter, rows sorted, repeats dropped
+        if (threadIdx.x == 0) S.flag = 0;
+        for (uint32_t v = threadIdx.x; v < n; v += NT) W.fa[v] = 0;
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < D.m; e += NT) {
-            uint32_t u = A.src[D.e_off + e], v = A.dst[D.e_off + e];
+            const uint32_t u = A.src[D.e_off + e], v = A.dst[D.e_off + e];
             if (u >= n || v >= n) {
                 S.flag = 1;
                 continue;
             }
             if (u == v) continue;
-            uint32_t at = atomicAdd(&S.cnt1, 2u);
-            W.k1[at] = u * n + v;
-            W.k1[at + 1] = v * n + u;
+            atomicAdd(&W.fa[u], 1u);
+            atomicAdd(&W.fa[v], 1u);
         }
         __syncthreads();
         if (S.flag) {
@@ -573,10 +760,23 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
             __syncthreads();
             continue;
         }
-        const uint32_t nkeys = S.cnt1;
-        const int kb = key_bits((uint64_t)n * n - 1);
-        block_radix_sort<NT>(W.k1, W.k2, nkeys, kb, S);
-        const uint32_t E = keys_to_csr<NT>(W.k1, nkeys, n, W.off, W.adj, S);
+        (void)block_prefix<NT>(W.fa, n, W.roff, S);
+        for (uint32_t v = threadIdx.x; v < n; v += NT) W.fa[v] = 0;
+        __syncthreads();
+        for (uint32_t e = threadIdx.x; e < D.m; e += NT) {
+            const uint32_t u = A.src[D.e_off + e], v = A.dst[D.e_off + e];
+            if (u == v) continue;
+            W.k1[W.roff[u] + atomicAdd(&W.fa[u], 1u)] = v;
+            W.k1[W.roff[v] + atomicAdd(&W.fa[v], 1u)] = u;
+        }
+        __syncthreads();
+        block_sort_rows<NT>(W.k1, W.k2, W.roff, W.fa, n, W.fb, S);
+        const uint32_t E = block_prefix<NT>(W.fa, n, W.off, S);
+        for (uint32_t v = wid; v < n; v += NW) {
+            const uint32_t from = W.roff[v], to = W.off[v], l = W.off[v + 1] - to;
+            for (uint32_t j = lane; j < l; j += 32) W.adj[to + j] = W.k1[from + j];
+        }
+        __syncthreads();
         R.m_clean = E / 2;
         // ---- degeneracy peel (the h = 2 decomposition)
         for (uint32_t v = threadIdx.x; v < n; v += NT) W.deg[v] = W.off[v + 1] - W.off[v];
@@ -613,13 +813,18 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
                 W.new_of[o] = i;
             }
             __syncthreads();
-            for (uint32_t v = threadIdx.x; v < n; v += NT) {
-                uint32_t nv = W.new_of[v];
-                for (uint32_t p = W.off[v]; p < W.off[v + 1]; p++) W.k1[p] = nv * n + W.new_of[W.adj[p]];
+            for (uint32_t i = threadIdx.x; i < n; i += NT) {
+                const uint32_t o = W.old_of[i];
+                W.fa[i] = W.off[o + 1] - W.off[o];
             }
             __syncthreads();
-            block_radix_sort<NT>(W.k1, W.k2, E, kb, S);
-            keys_to_csr<NT>(W.k1, E, n, W.roff, W.radj, S);
+            (void)block_prefix<NT>(W.fa, n, W.roff, S);
+            for (uint32_t i = wid; i < n; i += NW) {
+                const uint32_t from = W.off[W.old_of[i]], to = W.roff[i], l = W.roff[i + 1] - to;
+                for (uint32_t j = lane; j < l; j += 32) W.radj[to + j] = W.new_of[W.adj[from + j]];
+            }
+            __syncthreads();
+            block_sort_rows<NT>(W.radj, W.k1, W.roff, W.fa, n, W.fb, S);
             // N+(v): first entry above v; largest out-degree
             if (threadIdx.x == 0) S.cnt2 = 0;
             __syncthreads();
@@ -676,10 +881,14 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
                         tot = warp_sum(mine);
                     } else if (d <= 32) {
                         // h = 4: triangles of G[C] by the one-word bitmap DFS
-                        warp_build_rows32(C, d, W.roff + 1, W.radj, W.rsplit, rows);
+                        warp_rows32_ahead(C, d, W.roff, W.radj, W.rsplit, rows);
                         tot = warp_dfs32(rows, d, 3, cnt);
+                    } else if (d <= kBatchWarpRows) {
+                        // h = 4, |C| <= 128: symmetric rows of at most four
+                        // words and the edges of each upper row (cliques.cuh)
+                        tot = warp_triangles(C, d, W.roff, W.radj, W.rsplit, S.wbuf[wid]);
                     } else {
-                        // h = 4, |C| > 32: every edge (x, y) of G[C] with x < y,
+                        // h = 4, larger |C|: every edge (x, y) of G[C] with x < y,
                         // and each common higher neighbour z of x and y in C
                         for (uint32_t i = 0; i < d; i++) {
                             uint32_t x = C[i];
@@ -707,7 +916,11 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
                         }
                     }
                     __syncwarp();
-                    if (tot)
+                    if (tot && D.h == 4 && d > 32 && d <= kBatchWarpRows) {
+                        const unsigned long long* c64 = warp_counts64(S.wbuf[wid]);
+                        for (uint32_t i = lane; i < d; i += 32)
+                            if (c64[i]) atomicAdd(&W.deg[C[i]], c64[i]);
+                    } else if (tot)
                         for (uint32_t i = lane; i < d; i += 32)
                             if (cnt[i]) atomicAdd(&W.deg[C[i]], (unsigned long long)cnt[i]);
                     if (lane == 0 && tot) {

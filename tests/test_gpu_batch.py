@@ -185,3 +185,38 @@ def test_batch_wide_h4_graph_falls_back(L, orc):
     for x, y in zip(again, res):
         assert x["kmax"] == y["kmax"] and np.array_equal(x["core"], y["core"])
     b.close()
+
+
+def _clique(k, n, seed):
+    """K_k on random vertices of a sparse n-vertex graph."""
+    n, s, d = gg.er(n, 2.0 / n, seed)
+    return gg.plant(n, s, d, k, 1.0, seed + 1)[:3]
+
+
+def _hub(deg, seed):
+    """A hub of `deg` neighbours, every hub edge listed twice."""
+    rng = np.random.default_rng(seed)
+    ring = np.arange(1, deg + 1, dtype=np.uint32)
+    s = np.concatenate([np.zeros(deg), ring, rng.integers(0, deg + 1, 3 * deg)]).astype(np.uint32)
+    d = np.concatenate([ring, np.zeros(deg), rng.integers(0, deg + 1, 3 * deg)]).astype(np.uint32)
+    return deg + 1, s, d
+
+
+def test_batch_row_and_set_sizes(L, orc):
+    """Row lengths around the batch kernel's sort tiers (32, 512 entries before
+    repeats go) and h = 4 candidate sets around its row tiers (32, 128)."""
+    graphs = [(*_clique(k, 300, k), 4) for k in (32, 33, 34, 128, 129, 130, 140)]
+    graphs += [(*_hub(deg, deg), h) for deg in (16, 17, 255, 256, 257, 900) for h in (2, 3, 4)]
+    b = L.Batch(graphs, want_cores=True)
+    try:
+        b.run()
+        rs = b.results()
+    finally:
+        b.close()
+    for (n, s, d, h), r in zip(graphs, rs):
+        og = orc.csr(n, s, d)
+        core, k = orc.core_decompose(og, h)
+        w = orc.core_app(og, h, core, k)
+        assert r["status"] == 0 and r["kmax"] == k, (n, h)
+        assert np.array_equal(r["core"], core), (n, h)
+        assert r["densest_mu"] == w["densest_mu"] and r["densest_size"] == w["densest_size"]
