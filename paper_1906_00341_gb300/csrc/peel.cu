@@ -1295,16 +1295,16 @@ __device__ __forceinline__ void process_bands(
                 }
             }
         } else if (HC == 3) {
-            // a warp looks at `cs` consecutive items at once, one a lane, and
-            // takes the pairs among them one by one: most items name a
-            // vertex of a later band and need nothing more
-            uint32_t cs = 1;
-            while (cs < 32 && (uint64_t)cs * gwarps < T) cs <<= 1;
-            for (uint64_t t0 = gwarp * cs; t0 < T; t0 += gwarps * cs) {
-                const uint64_t t = t0 + lane;
+            // a warp looks at up to 32 items at once, one a lane, and takes the
+            // pairs among them one by one: most items name a vertex of a
+            // later band and need nothing more.  A lane's items lie gwarps
+            // apart: members of one band are neighbours in a row, and taken
+            // in runs they fell to a few warps
+            for (uint64_t t0 = gwarp; t0 < T; t0 += gwarps * 32) {
+                const uint64_t t = t0 + lane * gwarps;
                 uint32_t v = 0, u = 0, kv = 0;
                 bool dec = false;
-                if (lane < cs && t < T) {
+                if (t < T) {
                     const uint32_t i = at(t);
                     v = H[i];
                     u = P.wadj[P.off[v] + (t - s_pre[i])];
