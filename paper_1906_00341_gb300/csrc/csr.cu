@@ -2,6 +2,7 @@
 // unweighted, simple).  Counting pass, exclusive scan, scatter by atomic
 // cursors, per-row sort + unique, scan of the unique counts, row copy.
 #include "graph.cuh"
+#include "tiny.cuh"
 
 namespace dsd {
 namespace {
@@ -76,6 +77,11 @@ dsd_status build_csr(dsd_graph* g, uint64_t m, const uint32_t* src, const uint32
     if ((m >> 31) != 0) {
         set_error("edge lists of 2^31 or more entries are not supported by this library");
         return DSD_ERR_UNSUPPORTED;
+    }
+    if (n && n <= kTinyN && m <= kTinyM) {
+        bool done = false;
+        DSD_TRY(tiny_csr(g, (uint32_t)m, src, dst, &done));
+        if (done) return DSD_OK;
     }
     uint32_t* cnt = nullptr;      // [n] endpoint counts, then cursors
     uint32_t* err = nullptr;

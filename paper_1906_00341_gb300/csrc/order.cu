@@ -12,6 +12,7 @@
 // The second stage relabels vertices by rank and rebuilds the CSR with sorted rows, so that
 // N+(v) = {u in N(v) : u > v} is the tail of row v (start kept in rsplit).
 #include "graph.cuh"
+#include "tiny.cuh"
 
 #include <vector>
 
@@ -160,6 +161,14 @@ dsd_status ensure_order(dsd_graph* g) {
     g->prof_bytes[kPhaseOrderPeel] = pr.bytes;
     record_peel(g, 0, pr);
     R = pr.rounds + 1;
+    if (n <= kTinyN && g->m <= kTinyM) {
+        prof_begin(g, kPhaseOrient);
+        STEP(tiny_orient(g));
+        prof_end(g, kPhaseOrient);
+        g->prof_launches[kPhaseOrient] = 1;
+        g->ordered = true;
+        goto done;
+    }
 
     // rank by (round, id), relabel, rebuild rows
     prof_begin(g, kPhaseOrient);

@@ -129,3 +129,44 @@ def test_star_bands(L, graph, x):
         assert r[1] == got[0][1]
         for a, b in zip(r, got[0]):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("case", ["n3072", "n3073", "m16384", "m16385", "row256", "row257",
+                                  "row3000", "repeats", "bad"])
+def test_one_block_csr(L, orc, case):
+    """The one-block CSR build and orientation on both sides of their limits, a
+    row beyond the block's buffer through repeats, and a bad endpoint."""
+    rng = np.random.default_rng(7)
+    if case[0] == "n":
+        n, m = int(case[1:]), 12000
+        s, d = rng.integers(0, n, m), rng.integers(0, n, m)
+    elif case[0] == "m":
+        n, m = 3000, int(case[1:])
+        s, d = rng.integers(0, n, m), rng.integers(0, n, m)
+    elif case == "repeats":
+        n, m = 300, 16000
+        s, d = np.zeros(m, np.int64), rng.integers(0, n, m)
+    elif case == "bad":
+        with pytest.raises(L.DSDError) as ei:
+            L.Graph.from_edges(100, np.array([0, 5, 100], np.uint32),
+                               np.array([1, 6, 2], np.uint32))
+        assert ei.value.name == "DSD_ERR_INVALID"
+        return
+    else:
+        k = int(case[3:])
+        n = k + 50
+        s = np.concatenate([np.zeros(k, np.int64), rng.integers(0, n, 2 * k)])
+        d = np.concatenate([np.arange(1, k + 1), rng.integers(0, n, 2 * k)])
+    s, d = s.astype(np.uint32), d.astype(np.uint32)
+    og = orc.csr(n, s, d)
+    core, rnd = rounds_of(n, s, d)
+    rank = np.empty(n, np.int64)
+    rank[np.lexsort((np.arange(n), rnd))] = np.arange(n)
+    with L.Graph.from_edges(n, s, d) as g:
+        off, adj = g.csr()
+        c2, rk, _ = g.degeneracy_order()
+        deg, mu = g.clique_degrees(3)
+    assert np.array_equal(off, og.off) and np.array_equal(adj, og.adj)
+    assert np.array_equal(c2, core) and np.array_equal(rk, rank)
+    wdeg, wmu = orc.clique_degrees(og, 3)
+    assert mu == wmu and np.array_equal(deg, wdeg)
