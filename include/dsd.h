@@ -81,6 +81,11 @@ const char* dsd_version(void);
  * launches inside it. */
 uint64_t dsd_kernel_launches(void);
 
+/* Device memory comes from a pool of the library's own on each device, which
+ * keeps at most 2 GiB of freed memory for later calls.  This gives what is
+ * unused at the time back to the device (the current one).  DSD_ERR_CUDA. */
+dsd_status dsd_release_memory(void);
+
 /* Upper bound, in milliseconds, on every inter-block wait inside a
  * persistent kernel (grid barriers).  A wait that runs out makes the kernel
  * record the fault, leave its loop, and the call return DSD_ERR_TIMEOUT.

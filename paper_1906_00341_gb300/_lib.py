@@ -86,6 +86,7 @@ SIGNATURES = {
     "dsd_last_error": (ctypes.c_char_p, []),
     "dsd_version": (ctypes.c_char_p, []),
     "dsd_kernel_launches": (ctypes.c_uint64, []),
+    "dsd_release_memory": (_int, []),
     "dsd_set_wait_limit_ms": (_int, [_u32]),
     "dsd_set_peel_small_limit": (_int, [_u32]),
     "dsd_set_peel_tail_limit": (_int, [_u32]),
@@ -188,6 +189,10 @@ def dsd_version():
 
 def dsd_kernel_launches():
     return int(load().dsd_kernel_launches())
+
+
+def dsd_release_memory():
+    _check(load().dsd_release_memory())
 
 
 def dsd_set_wait_limit_ms(ms):

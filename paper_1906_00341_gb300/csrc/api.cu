@@ -386,6 +386,11 @@ dsd_status dsd_set_peel_items(uint32_t warp_max, uint32_t mid_max) {
     return DSD_OK;
 }
 
+dsd_status dsd_release_memory(void) {
+    set_error("");
+    return release_memory();
+}
+
 dsd_status dsd_set_checked(int on) {
     g_checked = on ? 1 : 0;
     return DSD_OK;

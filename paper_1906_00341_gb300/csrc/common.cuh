@@ -29,13 +29,14 @@ dsd_status cuda_fail(cudaError_t e, const char* what, const char* file, int line
 #define DSD_LAUNCHED() DSD_CU(cudaGetLastError())
 
 // ------------------------------------------------------- device memory
-// Stream-ordered allocations from the device's default memory pool.
+// Stream-ordered allocations from the library's memory pool of the device.
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
 };
 dsd_status dev_alloc(void** p, size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);
+dsd_status release_memory();   // unused memory of the current device's pool
 
 template <class T>
 inline dsd_status dalloc(T** p, size_t count, cudaStream_t s) {

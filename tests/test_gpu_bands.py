@@ -170,3 +170,19 @@ def test_one_block_csr(L, orc, case):
     assert np.array_equal(c2, core) and np.array_equal(rk, rank)
     wdeg, wmu = orc.clique_degrees(og, 3)
     assert mu == wmu and np.array_equal(deg, wdeg)
+
+
+def test_release_memory(L):
+    """The library's pool keeps at most 2 GiB and gives it back on request."""
+    import torch
+    L.dsd_release_memory()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    n, s, d = gg.er(200_000, 0.0002, 3)
+    for _ in range(2):
+        with L.Graph.from_edges(n, s, d) as g:
+            g.core_app(3)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] >= free0 - (2 << 30) - (64 << 20)
+    L.dsd_release_memory()
+    assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)
