@@ -66,8 +66,10 @@ struct AppParams {
     const uint64_t* snap;     // count of v in R_core(v) (rank space)
     const uint32_t* posof;    // rank -> position (levels ascending, caller id inside)
     const uint32_t* rank_at;  // position -> rank
-    unsigned long long* deg;  // by position: current count in the level's process
-    uint32_t* step;           // by position: removal step inside its level (kNoStep alive)
+    unsigned long long* deg;  // by rank: current count in the level's process
+    uint32_t* step;           // by rank: removal step inside its level (kNoStep alive)
+    const uint64_t* rb;       // by position: row start and end
+    const uint64_t* re;
     const uint64_t* lk;       // level records (k ascending, |R_k|, mu(R_k))
     const uint32_t* ls;
     const uint64_t* lm;
@@ -131,21 +133,81 @@ __device__ __forceinline__ bool ratio_gt(unsigned long long a, unsigned long lon
 // x lies in the current set S of level k: above the level, or an alive
 // member of it.
 __device__ __forceinline__ bool in_set(const AppParams& P, uint32_t x, unsigned long long k) {
-    unsigned long long c = P.core[x];
-    return c > k || (c == k && P.step[P.posof[x]] == kNoStep);
+    const unsigned long long c = P.core[x];
+    const uint32_t s = P.step[x];   // independent loads
+    return c > k || (c == k && s == kNoStep);
 }
 
+// An alive member x of the level loses c cliques.
+__device__ __forceinline__ void lower_member(const AppParams& P, const AppQ& Q, uint32_t x,
+                                             unsigned long long c) {
+    const uint32_t p = Q.B ? P.posof[x] - Q.base : 0u;
+    const unsigned long long old = atomicAdd(&P.deg[x], 0ull - c);
+    if (Q.B) {
+        Q.toggle(old, p);
+        Q.toggle(old - c, p);
+    }
+}
 __device__ __forceinline__ void lower(const AppParams& P, const AppQ& Q, uint32_t x,
                                       unsigned long long k, unsigned long long c) {
-    if (c && P.core[x] == k) {
-        uint32_t p = P.posof[x];
-        if (P.step[p] == kNoStep) {
-            unsigned long long old = atomicAdd(&P.deg[p], 0ull - c);
-            if (Q.B) {
-                Q.toggle(old, p - Q.base);
-                Q.toggle(old - c, p - Q.base);
+    if (!c) return;
+    const unsigned long long cx = P.core[x];
+    const uint32_t s = P.step[x];
+    if (cx == k && s == kNoStep) lower_member(P, Q, x, c);
+}
+
+// h = 3, a row of at most kAppRow entries: the triangles of S through the
+// removed vertex v (row adj[vb, vb + len)).  A step is a chain of dependent
+// loads, some twenty of them when every entry of every N+(w) was tested for
+// membership in S and searched for in v's row in L2; here the row, its
+// members' states and the bounds of their N+ lists come in two rounds of
+// independent loads, the lists are searched for in shared memory, and each
+// partner is lowered once.
+constexpr uint32_t kAppRow = 2048;
+struct AppRow {
+    uint32_t x[kAppRow];     // the row
+    uint32_t b[kAppRow];     // where N+(x) begins (2m < 2^32)
+    uint32_t len[kAppRow];   // and its length; 0 for x outside S
+    uint32_t cnt[kAppRow];   // triangles with v; bit 31: alive in the level, 30: in S
+};
+template <int NT>
+__device__ void app_row3(const AppParams& P, const AppQ& Q, uint64_t vb, uint32_t len,
+                         unsigned long long k, AppRow& R) {
+    constexpr uint32_t kMember = 1u << 31, kIn = 1u << 30, kCount = kIn - 1u;
+    const unsigned lane = lane_id(), wid = warp_id();
+    for (uint32_t i = threadIdx.x; i < len; i += NT) {
+        const uint32_t x = P.adj[vb + i];
+        const unsigned long long c = P.core[x];
+        const uint32_t s = P.step[x];
+        const uint64_t b = P.split[x], e = P.off[x + 1];
+        const bool member = c == k && s == kNoStep, in = c > k || member;
+        R.x[i] = x;
+        R.b[i] = (uint32_t)b;
+        R.len[i] = in ? (uint32_t)(e - b) : 0u;
+        R.cnt[i] = (in ? kIn : 0u) | (member ? kMember : 0u);
+    }
+    __syncthreads();
+    const uint32_t xmax = len ? R.x[len - 1] : 0u;
+    for (uint32_t i = wid; i < len; i += NT / 32) {
+        const uint32_t l = R.len[i], b = R.b[i];
+        uint32_t hits = 0;
+        for (uint32_t p = lane; p - lane < l; p += 32) {
+            const uint32_t y = p < l ? P.adj[(uint64_t)b + p] : kNone;
+            bool hit = false;
+            if (y <= xmax) {
+                const uint32_t pos = (uint32_t)lower_bound_u32(R.x, len, y);
+                hit = pos < len && R.x[pos] == y && (R.cnt[pos] & kIn);
+                if (hit) atomicAdd(&R.cnt[pos], 1u);
             }
+            hits += __popc(__ballot_sync(0xffffffffu, hit));
+            if (__shfl_sync(0xffffffffu, y, 31) > xmax) break;
         }
+        if (lane == 0 && hits) atomicAdd(&R.cnt[i], hits);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < len; i += NT) {
+        const uint32_t c = R.cnt[i];
+        if ((c & kMember) && (c & kCount)) lower_member(P, Q, R.x[i], c & kCount);
     }
 }
 
@@ -367,6 +429,7 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
     __shared__ unsigned long long s_kd[NW];
     __shared__ uint32_t s_kp[NW];
     __shared__ uint32_t s_lv, s_pick, s_nbig, s_it;
+    __shared__ unsigned long long s_sum;
     const unsigned lane = lane_id(), wid = warp_id();
     uint32_t* wC = smem + (size_t)wid * 3 * kAppWarpCand;
     unsigned* wCnt = wC + kAppWarpCand;
@@ -389,7 +452,7 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
         if (k == 0) {
             // no cliques here: removal in id order, no count changes; the
             // density only grows as the set shrinks
-            for (uint32_t i = threadIdx.x; i < sz; i += NT) P.step[base + i] = i;
+            for (uint32_t i = threadIdx.x; i < sz; i += NT) P.step[P.rank_at[base + i]] = i;
             if (threadIdx.x == 0) {
                 uint32_t bs = mu ? sz - 1 : 0;
                 P.best[j] = make_ulonglong2(mu, ((unsigned long long)(size0 - bs) << 32) | bs);
@@ -416,9 +479,10 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
             __syncthreads();
         }
         for (uint32_t i = threadIdx.x; i < sz; i += NT) {
-            const unsigned long long d = P.snap[P.rank_at[base + i]];
-            P.deg[base + i] = d;
-            P.step[base + i] = kNoStep;
+            const uint32_t r = P.rank_at[base + i];
+            const unsigned long long d = P.snap[r];
+            P.deg[r] = d;
+            P.step[r] = kNoStep;
             Q.toggle(d, i);
         }
         unsigned long long bmu = mu;
@@ -438,10 +502,38 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
                         pick = kPickDone;
                         break;
                     }
+                    uint32_t* word = &Q.M[(size_t)b * Q.n1 + (i >> 5)];
+                    if (b == 0) {
+                        // every member of this word, in position order; the
+                        // density rises with each removal (mu stays), so the
+                        // set before the last of them stands for all
+                        uint32_t w = lane == 0 ? *word : 0u;
+                        w = __shfl_sync(0xffffffffu, w, 0);
+                        const uint32_t z = __popc(w);
+                        if ((w >> lane) & 1u)
+                            P.step[P.rank_at[base + (i & ~31u) + lane]] =
+                                it + __popc(w & ((1u << lane) - 1u));
+                        const uint32_t last = it + z - 1;
+                        if (lane == 0) {
+                            *word = 0;
+                            Q.pop[0] -= z;
+                            if (last > 0 && ratio_gt(mu, size0 - last, bmu, bsize)) {
+                                bmu = mu;
+                                bsize = size0 - last;
+                                bstep = last;
+                            }
+                        }
+                        it += z;
+                        __syncwarp();
+                        if (it == sz) {
+                            pick = kPickDone;
+                            break;
+                        }
+                        continue;
+                    }
                     if (lane == 0) {
-                        Q.M[(size_t)b * Q.n1 + (i >> 5)] &= ~(1u << (i & 31u));
+                        *word &= ~(1u << (i & 31u));
                         Q.pop[b] -= 1u;
-                        if (P.deg[base + i] != b) atomicOr(P.err, 2u);
                         // the set before this removal: size0 - it vertices, mu cliques
                         if (it > 0 && ratio_gt(mu, size0 - it, bmu, bsize)) {
                             bmu = mu;
@@ -449,18 +541,11 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
                             bstep = it;
                         }
                         mu -= b;
-                        P.step[base + i] = it;
                     }
                     it++;
                     __syncwarp();
-                    if (b != 0) {
-                        pick = i;
-                        break;
-                    }
-                    if (it == sz) {
-                        pick = kPickDone;
-                        break;
-                    }
+                    pick = i;
+                    break;
                 }
                 if (lane == 0) {
                     s_pick = pick;
@@ -476,8 +561,9 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
                 unsigned long long md = ~0ull;
                 uint32_t mp = 0xffffffffu;
                 for (uint32_t i = threadIdx.x; i < sz; i += NT) {
-                    if (P.step[base + i] != kNoStep) continue;
-                    unsigned long long d = P.deg[base + i];
+                    const uint32_t r = P.rank_at[base + i];
+                    if (P.step[r] != kNoStep) continue;
+                    unsigned long long d = P.deg[r];
                     if (d < md) { md = d; mp = i; }   // i ascends: ties keep the first
                 }
 #pragma unroll
@@ -503,7 +589,6 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
                         bstep = it;
                     }
                     mu -= bd;
-                    P.step[base + bp] = it;
                     s_pick = bp;
                     s_it = it + 1;
                 }
@@ -513,8 +598,12 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
             }
             // ---- the cliques through the removed vertex lower its partners
             const uint32_t v = P.rank_at[base + pick];
-            const uint64_t vb = P.off[v], ve = P.off[v + 1];
-            if (P.h == 2) {
+            const uint64_t vb = P.rb[base + pick], ve = P.re[base + pick];
+            if (threadIdx.x == 0) P.step[v] = s_it - 1;   // no row holds v itself
+            if (P.h == 3 && ve - vb <= kAppRow) {
+                app_row3<NT>(P, Q, vb, (uint32_t)(ve - vb), k,
+                             *reinterpret_cast<AppRow*>(smem));
+            } else if (P.h == 2) {
                 for (uint64_t p = vb + threadIdx.x; p < ve; p += NT)
                     lower(P, Q, P.adj[p], k, 1ull);
             } else {
@@ -534,8 +623,22 @@ __global__ void __launch_bounds__(NT) k_peel_app(AppParams P) {
             __syncthreads();
             if (s_it >= sz) break;
         }
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
             P.best[j] = make_ulonglong2(bmu, ((unsigned long long)bsize << 32) | bstep);
+            s_sum = 0;
+        }
+        __syncthreads();
+        // the counts the members left with (no longer lowered then) are the
+        // cliques between this level's set and the next one's
+        unsigned long long sum = 0;
+        for (uint32_t i = threadIdx.x; i < sz; i += NT) sum += P.deg[P.rank_at[base + i]];
+        sum = warp_sum(sum);
+        if (lane == 0 && sum) atomicAdd(&s_sum, sum);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned long long after = j + 1 < P.nl ? P.lm[j + 1] : 0ull;
+            if (P.lm[j] - s_sum != after || mu != after) atomicOr(P.err, 2u);
+        }
         __syncthreads();
     }
 }
@@ -568,12 +671,15 @@ __global__ void k_app_place(uint32_t n, const uint32_t* lev, const uint32_t* ls,
 }
 
 __global__ void k_app_maps(uint32_t n, const uint32_t* ids, const uint32_t* new_of,
-                           uint32_t* rank_at, uint32_t* posof) {
+                           const uint64_t* off, uint32_t* rank_at, uint32_t* posof, uint64_t* rb,
+                           uint64_t* re) {
     for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (uint64_t)gridDim.x * blockDim.x) {
         uint32_t r = new_of[ids[p]];
         rank_at[p] = r;
         posof[r] = (uint32_t)p;
+        rb[p] = off[r];
+        re[p] = off[r + 1];
     }
 }
 
@@ -608,8 +714,9 @@ __global__ void k_app_emit(uint32_t n, const uint32_t* ids, const uint32_t* rank
          p += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t r = rank_at[p], o = ids[p];
         const unsigned long long c = core[r];
-        flag[o] = (c > kb || (c == kb && step[p] >= bstep)) ? 1u : 0u;
-        if (order) order[n - ls[lev[r]] + step[p]] = o;
+        const uint32_t st = step[r];
+        flag[o] = (c > kb || (c == kb && st >= bstep)) ? 1u : 0u;
+        if (order) order[n - ls[lev[r]] + st] = o;
     }
 }
 
@@ -668,6 +775,7 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
     uint64_t* lpos = nullptr;
     ulonglong2 *best = nullptr, *pick = nullptr;
     unsigned long long* pdeg = nullptr;
+    uint64_t* rowse = nullptr;   // row starts and ends by position
     unsigned long long mu = 0;
     dsd_status st = DSD_OK;
     cudaError_t e = cudaSuccess;
@@ -715,6 +823,7 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
     APP_TRY(dalloc(&lpos, (size_t)nl + 1, s));
     APP_TRY(dalloc(&rank_at, (size_t)n + 1, s));
     APP_TRY(dalloc(&posof, (size_t)n + 1, s));
+    APP_TRY(dalloc(&rowse, (size_t)2 * n + 2, s));
     APP_CU(cudaMemsetAsync(cur, 0, (size_t)nl * 4, s));
     k_app_levels<<<app_grid(n), 256, 0, s>>>(n, core, lk, nl, lev); note_launch();
     k_app_place<<<app_grid(n), 256, 0, s>>>(n, lev, ls, nl, g->old_of, cur, ids); note_launch();
@@ -741,7 +850,8 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
         APP_TRY(segmented_sort_unique(ids, tmp, lpos, lenv, newlen, nl, n, s));
         APP_CU(cudaStreamSynchronize(s));   // host vectors leave scope
     }
-    k_app_maps<<<app_grid(n), 256, 0, s>>>(n, ids, g->new_of, rank_at, posof); note_launch();
+    k_app_maps<<<app_grid(n), 256, 0, s>>>(n, ids, g->new_of, g->roff, rank_at, posof, rowse,
+                                           rowse + n); note_launch();
     APP_CU(cudaGetLastError());
     // ---- the per-level processes
     {
@@ -768,11 +878,14 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
         APP_TRY(dalloc(&best, (size_t)nl + 1, s));
         APP_TRY(dalloc(&pick, 2, s));
         P.deg = pdeg;
+        P.rb = rowse;
+        P.re = rowse + n;
         P.step = stepv;
         P.queue = stepv + n;
         P.lorder = lorder;
         P.best = best;
         size_t words = (size_t)(kAppNT / 32) * 3 * kAppWarpCand;
+        if (h == 3) words = std::max(words, sizeof(AppRow) / 4);
         if (h >= 4) {
             // (cap > kBitmapMax: the split search uses the full-size layout)
             size_t big = bitmap_words(P.bcap, kAppNT / 32);
@@ -907,7 +1020,7 @@ extern "C" dsd_status dsd_peel_app(dsd_graph* g, int h, uint32_t* densest, uint3
 done:
     for (void* p : {(void*)deg, (void*)core, (void*)snap, (void*)lk, (void*)ls, (void*)lm,
                     (void*)lev, (void*)cur, (void*)ids, (void*)tmp, (void*)lenv, (void*)newlen,
-                    (void*)lpos, (void*)rank_at, (void*)posof, (void*)pdeg, (void*)stepv,
+                    (void*)lpos, (void*)rank_at, (void*)posof, (void*)pdeg, (void*)stepv, (void*)rowse,
                     (void*)best, (void*)pick, (void*)lorder, (void*)bigw, (void*)flag,
                     (void*)pos, (void*)obuf, (void*)qBv, (void*)qoffv, (void*)qg, (void*)xl})
         dev_free(p, s);
