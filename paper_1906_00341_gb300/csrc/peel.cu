@@ -34,8 +34,8 @@
 //        belongs to the lowest band among its members, and only members in
 //        that band count it.
 // The 1M-vertex graph, h = 3: 7,016 rounds one level at a time (86 ms), 587
-// in the two phases (41 ms); R-MAT scale 17, h = 4: 8,232 and 428 (389 ms and
-// 114 ms).  Bound by the latency of a round (barriers, row walks) and by the
+// in the two phases (29 ms); R-MAT scale 17, h = 4: 8,232 and 428 (389 ms and
+// 22 ms).  Bound by the latency of a round (barriers, row walks) and by the
 // blocks that wait for the longest items of it.
 //
 // One persistent cooperative kernel runs every round; phases are separated

@@ -162,7 +162,9 @@ __device__ __forceinline__ void lower(const AppParams& P, const AppQ& Q, uint32_
 // membership in S and searched for in v's row in L2; here the row, its
 // members' states and the bounds of their N+ lists come in two rounds of
 // independent loads, the lists are searched for in shared memory, and each
-// partner is lowered once.
+// partner is lowered once (50,000 vertices of a power law: the call 31.4 ->
+// 28.0 ms).  Bound by the steps of the first level, one after another at some
+// 3.5 us.
 constexpr uint32_t kAppRow = 2048;
 struct AppRow {
     uint32_t x[kAppRow];     // the row
