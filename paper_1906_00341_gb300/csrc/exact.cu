@@ -454,10 +454,12 @@ __global__ void k_preflow(uint32_t nW, const uint64_t* head, const uint64_t* rev
 
 // Frontier lists: small nodes (warp each) and big nodes (block each); the
 // counters c[0], c[1] hold their lengths.
-__global__ void k_bfs_init(PR P, uint32_t* fs, uint32_t* fb, uint32_t* c) {
+__global__ void k_bfs_init(PR P, uint32_t* nh, uint32_t* fs, uint32_t* fb, uint32_t* c) {
     for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < P.N;
-         x += (uint64_t)gridDim.x * blockDim.x)
+         x += (uint64_t)gridDim.x * blockDim.x) {
         P.height[x] = x == 1 ? 0u : kUnset;
+        nh[x] = kUnset;   // heights not yet taken are replaced as well
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         bool big = is_big(P, 1);
         (big ? fb : fs)[0] = 1;
@@ -482,27 +484,36 @@ __device__ __forceinline__ void bfs_arc(const PR& P, uint32_t y, uint64_t e, uin
     warp_append(big, x, ob, oc + 1);
 }
 
-__global__ void k_bfs_small(PR P, const uint32_t* fs, const uint32_t* c, uint32_t d,
-                            uint32_t* os, uint32_t* ob, uint32_t* oc) {
-    uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t n = c[0];
-    for (uint64_t i = gw; i < n; i += nw) {
-        uint32_t y = fs[i];
-        const uint64_t end = P.head[y + 1];
-        for (uint64_t p0 = P.head[y]; p0 < end; p0 += 32)
-            bfs_arc(P, y, p0 + lane_id(), end, d, os, ob, oc);
-    }
+// A round's nodes in one launch: the big ones a block each from block 0 up,
+// then the small ones a warp each from the last block down, so that the two
+// kinds overlap; as launches of their own they ran one after the other, the
+// few big nodes of a round leaving most of the GPU idle.  With heights taken
+// over by the collect a round is three launches, not six: the minimum cut of a
+// 300,000-vertex power law, h = 3, 14.4 -> 11.8 ms a call.  Bound by the
+// launches and the host's waits of some hundred rounds and searches.
+__device__ __forceinline__ uint64_t small_warp() {
+    return (uint64_t)(gridDim.x - 1 - blockIdx.x) * (blockDim.x >> 5) + warp_id();
+}
+__device__ __forceinline__ uint64_t small_warps() {
+    return (uint64_t)gridDim.x * (blockDim.x >> 5);
 }
 
-__global__ void k_bfs_big(PR P, const uint32_t* fb, const uint32_t* c, uint32_t d,
-                          uint32_t* os, uint32_t* ob, uint32_t* oc) {
+__global__ void __launch_bounds__(kBigThreads) k_bfs(PR P, const uint32_t* fs, const uint32_t* fb,
+                                                     const uint32_t* c, uint32_t d, uint32_t* os,
+                                                     uint32_t* ob, uint32_t* oc) {
     const uint32_t n = c[1];
     for (uint64_t i = blockIdx.x; i < n; i += gridDim.x) {
         uint32_t y = fb[i];
         const uint64_t end = P.head[y + 1];
         for (uint64_t p0 = P.head[y]; p0 < end; p0 += blockDim.x)
             bfs_arc(P, y, p0 + threadIdx.x, end, d, os, ob, oc);
+    }
+    const uint32_t ns = c[0];
+    for (uint64_t i = small_warp(); i < ns; i += small_warps()) {
+        uint32_t y = fs[i];
+        const uint64_t end = P.head[y + 1];
+        for (uint64_t p0 = P.head[y]; p0 < end; p0 += 32)
+            bfs_arc(P, y, p0 + lane_id(), end, d, os, ob, oc);
     }
 }
 
@@ -515,12 +526,27 @@ __global__ void k_bfs_finish(PR P) {
     }
 }
 
-// Active nodes into the small (c[0]) and big (c[1]) lists.
-__global__ void k_collect(PR P, uint32_t* ls, uint32_t* lb, uint32_t* c) {
+// Relabelled nodes (nh, by node; kUnset: none) take their new height and
+// restart at their first arc; then the active nodes into the small (c[0]) and
+// big (c[1]) lists.  zero: the counters of the next round's lists.
+__global__ void k_collect(PR P, uint32_t* nh, uint32_t* ls, uint32_t* lb, uint32_t* c,
+                          uint32_t* zero) {
+    if (blockIdx.x == 0 && threadIdx.x < 2) zero[threadIdx.x] = 0;
     for (uint64_t x0 = (uint64_t)blockIdx.x * blockDim.x; x0 < P.N;
          x0 += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t x = x0 + threadIdx.x;
-        bool act = x >= 2 && x < P.N && P.excess[x] > 0 && P.height[x] < P.N;
+        bool act = false;
+        if (x >= 2 && x < P.N) {
+            const uint32_t v = nh[x];
+            uint32_t hx = P.height[x];
+            if (v != kUnset) {
+                hx = v;
+                P.height[x] = v;
+                P.cur[x] = P.head[x];
+                nh[x] = kUnset;
+            }
+            act = P.excess[x] > 0 && hx < P.N;
+        }
         bool big = act && is_big(P, (uint32_t)x);
         warp_append(act && !big, (uint32_t)x, ls, c);
         warp_append(big, (uint32_t)x, lb, c + 1);
@@ -551,14 +577,14 @@ __device__ __forceinline__ void push_arc(const PR& P, uint64_t a, uint32_t v,
 // Warp per small active node.  The prefix of the admissible residuals is
 // saturating: a saturated sum leaves the exclusive prefix above any excess
 // (residuals < 2^63, excess < 2^61), so no push is made from it.
-__global__ void k_push_small(PR P, const uint32_t* list, const uint32_t* c) {
-    uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+__device__ __forceinline__ void push_small(const PR& P, const uint32_t* list, uint32_t n) {
+    const uint64_t gw = small_warp(), nw = small_warps();
     unsigned lane = lane_id();
-    const uint32_t n = c[0];
     for (uint64_t i = gw; i < n; i += nw) {
         const uint32_t u = list[i];
-        const unsigned long long e0 = P.excess[u];
+        // one read for the warp: other nodes push to u meanwhile
+        const unsigned long long e0 =
+            __shfl_sync(0xffffffffu, lane == 0 ? atomicAdd(&P.excess[u], 0ull) : 0ull, 0);
         const uint32_t hu = P.height[u];
         const uint64_t end = P.head[u + 1];
         unsigned long long rem = e0;
@@ -586,23 +612,27 @@ __global__ void k_push_small(PR P, const uint32_t* list, const uint32_t* c) {
     }
 }
 
-// Block per big active node (kBigThreads threads).
-__global__ void __launch_bounds__(kBigThreads) k_push_big(PR P, const uint32_t* list,
-                                                          const uint32_t* c) {
+// Block per big active node (kBigThreads threads), then the small ones.
+__global__ void __launch_bounds__(kBigThreads) k_push(PR P, const uint32_t* list,
+                                                      const uint32_t* smalls, const uint32_t* c) {
     constexpr int NW = kBigThreads / 32;
     __shared__ unsigned long long s_w[NW];
-    __shared__ unsigned long long s_cur;
+    __shared__ unsigned long long s_cur, s_e0;
     const unsigned lane = lane_id(), warp = warp_id();
     const uint32_t n = c[1];
     for (uint64_t i = blockIdx.x; i < n; i += gridDim.x) {
         const uint32_t u = list[i];
-        const unsigned long long e0 = P.excess[u];
         const uint32_t hu = P.height[u];
         const uint64_t end = P.head[u + 1];
-        unsigned long long rem = e0;
         uint64_t p0 = P.cur[u];
-        if (threadIdx.x == 0) s_cur = end;
+        // read once for the block: other nodes push to u meanwhile
+        if (threadIdx.x == 0) {
+            s_cur = end;
+            s_e0 = atomicAdd(&P.excess[u], 0ull);
+        }
         __syncthreads();
+        const unsigned long long e0 = s_e0;
+        unsigned long long rem = e0;
         while (p0 < end && rem > 0) {
             uint32_t v;
             const uint64_t a = p0 + threadIdx.x;
@@ -634,22 +664,19 @@ __global__ void __launch_bounds__(kBigThreads) k_push_big(PR P, const uint32_t* 
         }
         __syncthreads();
     }
+    push_small(P, smalls, c[0]);
 }
 
 // New height of a node that holds excess with its current arc at the end:
 // 1 + the least height over its residual arcs (N if none), else kUnset.
-__global__ void k_relabel_small(PR P, const uint32_t* list, const uint32_t* c, uint32_t* nh) {
-    uint64_t gw = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+__device__ __forceinline__ void relabel_small(const PR& P, const uint32_t* list, uint32_t n,
+                                              uint32_t* nh) {
+    const uint64_t gw = small_warp(), nw = small_warps();
     unsigned lane = lane_id();
-    const uint32_t n = c[0];
     for (uint64_t i = gw; i < n; i += nw) {
         const uint32_t u = list[i];
         const uint64_t end = P.head[u + 1];
-        if (P.excess[u] == 0 || P.cur[u] < end) {
-            if (lane == 0) nh[i] = kUnset;
-            continue;
-        }
+        if (P.excess[u] == 0 || P.cur[u] < end) continue;
         uint32_t m = kUnset;
         for (uint64_t a = P.head[u] + lane; a < end; a += 32)
             if (P.cf[a] > 0) {
@@ -663,22 +690,20 @@ __global__ void k_relabel_small(PR P, const uint32_t* list, const uint32_t* c, u
         if (lane == 0) {
             uint64_t nv = m == kUnset ? P.N : (uint64_t)m + 1;
             if (nv > P.N) nv = P.N;
-            nh[i] = (uint32_t)nv;
+            nh[u] = (uint32_t)nv;
         }
     }
 }
 
-__global__ void __launch_bounds__(kBigThreads) k_relabel_big(PR P, const uint32_t* list,
-                                                             const uint32_t* c, uint32_t* nh) {
+__global__ void __launch_bounds__(kBigThreads) k_relabel(PR P, const uint32_t* list,
+                                                         const uint32_t* smalls,
+                                                         const uint32_t* c, uint32_t* nh) {
     __shared__ uint32_t s_m;
     const uint32_t n = c[1];
     for (uint64_t i = blockIdx.x; i < n; i += gridDim.x) {
         const uint32_t u = list[i];
         const uint64_t end = P.head[u + 1];
-        if (P.excess[u] == 0 || P.cur[u] < end) {
-            if (threadIdx.x == 0) nh[i] = kUnset;
-            continue;
-        }
+        if (P.excess[u] == 0 || P.cur[u] < end) continue;
         if (threadIdx.x == 0) s_m = kUnset;
         __syncthreads();
         uint32_t m = kUnset;
@@ -696,25 +721,11 @@ __global__ void __launch_bounds__(kBigThreads) k_relabel_big(PR P, const uint32_
         if (threadIdx.x == 0) {
             uint64_t nv = s_m == kUnset ? P.N : (uint64_t)s_m + 1;
             if (nv > P.N) nv = P.N;
-            nh[i] = (uint32_t)nv;
+            nh[u] = (uint32_t)nv;
         }
         __syncthreads();
     }
-}
-
-// Relabelled nodes take their new height and restart at their first arc.
-__global__ void k_apply(PR P, const uint32_t* ls, const uint32_t* lb, const uint32_t* c,
-                        const uint32_t* nhs, const uint32_t* nhb) {
-    const uint64_t ns = c[0], nb = c[1];
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ns + nb;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t u = i < ns ? ls[i] : lb[i - ns];
-        uint32_t v = i < ns ? nhs[i] : nhb[i - ns];
-        if (v != kUnset) {
-            P.height[u] = v;
-            P.cur[u] = P.head[u];
-        }
-    }
+    relabel_small(P, smalls, c[0], nh);
 }
 
 // Vertex v of the core is on the source side when it cannot reach t.
@@ -911,10 +922,9 @@ struct CutWork {
     uint64_t* cur = nullptr;
     uint32_t* ls = nullptr;       // active lists: small, big
     uint32_t* lb = nullptr;
-    uint32_t* nhs = nullptr;      // new heights for them
-    uint32_t* nhb = nullptr;
+    uint32_t* nh = nullptr;       // new heights not yet taken, by node
     uint32_t* f[4] = {};          // frontiers: small/big, two levels
-    uint32_t* ctr = nullptr;      // [0,1] active, [2..5] frontier counters
+    uint32_t* ctr = nullptr;      // [0,1], [6,7] active of even and odd rounds, [2..5] frontiers
     unsigned long long* cnt = nullptr;
 };
 
@@ -924,8 +934,7 @@ dsd_status cut_alloc(CutWork* w, uint64_t N, cudaStream_t s) {
     DSD_TRY(dalloc(&w->cur, N + 1, s));
     DSD_TRY(dalloc(&w->ls, N + 1, s));
     DSD_TRY(dalloc(&w->lb, N + 1, s));
-    DSD_TRY(dalloc(&w->nhs, N + 1, s));
-    DSD_TRY(dalloc(&w->nhb, N + 1, s));
+    DSD_TRY(dalloc(&w->nh, N + 1, s));
     for (auto& f : w->f) DSD_TRY(dalloc(&f, N + 1, s));
     DSD_TRY(dalloc(&w->ctr, 8, s));
     DSD_TRY(dalloc(&w->cnt, 1, s));
@@ -933,14 +942,13 @@ dsd_status cut_alloc(CutWork* w, uint64_t N, cudaStream_t s) {
 }
 
 void cut_free(CutWork* w, cudaStream_t s) {
-    void* ptrs[] = {w->excess, w->height, w->cur, w->ls, w->lb, w->nhs, w->nhb,
+    void* ptrs[] = {w->excess, w->height, w->cur, w->ls, w->lb, w->nh,
                     w->f[0], w->f[1], w->f[2], w->f[3], w->ctr, w->cnt};
     for (void* p : ptrs) dev_free(p, s);
     *w = CutWork();
 }
 
-constexpr unsigned kSmallGrid = 152 * 8;   // blocks of 256 threads (warp per node)
-constexpr unsigned kBigGrid = 152 * 4;     // blocks of kBigThreads (block per node)
+constexpr unsigned kBigGrid = 152 * 2;     // blocks of kBigThreads
 
 // Backward breadth-first search from t: exact residual distances to t, N for
 // nodes that cannot reach it (and for s); resets the current arcs.  The
@@ -952,13 +960,11 @@ dsd_status global_relabel(const PR& P, CutWork& w, cudaStream_t s) {
     uint32_t *fs = w.f[0], *fb = w.f[1], *os = w.f[2], *ob = w.f[3];
     uint32_t* cin = w.ctr + 2;
     uint32_t* cout = w.ctr + 4;
-    k_bfs_init<<<grid_for_n(P.N), 256, 0, s>>>(P, fs, fb, cin); note_launch();
+    k_bfs_init<<<grid_for_n(P.N), 256, 0, s>>>(P, w.nh, fs, fb, cin); note_launch();
     for (uint32_t d0 = 0;; d0 += kBfsBatch) {
         for (uint32_t d = d0; d < d0 + kBfsBatch; d++) {
             DSD_CU(cudaMemsetAsync(cout, 0, 8, s));
-            k_bfs_small<<<kSmallGrid, 256, 0, s>>>(P, fs, cin, d, os, ob, cout);
-            k_bfs_big<<<kBigGrid, kBigThreads, 0, s>>>(P, fb, cin, d, os, ob, cout);
-            note_launch();
+            k_bfs<<<kBigGrid, kBigThreads, 0, s>>>(P, fs, fb, cin, d, os, ob, cout);
             note_launch();
             uint32_t* t;
             t = fs; fs = os; os = t;
@@ -1012,27 +1018,27 @@ dsd_status min_cut(const Net& net, int h, uint64_t p, uint64_t q, cudaStream_t s
     note_launch();
     XSTEP(global_relabel(P, w, s));
     cs->relabels++;
+    // a round: heights and lists, pushes, relabels; the list counters of two
+    // rounds alternate (w.ctr + 0 and + 6), each zeroed a round ahead
+    XCU(cudaMemsetAsync(w.ctr, 0, 8 * sizeof(uint32_t), s));
     for (;;) {
         uint32_t na[2] = {0, 0};
-        XCU(cudaMemsetAsync(w.ctr, 0, 8, s));
-        k_collect<<<grid_for_n(N), 256, 0, s>>>(P, w.ls, w.lb, w.ctr); note_launch();
-        XCU(cudaMemcpyAsync(na, w.ctr, 8, cudaMemcpyDeviceToHost, s));
-        XCU(cudaStreamSynchronize(s));
-        if (na[0] + na[1] == 0) break;
         for (int it = 0; it < kRoundsPerRelabel; it++) {
-            if (it) {
-                XCU(cudaMemsetAsync(w.ctr, 0, 8, s));
-                k_collect<<<grid_for_n(N), 256, 0, s>>>(P, w.ls, w.lb, w.ctr);
-                note_launch();
+            uint32_t* c = w.ctr + (it & 1 ? 6 : 0);
+            k_collect<<<grid_for_n(N), 256, 0, s>>>(P, w.nh, w.ls, w.lb, c,
+                                                    w.ctr + (it & 1 ? 0 : 6));
+            note_launch();
+            if (it == 0) {
+                XCU(cudaMemcpyAsync(na, c, 8, cudaMemcpyDeviceToHost, s));
+                XCU(cudaStreamSynchronize(s));
+                if (na[0] + na[1] == 0) break;
             }
-            k_push_small<<<kSmallGrid, 256, 0, s>>>(P, w.ls, w.ctr);
-            k_push_big<<<kBigGrid, kBigThreads, 0, s>>>(P, w.lb, w.ctr);
-            k_relabel_small<<<kSmallGrid, 256, 0, s>>>(P, w.ls, w.ctr, w.nhs);
-            k_relabel_big<<<kBigGrid, kBigThreads, 0, s>>>(P, w.lb, w.ctr, w.nhb);
-            k_apply<<<kSmallGrid, 256, 0, s>>>(P, w.ls, w.lb, w.ctr, w.nhs, w.nhb);
-            for (int k = 0; k < 5; k++) note_launch();
+            k_push<<<kBigGrid, kBigThreads, 0, s>>>(P, w.lb, w.ls, c);
+            k_relabel<<<kBigGrid, kBigThreads, 0, s>>>(P, w.lb, w.ls, c, w.nh);
+            for (int k = 0; k < 2; k++) note_launch();
             cs->rounds++;
         }
+        if (na[0] + na[1] == 0) break;
         XCU(cudaGetLastError());
         XSTEP(global_relabel(P, w, s));
         cs->relabels++;
