@@ -409,6 +409,15 @@ struct BitmapWarp {
     }
 };
 
+// Bitwise ones + x + y: ones takes the sums' low bits, the carries are returned
+// (a full adder a bit).  Two words then cost one popc and two three-input
+// logic operations, which run at four times the rate, instead of two popc.
+__device__ __forceinline__ uint32_t carry_add(uint32_t& ones, uint32_t x, uint32_t y) {
+    const uint32_t c = (ones & x) | (ones & y) | (x & y);
+    ones ^= x ^ y;
+    return c;
+}
+
 // Edges of G[P] (this lane's word of P given; all lanes get the result); each
 // end is credited with its degree.
 __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, uint32_t Pw) {
@@ -441,12 +450,13 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
             const uint32_t j = B.list[q];
             const uint4* row = reinterpret_cast<const uint4*>(B.rows + j * B.Ws);
             const uint4* P4 = reinterpret_cast<const uint4*>(B.sP);
-            unsigned s = 0;
+            unsigned twos = 0, ones = 0;
             for (uint32_t v = lo; v < hi; v++) {
                 const uint4 a = row[v], p = P4[v];
-                s += __popc(a.x & p.x) + __popc(a.y & p.y);
-                s += __popc(a.z & p.z) + __popc(a.w & p.w);
+                twos += __popc(carry_add(ones, a.x & p.x, a.y & p.y));
+                twos += __popc(carry_add(ones, a.z & p.z, a.w & p.w));
             }
+            const unsigned s = 2 * twos + __popc(ones);
             if (s) B.credit(j, s);
             sum += s;
         }
