@@ -260,8 +260,10 @@ __device__ __forceinline__ unsigned long long warp_dfs32(const uint32_t* rows, u
 // is the number of cliques.  A lane per candidate needs no reduction, no
 // leaf bit-counters and one shared atomic per candidate, where a lane per word
 // needed some 25 instructions for every candidate: listing R-MAT scale 18,
-// h = 5: 164 -> 43 ms, scale 17, h = 4: 7.2 -> 4.3 ms.  Bound by popc (16
-// lanes a clock and SM) and the instructions around a node.
+// h = 5: 164 -> 43 ms, scale 17, h = 4: 7.2 -> 4.3 ms.  Bound by the row loads
+// (bank conflicts between candidates' rows) and the instructions around a
+// node; small sets of three members to go are searched in registers instead
+// (warp_triangles_reg).
 //
 // The stride is 4 words times an odd number, so that the 16-byte row loads of
 // eight lanes fall into different banks.
@@ -418,6 +420,29 @@ __device__ __forceinline__ uint32_t carry_add(uint32_t& ones, uint32_t x, uint32
     return c;
 }
 
+// The positions base .. base + kLeafList - 1 among P's set bits into B.list
+// (pc, inc: bits of this lane's word and of the words up to it).
+__device__ __forceinline__ void warp_list(const BitmapWarp& B, uint32_t Pw, uint32_t pc,
+                                          uint32_t inc, uint32_t base) {
+    uint32_t at = inc - pc, w = Pw;
+    while (w) {
+        const uint32_t b = __ffs(w) - 1u;
+        w &= w - 1u;
+        if (at >= base && at < base + kLeafList)
+            B.list[at - base] = (uint16_t)(lane_id() * 32 + b);
+        at++;
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ uint32_t warp_incl_sum(uint32_t x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if ((int)lane_id() >= o) x += y;
+    }
+    return x;
+}
+
 // Edges of G[P] (this lane's word of P given; all lanes get the result); each
 // end is credited with its degree.
 __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, uint32_t Pw) {
@@ -426,25 +451,13 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
     if (!nz) return 0;
     const uint32_t lo = (uint32_t)(__ffs(nz) - 1) >> 2, hi = ((31u - __clz(nz)) >> 2) + 1u;
     const uint32_t pc = __popc(Pw);
-    uint32_t inc = pc;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(full, inc, o);
-        if ((int)lane >= o) inc += y;
-    }
+    const uint32_t inc = warp_incl_sum(pc);
     const uint32_t total = __shfl_sync(full, inc, 31);
     if (total < 2) return 0;
     if (lane < B.Ws) B.sP[lane] = Pw;
     unsigned sum = 0;
     for (uint32_t base = 0; base < total; base += kLeafList) {
-        uint32_t at = inc - pc, w = Pw;
-        while (w) {
-            const uint32_t b = __ffs(w) - 1u;
-            w &= w - 1u;
-            if (at >= base && at < base + kLeafList) B.list[at - base] = (uint16_t)(lane * 32 + b);
-            at++;
-        }
-        __syncwarp();
+        warp_list(B, Pw, pc, inc, base);
         const uint32_t m = total - base < kLeafList ? total - base : kLeafList;
         for (uint32_t q = lane; q < m; q += 32) {
             const uint32_t j = B.list[q];
@@ -465,13 +478,98 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
     return __reduce_add_sync(full, sum) >> 1;   // sum <= 1024 * 1023
 }
 
+// Triangles of G[P] for p members of P, 32 (K - 1) < p <= 32 K, their positions
+// in B.list: G[P] is gathered into registers, a lane holding the rows of K
+// members over the members only, so that a node of the search (the members
+// above j adjacent to it) takes no shared memory at all: K broadcasts and at
+// most K * K popc.  In the shared rows a node costs its list, its row loads
+// over the whole width of G[C] (with bank conflicts) and its credits, some 570
+// issue slots on R-MAT scale 18 (h = 5, 27 candidates a node).  That listing
+// call: 49.9 -> 24.7 ms.  Bound by popc and the broadcasts of a node.
+template <int K>
+__device__ unsigned warp_triangles_reg(const BitmapWarp& B, uint32_t p) {
+    const unsigned full = 0xffffffffu, lane = lane_id();
+    uint32_t pos[K], row[K][K], cnt[K];
+    const uint32_t last = p & 31u ? (1u << (p & 31u)) - 1u : full;   // members of the last 32
+#pragma unroll
+    for (int s = 0; s < K; s++) {
+        pos[s] = s * 32 + lane < p ? B.list[s * 32 + lane] : 0u;
+        cnt[s] = 0;
+    }
+#pragma unroll
+    for (int s = 0; s < K; s++) {
+#pragma unroll
+        for (int w = 0; w < K; w++) row[s][w] = 0;
+        const uint32_t na = p - s * 32 < 32u ? p - s * 32 : 32u;
+        for (uint32_t a = 0; a < na; a++) {
+            const uint32_t* r = B.rows + __shfl_sync(full, pos[s], a) * B.Ws;
+#pragma unroll
+            for (int w = 0; w < K; w++) {
+                unsigned m = __ballot_sync(full, (r[pos[w] >> 5] >> (pos[w] & 31u)) & 1u);
+                if (w == K - 1) m &= last;
+                if (lane == a) row[s][w] = m;
+            }
+        }
+    }
+    unsigned total = 0;
+#pragma unroll
+    for (int s = 0; s < K; s++) {
+        const uint32_t na = p - s * 32 < 32u ? p - s * 32 : 32u;
+        for (uint32_t a = 0; a < na; a++) {
+            uint32_t pn[K], any = 0;
+#pragma unroll
+            for (int w = s; w < K; w++) {
+                pn[w] = __shfl_sync(full, row[s][w], a);
+                if (w == s) pn[w] &= 0xfffffffeu << a;
+                any |= pn[w];
+            }
+            if (!any) continue;
+            unsigned sum = 0;
+#pragma unroll
+            for (int q = s; q < K; q++) {
+                unsigned c = 0;
+#pragma unroll
+                for (int w = s; w < K; w++) c += __popc(row[q][w] & pn[w]);
+                if (!((pn[q] >> lane) & 1u)) c = 0;
+                cnt[q] += c;
+                sum += c;
+            }
+            sum = __reduce_add_sync(full, sum) >> 1;
+            if (lane == a) cnt[s] += sum;
+            total += sum;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < K; s++)
+        if (s * 32 + lane < p && cnt[s]) B.credit(pos[s], cnt[s]);
+    __syncwarp();   // B.list is used again
+    return total;
+}
+// P above this is searched in the shared rows: K = 5 needs 25 registers of rows
+// alone, of the 64 that a block of 1,024 threads has a thread.
+constexpr uint32_t kRegMembers = 32 * 4;
+
 // RR-cliques of G[P], RR >= 2; each member is credited with those it is in.
-template <int RR>
+// REG: triangles of at most kRegMembers members in registers (for callers with
+// the registers to spare: r >= 4).
+template <int RR, bool REG>
 __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
     if constexpr (RR == 2) {
         return warp_edges(B, Pw);
     } else {
         const unsigned full = 0xffffffffu, lane = lane_id();
+        if constexpr (RR == 3 && REG) {
+            const uint32_t pc = __popc(Pw);
+            const uint32_t p = __reduce_add_sync(full, pc);
+            if (p < 3) return 0;
+            if (p <= kRegMembers) {
+                warp_list(B, Pw, pc, warp_incl_sum(pc), 0);
+                if (p <= 32) return warp_triangles_reg<1>(B, p);
+                if (p <= 64) return warp_triangles_reg<2>(B, p);
+                if (p <= 96) return warp_triangles_reg<3>(B, p);
+                return warp_triangles_reg<4>(B, p);
+            }
+        }
         unsigned long long acc = 0;
         uint32_t rem = Pw;
         for (;;) {
@@ -488,7 +586,7 @@ __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
                 sub = warp_edges(B, pn);
             } else {
                 if (__reduce_add_sync(full, (unsigned)__popc(pn)) < RR - 1) continue;
-                sub = warp_cliques<RR - 1>(B, pn);
+                sub = warp_cliques<RR - 1, REG>(B, pn);
             }
             if (sub) {
                 if (lane == 0) B.credit(j, sub);
@@ -499,14 +597,15 @@ __device__ unsigned long long warp_cliques(const BitmapWarp& B, uint32_t Pw) {
     }
 }
 
+template <bool REG>
 __device__ __forceinline__ unsigned long long warp_cliques_of(const BitmapWarp& B, uint32_t Pw,
                                                              int rr) {
     switch (rr) {
-        case 2: return warp_cliques<2>(B, Pw);
-        case 3: return warp_cliques<3>(B, Pw);
-        case 4: return warp_cliques<4>(B, Pw);
-        case 5: return warp_cliques<5>(B, Pw);
-        default: return warp_cliques<6>(B, Pw);   // r <= DSD_MAX_H - 1 = 7
+        case 2: return warp_cliques<2, REG>(B, Pw);
+        case 3: return warp_cliques<3, REG>(B, Pw);
+        case 4: return warp_cliques<4, REG>(B, Pw);
+        case 5: return warp_cliques<5, REG>(B, Pw);
+        default: return warp_cliques<6, REG>(B, Pw);   // r <= DSD_MAX_H - 1 = 7
     }
 }
 
@@ -534,6 +633,7 @@ __device__ __forceinline__ BitmapWarp bitmap_warp(const uint32_t* rows, uint32_t
 // go first); r >= 3: only those of start, start + step, ... below nd, and
 // only candidates below nd are credited.  scratch: kWarpScratch words a warp, 16-byte aligned.  Returns this
 // thread's share of the total (sum over the block = total).
+template <bool REG = false>
 __device__ __forceinline__ unsigned long long block_dfs(const uint32_t* rows, uint32_t nc,
                                                        uint32_t W, int r,
                                                        unsigned long long* cnt,
@@ -570,7 +670,7 @@ __device__ __forceinline__ unsigned long long block_dfs(const uint32_t* rows, ui
         if (lane < iw) P = 0;
         else if (lane == iw) P &= (i & 31u) == 31u ? 0u : 0xffffffffu << ((i & 31u) + 1u);
         if ((int)__reduce_add_sync(full, (unsigned)__popc(P)) < r - 1) continue;
-        const unsigned long long c = warp_cliques_of(B, P, r - 1);
+        const unsigned long long c = warp_cliques_of<REG>(B, P, r - 1);
         if (c) {
             if (lane == 0) B.credit(i, c);
             total += c;

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count_small(CountArgs A) {
 }
 
 // Tier M: one block per vertex, |N+(u)| in (32, 1024].
-template <int NT>
+template <int NT, bool REG>
 __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
     extern __shared__ __align__(16) uint32_t smem[];
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(smem);  // 1024
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(NT) k_count_medium(CountArgs A) {
         } else {
             block_build_rows(C, d, W, A.off + 1, A.adj, A.split, rows, win);
             __syncthreads();
-            mine = block_dfs(rows, d, W, A.r, cnt, &s_next, scratch);
+            mine = block_dfs<REG>(rows, d, W, A.r, cnt, &s_next, scratch);
         }
         if (mine) atomicAdd(&s_tot, mine);
         __syncthreads();
@@ -376,11 +376,11 @@ dsd_status count_cliques(dsd_graph* g, int h, unsigned long long* deg_new,
                              : (size_t)(3 * kBitmapMax + kWindowWords) * 4;
         if (h >= 4) {
             // one block per SM (the rows fill its shared memory): 32 warps
-            cudaFuncSetAttribute(k_count_medium<1024>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemM);
-            k_count_medium<1024><<<sms, 1024, smemM, s>>>(A);
+            const auto kern = h >= 5 ? k_count_medium<1024, true> : k_count_medium<1024, false>;
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemM);
+            kern<<<sms, 1024, smemM, s>>>(A);
         } else {
-            k_count_medium<kCountThreads><<<sms * 4, kCountThreads, smemM, s>>>(A);
+            k_count_medium<kCountThreads, false><<<sms * 4, kCountThreads, smemM, s>>>(A);
         }
         note_launch();
         if (h == 3) {

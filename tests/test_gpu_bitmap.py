@@ -50,6 +50,17 @@ def test_random_dense(L, orc, n, p, h):
         assert k == wk and np.array_equal(core, wcore)
 
 
+@pytest.mark.parametrize("n,p,h", [(36, 0.97, 5), (70, 0.95, 5), (105, 0.9, 5), (136, 0.97, 5),
+                                   (150, 0.85, 5), (80, 0.9, 6), (60, 0.9, 7)])
+def test_register_search(L, orc, n, p, h):
+    """Sets of up to and just above 32, 64, 96 and 128 members below a node."""
+    n, s, d = gg.er(n, p, seed=3 * n + h)
+    wdeg, wmu = orc.clique_degrees(orc.csr(n, s, d), h)
+    with L.Graph.from_edges(n, s, d) as g:
+        deg, mu = g.clique_degrees(h)
+    assert mu == wmu and np.array_equal(deg, wdeg)
+
+
 @pytest.mark.parametrize("d", [31, 32, 33, 63, 64, 1024, 1025, 12288, 12289])
 def test_noalloc_row_tiers(L, d):
     """dsd_triangle_degrees_noalloc on both sides of its row tiers: a hub of
