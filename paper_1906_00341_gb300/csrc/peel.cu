@@ -462,7 +462,9 @@ __device__ void process_vw(const PeelParams& P, const NPlus& R, uint32_t v, uint
                                                      next_cnt, bytes);
         __syncwarp();
         if (nc < (uint32_t)r) return;
-        if (nc <= kWarpCand && !dec_w && !__any_sync(0xffffffffu, anyd)) return;   // none count
+        // none count -- known only of a complete walk: one that stopped past
+        // gather_cap has not seen the rest (a block looks again, process_big)
+        if (nc <= P.gather_cap && !dec_w && !__any_sync(0xffffffffu, anyd)) return;
         if (nc > P.warp_cand) {
             // mid item: its candidates go with it to a warp group; else a block
             if (nc <= kWarpCand && P.mid_cap) {

@@ -1,0 +1,83 @@
+"""Calls that earlier forms of the kernels answered wrongly, refused or slowed
+down, each at the smallest input that shows it."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1906_00341_gb300 import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_1906_00341_gb300 import build as b
+    b.build()
+    from paper_1906_00341_gb300 import _lib
+    _lib.load()
+    return _lib
+
+
+def clique(v):
+    v = np.asarray(v, np.int64)
+    i, j = np.triu_indices(v.size, 1)
+    return v[i], v[j]
+
+
+def late_member():
+    """h = 5: an item (v, w) whose first 128 entries of N+(w) hold more than
+    four members of later bands and only then x, which is in v's band.
+
+    Ids 0-9 are W, a clique with v and x (so v has C(11, 4) = 330 cliques) and
+    with 10 more vertices Z (a later band); each of W has 150 further
+    neighbours among Q, which lie between W and x in the degeneracy order: Q
+    is one side of a complete bipartite graph (no triangles there) and x is of
+    the other side.  x is in 35 cliques of a K13 besides.  400 disjoint K14,
+    one vertex of each next to v, keep v's row long.  K5, K6 and K7 give v's
+    band its first levels."""
+    W = np.arange(10)
+    at = [10]
+
+    def take(k):
+        at[0] += k
+        return np.arange(at[0] - k, at[0])
+    v, = take(1)
+    Z = take(10)
+    Q = take(1500)
+    P = take(220)
+    x = P[0]
+    E = [clique(np.concatenate([W, [v, x]])), clique(np.concatenate([W, Z]))]
+    E.append((np.repeat(P, Q.size), np.tile(Q, P.size)))
+    E += [(np.full(150, w), Q[150 * w:150 * w + 150]) for w in W]
+    k13 = take(13)
+    E += [clique(k13), (np.full(7, x), k13[:7])]
+    for _ in range(400):
+        c = take(14)
+        E += [clique(c), (np.array([v]), c[:1])]
+    E += [clique(take(k)) for k in (5, 6, 7)]
+    return (at[0], np.concatenate([a for a, _ in E]).astype(np.uint32),
+            np.concatenate([b for _, b in E]).astype(np.uint32), v, x)
+
+
+@pytest.mark.parametrize("warp_max", [4, 16, 32])
+def test_queue_off_long_rows(L, orc, warp_max):
+    """dsd_set_peel_items(w, 0): a candidate walk that stops at w candidates says
+    nothing about the rest of the row, so its item must reach a block."""
+    n, s, d, v, x = late_member()
+    og = orc.csr(n, s, d)
+    wcore, wk = orc.core_decompose(og, 5)
+    wl = orc.level_stats(og, 5, wcore)
+    assert wcore[v] == wcore[x] == 330
+    L.dsd_set_peel_items(warp_max, 0)
+    try:
+        with L.Graph.from_edges(n, s, d) as g:
+            core, k = g.core_decompose(5)
+            lv = g.level_stats(5)
+    finally:
+        L.dsd_set_peel_items(4, 1 << 20)
+    assert k == wk and np.array_equal(core, wcore)
+    for a, b in zip(lv, wl):
+        assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
