@@ -554,8 +554,9 @@ dsd_status decompose(dsd_graph* g, int pattern, int x, PatWork* w, Levels* L, ui
     };
     if (pattern == kStar && peel_tail_limit() > 0) {
         // in bands (26 times faster at 50,000 vertices), unless a sum of
-        // counts could wrap around 2^64: bands need counts that only fall,
-        // and the one-level peel compares whatever the wrapped counts are
+        // counts could wrap around 2^64 (bands need counts that only fall,
+        // and the one-level peel compares whatever the wrapped counts are) or
+        // the device has no room for them
         uint32_t nl = 0;
         bool done = false;
         DSD_TRY(star_bands(g, x, w, &nl, kmax, &done));

@@ -81,3 +81,27 @@ def test_queue_off_long_rows(L, orc, warp_max):
     assert k == wk and np.array_equal(core, wcore)
     for a, b in zip(lv, wl):
         assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
+
+
+def test_star_without_room(L):
+    """The x-star peel on a device with room for the one-level peel but not for
+    the bands' 56 bytes an edge (20M edges): the same result, no error."""
+    import torch
+    n, w = 1_000_000, 20
+    i = np.arange(n, dtype=np.int64)
+    s = np.tile(i, w).astype(np.uint32)
+    d = np.concatenate([(i + j) % n for j in range(1, w + 1)]).astype(np.uint32)
+    with L.Graph.from_edges(n, s, d) as g:
+        want = g.pattern_core_decompose(L.DSD_PATTERN_STAR, 2)
+        L.dsd_release_memory()
+        torch.cuda.synchronize()
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - (600 << 20), dtype=torch.uint8,
+                           device="cuda")
+        try:
+            got = g.pattern_core_decompose(L.DSD_PATTERN_STAR, 2)
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+    assert got[1] == want[1] == 780 + 40 * 39   # C(40, 2) + 40 C(39, 1) at every vertex
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
