@@ -82,9 +82,15 @@ const char* dsd_version(void);
 uint64_t dsd_kernel_launches(void);
 
 /* Device memory comes from a pool of the library's own on each device, which
- * keeps at most 2 GiB of freed memory for later calls.  This gives what is
- * unused at the time back to the device (the current one).  DSD_ERR_CUDA. */
+ * keeps at most 2 GiB of freed memory for later calls (dsd_set_memory_keep
+ * changes the bound).  This gives what is unused at the time back to the
+ * device (the current one).  DSD_ERR_CUDA. */
 dsd_status dsd_release_memory(void);
+/* What that pool keeps of freed memory, in bytes (default 2 GiB), on the
+ * current device; what it holds unused beyond the bound goes back at once, and
+ * later at each synchronisation.  0: nothing is kept, for a process whose other
+ * allocators need the memory.  DSD_ERR_CUDA. */
+dsd_status dsd_set_memory_keep(uint64_t bytes);
 
 /* Upper bound, in milliseconds, on every inter-block wait inside a
  * persistent kernel (grid barriers).  A wait that runs out makes the kernel

@@ -87,6 +87,7 @@ SIGNATURES = {
     "dsd_version": (ctypes.c_char_p, []),
     "dsd_kernel_launches": (ctypes.c_uint64, []),
     "dsd_release_memory": (_int, []),
+    "dsd_set_memory_keep": (_int, [ctypes.c_uint64]),
     "dsd_set_wait_limit_ms": (_int, [_u32]),
     "dsd_set_peel_small_limit": (_int, [_u32]),
     "dsd_set_peel_tail_limit": (_int, [_u32]),
@@ -193,6 +194,11 @@ def dsd_kernel_launches():
 
 def dsd_release_memory():
     _check(load().dsd_release_memory())
+
+
+def dsd_set_memory_keep(nbytes):
+    """What the library keeps of freed device memory (default 2 GiB; 0: nothing)."""
+    _check(load().dsd_set_memory_keep(int(nbytes)))
 
 
 def dsd_set_wait_limit_ms(ms):

@@ -391,6 +391,11 @@ dsd_status dsd_release_memory(void) {
     return release_memory();
 }
 
+dsd_status dsd_set_memory_keep(uint64_t bytes) {
+    set_error("");
+    return set_memory_keep(bytes);
+}
+
 dsd_status dsd_set_checked(int on) {
     g_checked = on ? 1 : 0;
     return DSD_OK;

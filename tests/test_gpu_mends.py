@@ -105,3 +105,25 @@ def test_star_without_room(L):
     assert got[1] == want[1] == 780 + 40 * 39   # C(40, 2) + 40 C(39, 1) at every vertex
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("keep", [0, 64 << 20])
+def test_memory_keep(L, keep):
+    """dsd_set_memory_keep: after a synchronisation no more than the bound of
+    freed memory stays with the library (the default keeps up to 2 GiB, which
+    another allocator of the process could not have)."""
+    import torch
+    L.dsd_release_memory()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    n, s, d = gg.er(200_000, 0.0002, 3)   # 4M edges: some 500 MB in use at a time
+    L.dsd_set_memory_keep(keep)
+    try:
+        for _ in range(2):
+            with L.Graph.from_edges(n, s, d) as g:
+                g.core_app(3)
+            torch.cuda.synchronize()
+            assert torch.cuda.mem_get_info()[0] >= free0 - keep - (64 << 20)
+    finally:
+        L.dsd_set_memory_keep(2 << 30)
+        L.dsd_release_memory()
