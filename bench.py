@@ -826,7 +826,7 @@ def run_c3(args, local):
             "densest": [int(r0.densest_mu), int(r0.densest_size)],
             "kmax_core_size": int(r0.kmax_core_size),
             "peel": {k: ps[k] for k in ("rounds", "levels", "items", "barrier_ns", "barriers",
-                                        "small_round")},
+                                        "bands", "grid_rounds")},
             "roofline_listing": roof,
         }
     L.dsd_set_wait_limit_ms(20000)

@@ -142,13 +142,13 @@ SIGNATURES = {
                                     ctypes.POINTER(CoreAppResult)]),
 }
 
+# dsd_peel_stats' words in order (None: not used).
 PEEL_STATS = ("rounds", "levels", "items", "bytes", "barrier_ns", "barriers", "compactions",
-              "threads", "grid", "kmax", "small_round",
-              "t_large_retire", "t_large_scan", "t_large_jump", "t_large_enum",
-              "t_small_retire", "t_small_jump", "t_small_mark", "t_small_enum",
-              "tail_n", "tail_round", "tail_ns",
-              "t_tail_build", "t_tail_front", "t_tail_jump", "t_tail_prefix", "t_tail_work",
-              "t_tail_sync", "t_tail_retire")
+              "threads", "grid", "kmax", None,
+              "t_band_retire", "t_band_scan", "t_band_jump", "t_band_enum",
+              "t_level_book", "t_level_rows", "t_level_enum", "t_level_queued",
+              "band_n", "band_round", "phase2_ns", "bands", "grid_rounds",
+              None, None, None, None, None)
 
 
 def load(path: str = LIB_PATH):
@@ -447,7 +447,9 @@ def dsd_phase_stats(g):
 def dsd_peel_stats(g, which):
     out = (ctypes.c_uint64 * len(PEEL_STATS))()
     _check(load().dsd_peel_stats(g, which, ctypes.addressof(out)))
-    return dict(zip(PEEL_STATS, [int(x) for x in out]))
+    st = {k: int(x) for k, x in zip(PEEL_STATS, out) if k}
+    st["tail_n"] = st["band_n"]   # the alive set's size at that point by its earlier name
+    return st
 
 
 def dsd_check_barrier_timeout(absent_block, wait_ms, stream_ptr):

@@ -43,7 +43,7 @@ void record_peel(dsd_graph* g, int which, const PeelResult& r) {
     o[7] = r.threads;
     o[8] = r.grid;
     o[9] = r.kmax;
-    o[10] = 0;   // the replicated small regime is gone
+    o[10] = 0;
     for (int i = 0; i < 8; i++) o[11 + i] = r.tph[i];
     o[19] = r.band_n;
     o[20] = r.band_round;

@@ -127,3 +127,32 @@ def test_memory_keep(L, keep):
     finally:
         L.dsd_set_memory_keep(2 << 30)
         L.dsd_release_memory()
+
+
+def test_peel_stats_names(L):
+    """Every word of dsd_peel_stats under the name of what it holds: the 100
+    levels of a K3 .. K102 each (h = 2) in bands, and none with bands off."""
+    sizes = range(3, 103)
+    base = np.cumsum([0] + [k for k in sizes])
+    E = [clique(b + np.arange(k)) for b, k in zip(base, sizes)]
+    n = int(base[-1]) + 20_000   # vertices without edges: not one block's graph
+    s = np.concatenate([a for a, _ in E]).astype(np.uint32)
+    d = np.concatenate([b for _, b in E]).astype(np.uint32)
+    for limit in (1 << 30, 0):
+        L.dsd_set_peel_tail_limit(limit)
+        try:
+            with L.Graph.from_edges(n, s, d) as g:
+                g.core_app(3)
+                st = L.dsd_peel_stats(g.handle, 1)
+        finally:
+            L.dsd_set_peel_tail_limit(1 << 30)
+        assert st["levels"] == 101 and st["kmax"] == 101 * 100 // 2
+        if limit:
+            # bands of more than one level, all begun on the 5,250 vertices left
+            # after level 0 or before it; fewer grid rounds than rounds
+            assert 1 <= st["bands"] <= 50 and 0 < st["band_n"] <= n
+            assert 0 < st["phase2_ns"] < 10 ** 10
+            assert st["grid_rounds"] < st["rounds"]
+        else:
+            assert st["bands"] == st["band_n"] == st["phase2_ns"] == 0
+            assert st["grid_rounds"] == st["rounds"]
