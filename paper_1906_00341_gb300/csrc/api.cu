@@ -29,7 +29,11 @@ static std::atomic<int> g_checked{0};
 bool checked_mode() { return g_checked.load() != 0; }
 
 static std::atomic<unsigned long long> g_launches{0};
-void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+static thread_local uint32_t t_launches = 0;   // this thread's, for a phase's count
+void note_launch() {
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    t_launches++;
+}
 
 void record_peel(dsd_graph* g, int which, const PeelResult& r) {
     uint64_t* o = g->peel_stats[which];
@@ -54,10 +58,12 @@ void record_peel(dsd_graph* g, int which, const PeelResult& r) {
 }
 
 void prof_begin(dsd_graph* g, int phase) {
+    g->prof_launches[phase] = t_launches;
     if (!g->profiling) return;
     cudaEventRecord(g->ev[2 * phase], g->stream);
 }
 void prof_end(dsd_graph* g, int phase) {
+    g->prof_launches[phase] = t_launches - g->prof_launches[phase];
     if (!g->profiling) return;
     cudaEventRecord(g->ev[2 * phase + 1], g->stream);
     g->prof_ms[phase] = -1.f;   // resolved lazily in dsd_phase_stats
@@ -221,7 +227,6 @@ dsd_status decompose(dsd_graph* g, int h) {
         st = run_peel(g, h, n, g->roff, g->radj, g->rsplit, g->maxdplus, deg, mu, core_new,
                       nullptr, g->lvl_k, g->lvl_size, g->lvl_mu, &pr);
         prof_end(g, kPhasePeel);
-        g->prof_launches[kPhasePeel] = 2;
     }
     if (st == DSD_OK && n) {
         k_map_u64<<<grid_for(n), 256, 0, s>>>(n, g->old_of, core_new, g->core); note_launch();
@@ -439,7 +444,6 @@ dsd_status dsd_graph_from_edges(uint32_t n, uint64_t m, const uint32_t* src, con
     }
     if (st == DSD_OK) st = build_csr(g, m, ds, dd);
     prof_end(g, kPhaseCsr);
-    g->prof_launches[kPhaseCsr] = 12;
     dev_free(tmp, s);
     if (st != DSD_OK) {
         dsd_graph_destroy(g);
@@ -704,7 +708,6 @@ dsd_status dsd_core_app(dsd_graph* g, int h, uint32_t* kmax_core, uint32_t* dens
         }
     }
     prof_end(g, kPhaseExtract);
-    g->prof_launches[kPhaseExtract] = 1 + (kmax_core ? 5 : 0) + (densest ? 5 : 0);
     if (st == DSD_OK) {
         e = cudaMemcpyAsync(&hr, dr, sizeof(hr), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -410,7 +410,6 @@ dsd_status count_cliques(dsd_graph* g, int h, unsigned long long* deg_new,
         set_error("h=%d: a clique-degree or mu exceeds 2^64 - 1 (checked mode)", h);
         return DSD_ERR_OVERFLOW;
     }
-    g->prof_launches[kPhaseCount] = h == 3 ? 6 : (g->maxdplus > kBitmapMax ? 6 : 5);
     return st;
 }
 

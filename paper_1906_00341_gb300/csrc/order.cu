@@ -192,7 +192,6 @@ dsd_status ensure_order(dsd_graph* g) {
     STEP(run_peel(g, 2, n, g->off, g->adj, nullptr, 0, deg, g->m, g->core2, g->rnd, g->lvl2_k,
                   g->lvl2_size, g->lvl2_mu, &pr));
     prof_end(g, kPhaseOrderPeel);
-    g->prof_launches[kPhaseOrderPeel] = 3;
     g->degeneracy = (uint32_t)pr.kmax;
     g->order_kmax = pr.kmax;
     g->nlevels2 = pr.nlevels;
@@ -203,7 +202,6 @@ dsd_status ensure_order(dsd_graph* g) {
         prof_begin(g, kPhaseOrient);
         STEP(tiny_orient(g));
         prof_end(g, kPhaseOrient);
-        g->prof_launches[kPhaseOrient] = 1;
         g->ordered = true;
         goto done;
     }
@@ -252,7 +250,6 @@ dsd_status ensure_order(dsd_graph* g) {
     CUSTEP(cudaStreamSynchronize(s));
     g->maxdplus = hmax;
     prof_end(g, kPhaseOrient);
-    g->prof_launches[kPhaseOrient] = 12;
     g->ordered = true;
 done:
 #undef STEP

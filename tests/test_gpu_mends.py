@@ -156,3 +156,22 @@ def test_peel_stats_names(L):
         else:
             assert st["bands"] == st["band_n"] == st["phase2_ns"] == 0
             assert st["grid_rounds"] == st["rounds"]
+
+
+@pytest.mark.parametrize("n,p", [(2000, 0.005), (40_000, 0.0005)])
+def test_phase_launches(L, n, p):
+    """The kernels dsd_phase_stats says each phase launched, against the
+    library's own count: one-block stages and the general ones."""
+    n, s, d = gg.er(n, p, 1)
+    at = [L.dsd_kernel_launches()]
+    with L.Graph.from_edges(n, s, d) as g:
+        at.append(L.dsd_kernel_launches())
+        g.degeneracy_order()
+        at.append(L.dsd_kernel_launches())
+        g.clique_degrees(3)
+        at.append(L.dsd_kernel_launches())
+        csr, peel, orient, count = [int(x) for x in L.dsd_phase_stats(g.handle)[2][:4]]
+    assert min(csr, peel, orient, count) > 0
+    assert csr == at[1] - at[0]
+    assert peel + orient <= at[2] - at[1] <= peel + orient + 1   # and the core numbers' map
+    assert count <= at[3] - at[2] <= count + 1                   # and the counts'
