@@ -20,6 +20,12 @@ constexpr uint32_t kBandMax = 8192;
 // 1M-vertex graph (h = 3) and R-MAT scale 17 (h = 4) take the same time within
 // 3 % from 1 to 16.
 constexpr float kBandFill = 2.0f;
+// ... and never at more than kBandAim: from 33.5M vertices on a first frontier
+// alone could pass kBandMax, so that every cascade would be undone.
+__device__ __forceinline__ uint32_t band_aim(uint32_t left) {
+    const uint32_t t = (uint32_t)sqrtf(kBandFill * (float)left);
+    return t < kBandAim ? t : kBandAim;
+}
 
 // Warp-aggregated append of `val` where pred holds (all lanes call).
 __device__ __forceinline__ void warp_append(bool pred, uint32_t val, uint32_t* counter,

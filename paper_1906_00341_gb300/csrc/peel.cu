@@ -1579,7 +1579,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             seg = retired;
             unsigned long long kt = 0;
             if (banding && m2 > k) {
-                const uint32_t tmax = (uint32_t)sqrtf(kBandFill * (float)left);
+                const uint32_t tmax = band_aim(left);
                 kt = pick_threshold<NT>(ghist, k, tmax, tmax / 8, s_wtot, &s_n);
                 multi = kt > m2;
             }

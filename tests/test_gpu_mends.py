@@ -175,3 +175,27 @@ def test_phase_launches(L, n, p):
     assert csr == at[1] - at[0]
     assert peel + orient <= at[2] - at[1] <= peel + orient + 1   # and the core numbers' map
     assert count <= at[3] - at[2] <= count + 1                   # and the counts'
+
+
+def test_band_aim(L):
+    """However many vertices are alive, a band's threshold is set for at most
+    2,048 of them: 4M vertices in K6 (10 triangles each), 1,800 in single
+    triangles and 600 in K4 (3 each) make no band of several levels."""
+    def many(k, count, at):
+        i, j = np.triu_indices(k, 1)
+        o = at + k * np.arange(count)[:, None]
+        return (o + i).ravel(), (o + j).ravel(), at + k * count
+    s6, d6, at = many(6, 666_700, 0)
+    s3, d3, at = many(3, 600, at)
+    s4, d4, n = many(4, 150, at)
+    s = np.concatenate([s6, s3, s4]).astype(np.uint32)
+    d = np.concatenate([d6, d3, d4]).astype(np.uint32)
+    with L.Graph.from_edges(n, s, d) as g:
+        core, k = g.core_decompose(3)
+        lk, ls, lm = g.level_stats(3)
+        st = L.dsd_peel_stats(g.handle, 1)
+    assert k == 10 and np.array_equal(lk, [1, 3, 10])
+    assert np.array_equal(ls, [n, n - 1800, n - 2400])
+    assert np.array_equal(lm, [20 * 666_700 + 600 + 4 * 150, 20 * 666_700 + 4 * 150, 20 * 666_700])
+    assert np.array_equal(core, np.repeat([10, 1, 3], [6 * 666_700, 1800, 600]))
+    assert st["bands"] == 0
