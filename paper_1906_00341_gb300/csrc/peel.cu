@@ -1409,6 +1409,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
     uint32_t nb = 0;                       // multi-level bands so far
     bool multi = false;                    // the current band has several levels
     uint32_t seg = 0;                      // where it starts in mem
+    uint32_t rjump = 0;                    //   and its first round
     uint32_t fails = 0, hold = 0;          // cascades undone in a row; jumps without bands
     unsigned long long gone0 = 0;          // lead: cliques destroyed before the band
     uint32_t rs = 0;                       // rounds of single-level bands so far
@@ -1462,7 +1463,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
         }
         uint32_t fcur = c->fcnt[r % 3];
         uint32_t* Fcur = P.front[r % 3];
-        const bool undo = multi && retired - seg + fcur > kBandMax;
+        const bool undo = multi && (retired - seg + fcur > kBandMax ||
+                                    (fcur && r - rjump >= kBandRounds));
         // the bitmaps of F_{r-1}'s hubs are zeroed for round r+1
         if (r && P.hub_slots) {
             uint32_t nhub = c->hubcnt[(r + 1) & 1];
@@ -1577,6 +1579,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             multi = false;
             klow = k;
             seg = retired;
+            rjump = r;
             unsigned long long kt = 0;
             if (banding && m2 > k) {
                 const uint32_t tmax = band_aim(left);

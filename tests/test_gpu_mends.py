@@ -199,3 +199,31 @@ def test_band_aim(L):
     assert np.array_equal(lm, [20 * 666_700 + 600 + 4 * 150, 20 * 666_700 + 4 * 150, 20 * 666_700])
     assert np.array_equal(core, np.repeat([10, 1, 3], [6 * 666_700, 1800, 600]))
     assert st["bands"] == 0
+
+
+def strip(n, w):
+    """Vertices in a row, each next to the w before and after it: one level that
+    leaves from the two ends, a vertex each a round."""
+    i = np.arange(n, dtype=np.int64)
+    s = np.concatenate([i[:n - j] for j in range(1, w + 1)])
+    d = np.concatenate([i[j:] for j in range(1, w + 1)])
+    return n, s.astype(np.uint32), d.astype(np.uint32)
+
+
+@pytest.mark.parametrize("n,h", [(3000, 3), (3000, 5), (7000, 4), (40_000, 2)])
+def test_long_cascade(L, orc, n, h):
+    """A cascade along a path is not run twice (as a band and again level by
+    level): 48 rounds a try at most on top of the peel's own."""
+    n, s, d = strip(n, max(h - 1, 1))
+    og = orc.csr(n, s, d)
+    wcore, wk = orc.core_decompose(og, h)
+    wl = orc.level_stats(og, h, wcore)
+    with L.Graph.from_edges(n, s, d) as g:
+        core, k = g.core_decompose(h)
+        lv = g.level_stats(h)
+        st = L.dsd_peel_stats(g.handle, 0 if h == 2 else 1)
+    assert k == wk and np.array_equal(core, wcore)
+    for a, b in zip(lv, wl):
+        assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
+    assert st["rounds"] >= n // 2 - 8
+    assert st["grid_rounds"] <= st["rounds"] + 4 * 48
