@@ -227,3 +227,40 @@ def test_long_cascade(L, orc, n, h):
         assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
     assert st["rounds"] >= n // 2 - 8
     assert st["grid_rounds"] <= st["rounds"] + 4 * 48
+
+
+@pytest.mark.parametrize("x", [2, 3])
+@pytest.mark.parametrize("graph", ["strips", "path", "er", "power"])
+def test_star_long_cascade(L, graph, x):
+    """A round of the x-star peel that changes little costs little: 2,000 strips of
+    400 vertices (200 rounds; gathered anew each round it took 5.6 times the
+    one-level peel).  The other graphs mix rounds passed on as differences with
+    gathered ones; all equal the one-level peel."""
+    import time
+    if graph == "strips":
+        _, s1, d1 = strip(400, 2)
+        at = 400 * np.arange(2000)[:, None]
+        n, s, d = 800_000, (s1 + at).ravel().astype(np.uint32), (d1 + at).ravel().astype(np.uint32)
+    elif graph == "path":
+        n, s, d = strip(9000, 1)
+    elif graph == "er":
+        n, s, d = gg.er(60_000, 0.0001, 4)
+    else:
+        n, s, d = gg.chung_lu(20_000, 160_000, 2.1, 900.0, 5)
+    best = {}
+    got = {}
+    with L.Graph.from_edges(n, s, d) as g:
+        for limit in (0, 1 << 30):
+            L.dsd_set_peel_tail_limit(limit)
+            try:
+                for _ in range(3):
+                    t = time.perf_counter()
+                    got[limit] = g.pattern_core_decompose(L.DSD_PATTERN_STAR, x)
+                    t = time.perf_counter() - t
+                    best[limit] = min(best.get(limit, t), t)
+            finally:
+                L.dsd_set_peel_tail_limit(1 << 30)
+    for a, b in zip(got[0], got[1 << 30]):
+        assert np.array_equal(a, b)
+    if graph == "strips":
+        assert best[1 << 30] < 2 * best[0]
