@@ -16,9 +16,9 @@ constexpr uint32_t kBandAim = 2048;
 constexpr uint32_t kBandMax = 8192;
 // A cascade longer than kBandRounds is undone likewise: it runs along a path
 // of the graph, one level's worth of rounds or nearly, and phase 2 would run
-// them all again (a strip of 3,000 triangles, h = 3: 1,500 rounds in one level, the call 26.6
-// ms, 20.1 undone after 48).  On the power-law, R-MAT
-// and Erdos-Renyi graphs measured, h = 2..5, no cascade takes more than 30.
+// them all again (a strip of 3,000 triangles, h = 3, 1,500 rounds in one level:
+// the call 26.6 ms, 20.1 undone after 48).  On the power-law, R-MAT and
+// Erdos-Renyi graphs measured, h = 2..5, no cascade takes more than 30.
 constexpr uint32_t kBandRounds = 48;
 // With N vertices left a band aims at sqrt(kBandFill N) of them: a cascade
 // takes 2-5 rounds, so phase 1 runs ~3 N / T rounds for bands of T vertices and

@@ -612,49 +612,6 @@ __device__ __forceinline__ unsigned long long* warp_counts64(uint32_t* buf) {
     return reinterpret_cast<unsigned long long*>(buf + kBatchWarpRows);
 }
 
-// warp_build_rows32 with the bounds of all lists loaded by a lane each and four
-// lists' first entries in flight: a CTA's 32 warps alone do not hide the two
-// dependent loads a list takes otherwise.
-__device__ void warp_rows32_ahead(const uint32_t* C, uint32_t nc, const uint32_t* off,
-                                  const uint32_t* adj, const uint32_t* nb, uint32_t* rows) {
-    const unsigned full = 0xffffffffu, lane = lane_id();
-    const uint32_t cmax = C[nc - 1], m = nc - 1;
-    uint32_t lb = 0, le = 0;
-    if (lane < m) {
-        lb = nb[C[lane]];
-        le = off[C[lane] + 1];
-    }
-    for (uint32_t i0 = 0; i0 < m; i0 += 4) {
-        uint32_t b[4], e[4], y[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint32_t i = i0 + q < m ? i0 + q : m - 1;
-            b[q] = __shfl_sync(full, lb, i);
-            e[q] = __shfl_sync(full, le, i);
-            y[q] = b[q] + lane < e[q] ? adj[b[q] + lane] : kNone;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const uint32_t i = i0 + q;
-            if (i >= m) break;
-            uint32_t bits = 0;
-            for (uint32_t p = b[q];;) {
-                if (y[q] <= cmax) {
-                    const uint32_t pos = (uint32_t)lower_bound_u32(C, nc, y[q]);
-                    if (pos < nc && C[pos] == y[q]) bits |= 1u << pos;
-                }
-                p += 32;
-                if (p >= e[q] || __shfl_sync(full, y[q], 31) > cmax) break;
-                y[q] = p + lane < e[q] ? adj[p + lane] : kNone;
-            }
-            bits = __reduce_or_sync(full, bits);
-            if (lane == 0) rows[i] = bits;
-        }
-    }
-    if (lane == 0) rows[m] = 0;
-    __syncwarp();
-}
-
 // Triangles of G[C], 32 < nc <= kBatchWarpRows, by one warp: the total; each
 // candidate's count in warp_counts64(buf).  C is buf's start.
 __device__ unsigned long long warp_triangles(const uint32_t* C, uint32_t nc, const uint32_t* off,
@@ -881,7 +838,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
                         tot = warp_sum(mine);
                     } else if (d <= 32) {
                         // h = 4: triangles of G[C] by the one-word bitmap DFS
-                        warp_rows32_ahead(C, d, W.roff, W.radj, W.rsplit, rows);
+                        warp_rows32_ahead(C, d, W.roff + 1, W.radj, W.rsplit, rows);
                         tot = warp_dfs32(rows, d, 3, cnt);
                     } else if (d <= kBatchWarpRows) {
                         // h = 4, |C| <= 128: symmetric rows of at most four

@@ -119,6 +119,52 @@ __device__ __forceinline__ void warp_build_rows32(const uint32_t* C, uint32_t nc
     __syncwarp();
 }
 
+// warp_build_rows32 (nc > 0) with the bounds of all lists loaded by a lane each
+// and four lists' first entries in flight: 32 warps an SM alone do not hide the
+// two dependent loads a list takes otherwise.
+template <class OFF>
+__device__ __forceinline__ void warp_rows32_ahead(const uint32_t* C, uint32_t nc, const OFF* ne,
+                                                  const uint32_t* adj, const OFF* nb,
+                                                  uint32_t* rows) {
+    const unsigned full = 0xffffffffu, lane = lane_id();
+    const uint32_t cmax = C[nc - 1], m = nc - 1;
+    OFF lb = 0, le = 0;
+    if (lane < m) {
+        lb = nb[C[lane]];
+        le = ne[C[lane]];
+    }
+    for (uint32_t i0 = 0; i0 < m; i0 += 4) {
+        OFF b[4], e[4];
+        uint32_t y[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t i = i0 + q < m ? i0 + q : m - 1;
+            b[q] = __shfl_sync(full, lb, i);
+            e[q] = __shfl_sync(full, le, i);
+            y[q] = b[q] + lane < e[q] ? adj[b[q] + lane] : kNone;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t i = i0 + q;
+            if (i >= m) break;
+            uint32_t bits = 0;
+            for (OFF p = b[q];;) {
+                if (y[q] <= cmax) {
+                    const uint32_t pos = (uint32_t)lower_bound_u32(C, nc, y[q]);
+                    if (pos < nc && C[pos] == y[q]) bits |= 1u << pos;
+                }
+                p += 32;
+                if (p >= e[q] || __shfl_sync(full, y[q], 31) > cmax) break;
+                y[q] = p + lane < e[q] ? adj[p + lane] : kNone;
+            }
+            bits = __reduce_or_sync(full, bits);
+            if (lane == 0) rows[i] = bits;
+        }
+    }
+    if (lane == 0) rows[m] = 0;
+    __syncwarp();
+}
+
 // ---------------------------------------------------------------------------
 // Per-candidate credits.  An r-clique listed as positions j1 < ... < jr of C
 // adds one to each member's counter.  The last member of a clique is one bit

@@ -93,6 +93,12 @@ constexpr uint32_t kMaxSlices = 8;      // blocks sharing one such vertex
 // short rows of a common neighbourhood (R-MAT scale 15: peel 22 ms against 28
 // with whole rows).  In frontiers above kSmallFront only rows above kLongRow
 // are spread, and those above kHubRow get bitmaps.
+// h >= 3, phase 1: runs of rounds whose frontiers are at most kSoloFront
+// vertices, all with rows of at most kSoloRow entries, go to block 0 alone
+// (solo_rounds), at most kSoloRounds of them between two grid barriers.
+constexpr uint32_t kSoloFront = 64;
+constexpr uint32_t kSoloRow = 16;
+constexpr uint32_t kSoloRounds = 256;
 constexpr uint32_t kLongRow = 128;
 constexpr uint32_t kHubRow = 512;
 constexpr uint32_t kMidWords = 3 + kWarpCand;    // a mid item: v, w, |C|, C
@@ -151,9 +157,11 @@ struct PeelCtrl {
     uint32_t grab[3];               // frontier vertices taken by warps
     uint32_t bgrab[6];              // big items [s] and mid items [3 + s] taken
     uint32_t hubcnt[2];             // bitmap slots asked for, by round parity
+    uint32_t lrow[3];               // some frontier vertex has more than kSoloRow entries
+    uint32_t solo[3];               // after solo_rounds: round, vertices retired, rounds of levels
     uint32_t busy[3];               // phase 2: bands with vertices left, by round
     unsigned long long destroyed;   // phase 1: cliques destroyed so far
-    uint32_t pad0[10];
+    uint32_t pad0[4];
     uint32_t bar_count;
     uint32_t pad1[31];
     uint32_t bar_gen;
@@ -883,11 +891,12 @@ __device__ __forceinline__ const uint32_t* hub_bm_of(const PeelParams& P, uint32
 // parity's hub list).
 template <int HC>
 __device__ __forceinline__ uint32_t front_word(const PeelParams& P, PeelCtrl* c, uint32_t v,
-                                               uint32_t par, uint32_t& cls) {
+                                               uint32_t par, uint32_t slot, uint32_t& cls) {
     cls = 0;
     if (P.deg[v] == 0) return kGone;
     if (HC == 2) return kFront;
     const uint64_t d = P.wend[v] - P.off[v];
+    if (d > kSoloRow) c->lrow[slot] = 1;
     if (HC != 4) cls = d > kLongRow ? 2u : 0u;
     else cls = d > kBitmapMax ? 2u : (d > kTinyRow ? 1u : 0u);
     uint32_t w = kFront | (cls ? kListedBit : 0u);
@@ -933,7 +942,7 @@ __device__ __forceinline__ void hub_bitmaps(const PeelParams& P, uint32_t nhub, 
 // Every clique through frontier vertex v of a short row (at most kTinyRow
 // entries), by one warp: the members of the current set among its neighbours
 // and the (h-1)-cliques they span; C, cnt, rows are the warp's buffers.
-template <int HC>
+template <int HC, bool AHEAD = false>
 __device__ void process_tiny(const PeelParams& P, const NPlus& R, uint32_t v,
                              unsigned long long k, uint32_t* next, uint32_t* next_cnt,
                              uint32_t* C, unsigned* cnt, uint32_t* rows,
@@ -958,7 +967,11 @@ __device__ void process_tiny(const PeelParams& P, const NPlus& R, uint32_t v,
     cnt[lane] = 0;
     __syncwarp();
     if (lane < nc) bytes += 16 + 4ull * (R.ne[C[lane]] - R.nb[C[lane]]);
-    if (r == 2) {
+    if (AHEAD) {
+        // nothing else hides the latency of a round of few vertices
+        warp_rows32_ahead(C, nc, R.ne, R.adj, R.nb, rows);
+        (void)warp_dfs32(rows, nc, r, cnt);
+    } else if (r == 2) {
         const uint32_t cmax = C[nc - 1];
         for (uint32_t i = 0; i + 1 < nc; i++) {
             const uint32_t y = C[i];
@@ -1251,6 +1264,100 @@ __device__ __forceinline__ void process_frontier(
     }
 }
 
+// P2, phase 1, from round r on: frontiers of at most kSoloFront vertices with
+// rows of at most kSoloRow entries, by this block alone, a warp a vertex.  A
+// level that leaves along a path has thousands of such rounds; between grid
+// barriers each takes 10.6 us (a strip of 3,000 triangles), here 3.1: the loads
+// of a vertex's row, of its members' states and of their rows, one after
+// another.  Ends when the next frontier is empty, too large or all that is left, when a cascade has
+// to be looked at, or after kSoloRounds (the other blocks' waits are bounded).
+// F_r is marked on entry; on return F_{r+1} is not, and F_r not retired, as
+// at the top of a round (c->solo, c->fcnt).  key, seg, r_end: the band; a
+// cascade (multi) ends before round r_end.
+template <int NT, int HC>
+__device__ __forceinline__ void solo_rounds(const PeelParams& P, const NPlus& R, uint32_t r,
+                                            uint32_t f, uint32_t retired, uint32_t rs,
+                                            unsigned long long k, bool multi, uint32_t key,
+                                            uint32_t seg, uint32_t r_end, uint32_t* wC,
+                                            unsigned* wCnt, uint32_t* wRows,
+                                            unsigned long long& items,
+                                            unsigned long long& bytes) {
+    __shared__ uint32_t s_cnt, s_late;
+    PeelCtrl* c = P.ctrl;
+    const unsigned lane = lane_id(), wid = warp_id();
+    const uint64_t t0 = threadIdx.x == 0 ? globaltimer_ns() : 0;
+    if (threadIdx.x == 0) s_cnt = s_late = 0;
+    __syncthreads();
+    for (uint32_t step = 1;; step++) {
+        const uint32_t* F = P.front[r % 3];
+        uint32_t* N = P.front[(r + 1) % 3];
+        for (uint32_t i = wid; i < f; i += NT / 32) {
+            const uint32_t v = F[i];
+            if (st_of(P.sl[v]) != kFront) continue;
+            process_tiny<HC, true>(P, R, v, k, N, &s_cnt, wC, wCnt, wRows, bytes);
+            if (lane == 0) {
+                items += P.wend[v] - P.off[v];
+                bytes += 24;
+            }
+        }
+        if (threadIdx.x == 0 && (step & 15u) == 0 && globaltimer_ns() - t0 > P.wait_ns / 4)
+            s_late = 1;
+        __syncthreads();
+        const uint32_t fn = s_cnt;
+        bool stop = fn == 0 || fn > kSoloFront || step == kSoloRounds || s_late ||
+                    retired + f + fn == P.n ||
+                    (multi && (retired + f - seg + fn > kBandMax || r + 1 >= r_end));
+        unsigned long long d = 1;
+        if (threadIdx.x < fn && !stop) {
+            const uint32_t v = N[threadIdx.x];
+            d = P.deg[v];
+            if (P.wend[v] - P.off[v] > kSoloRow) stop = true;
+        }
+        if (__syncthreads_or(stop)) {
+            if (threadIdx.x == 0) {
+                c->fcnt[r % 3] = f;
+                c->fcnt[(r + 1) % 3] = fn;
+                c->solo[0] = r + 1;
+                c->solo[1] = retired;
+                c->solo[2] = rs;
+                // the counters by round, which no round in between has cleared
+                for (int i = 0; i < 3; i++)
+                    c->hcnt[i] = c->vcnt[i] = c->vgrab[i] = c->grab[i] = c->lrow[i] = 0;
+                for (int i = 0; i < 6; i++) c->big_cnt[i] = c->bgrab[i] = 0;
+            }
+            return;
+        }
+        // retire F_r, mark F_{r+1}
+        unsigned long long gone = 0;
+        if (threadIdx.x < f) {
+            const uint32_t v = F[threadIdx.x];
+            gone = P.deg[v];
+            P.sl[v] = kGone;
+            P.band_of[v] = key;
+            P.mem[retired + threadIdx.x] = v;
+            if (!multi) {
+                P.core[v] = k;
+                if (P.rnd) P.rnd[v] = rs;
+            }
+            bytes += 4 + 4 + 8 + 8 + 4 + (P.rnd ? 4 : 0);
+        }
+        if (wid < (kSoloFront + 31) / 32) {
+            gone = warp_sum(gone);
+            if (lane == 0 && gone) atomicAdd(&c->destroyed, gone);
+        }
+        if (threadIdx.x < fn) {
+            P.sl[N[threadIdx.x]] = d ? kFront : kGone;
+            bytes += 4 + 4 + 8 + 16;
+        }
+        retired += f;
+        if (!multi) rs++;
+        f = fn;
+        r++;
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+    }
+}
+
 // P2, phase 2: the frontiers of all bands together (nf vertices), in batches
 // whose items are flattened over the grid.
 template <int NT, int HC>
@@ -1477,7 +1584,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             uint32_t v = 0, cls = 0;
             if (i < fcur) {
                 v = Fcur[i];
-                P.sl[v] = front_word<HC>(P, c, v, r & 1, cls);
+                P.sl[v] = front_word<HC>(P, c, v, r & 1, r % 3, cls);
                 bytes += 4 + 4 + 8 + (HC > 2 ? 16 : 0);
             }
             if (HC > 2) {
@@ -1494,6 +1601,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             }
             c->fcnt[(r + 1) % 3] = 0;
             c->hcnt[(r + 1) % 3] = 0;
+            c->lrow[(r + 1) % 3] = 0;
             c->vcnt[(r + 1) % 3] = 0;
             c->vgrab[(r + 1) % 3] = 0;
             c->grab[(r + 1) % 3] = 0;
@@ -1628,7 +1736,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
                     bytes += 4 + 8;
                     if (P.deg[v] <= k) {
                         in = true;
-                        P.sl[v] = front_word<HC>(P, c, v, r & 1, cls);
+                        P.sl[v] = front_word<HC>(P, c, v, r & 1, r % 3, cls);
                         bytes += 4 + 4 + (HC > 2 ? 16 : 0);
                     }
                 }
@@ -1650,6 +1758,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
                 hub_bitmaps<NT>(P, nhub, r & 1, false, s_pre, s_red, bytes);
                 BARRIER(3);
             }
+        }
+        if (HC > 2 && fcur <= kSoloFront && retired + fcur < P.n && k > 0 && !c->lrow[r % 3]) {
+            if (blockIdx.x == 0)
+                solo_rounds<NT, HC>(P, R1, r, fcur, retired, rs, k, multi,
+                                    2u * nb - (multi ? 1u : 0u), seg, rjump + kBandRounds, wC,
+                                    wCnt, wRows, items, bytes);
+            BARRIER(3);
+            r = *(volatile uint32_t*)&c->solo[0];
+            retired = *(volatile uint32_t*)&c->solo[1];
+            rs = *(volatile uint32_t*)&c->solo[2];
+            continue;
         }
         // when everything left leaves at once there is no count to lower
         if (retired + fcur < P.n) {

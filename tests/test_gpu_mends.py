@@ -264,3 +264,40 @@ def test_star_long_cascade(L, graph, x):
         assert np.array_equal(a, b)
     if graph == "strips":
         assert best[1 << 30] < 2 * best[0]
+
+
+@pytest.mark.parametrize("h,w,count,length", [
+    (3, 2, 1, 3000),     # a vertex at each end a round
+    (3, 2, 32, 300),     # 64 vertices a round: one block's
+    (3, 2, 33, 300),     # 66: the grid's
+    (4, 8, 3, 500),      # rows of 16
+    (4, 9, 3, 500),      # rows of 18
+    (5, 4, 2, 900), (6, 5, 1, 700), (3, 2, 1, 9)])
+def test_narrow_rounds(L, orc, h, w, count, length):
+    """Rounds of a few vertices with short rows run in one block (they took two
+    grid barriers each), on both sides of its limits and beside a larger graph
+    whose rounds are the grid's."""
+    _, s1, d1 = strip(length, w)
+    at = length * np.arange(count)[:, None]
+    n = length * count
+    _, se, de = gg.er(500, 0.1, 3)
+    s = np.concatenate([(s1 + at).ravel(), se + n]).astype(np.uint32)
+    d = np.concatenate([(d1 + at).ravel(), de + n]).astype(np.uint32)
+    for nn, m in ((n, count * s1.size), (n + 500, s.size)):
+        og = orc.csr(nn, s[:m], d[:m])
+        wcore, wk = orc.core_decompose(og, h)
+        wl = orc.level_stats(og, h, wcore)
+        for limit in (1 << 30, 0):
+            L.dsd_set_peel_tail_limit(limit)
+            try:
+                with L.Graph.from_edges(nn, s[:m], d[:m]) as g:
+                    core, k = g.core_decompose(h)
+                    lv = g.level_stats(h)
+                    st = L.dsd_peel_stats(g.handle, 1)
+            finally:
+                L.dsd_set_peel_tail_limit(1 << 30)
+            assert k == wk and np.array_equal(core, wcore)
+            for a, b in zip(lv, wl):
+                assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
+            if nn == n and 2 * count <= 64 and 2 * w <= 16 and length > 100 and limit == 0:
+                assert st["barriers"] < st["rounds"] // 2 + 20
