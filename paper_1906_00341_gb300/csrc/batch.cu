@@ -40,8 +40,8 @@ struct BatchRes {
 
 // Per-CTA workspace (global memory), sized for the largest graph.
 struct Work {
-    uint32_t* k1;       // keys / scratch, E
-    uint32_t* k2;       // keys / scratch, E
+    uint32_t* k1;       // rows being built / scratch, max(E, n)
+    uint32_t* k2;       // scratch; (round, id) keys of the vertices, max(E, n)
     uint32_t* adj;      // rows (caller ids), E
     uint32_t* radj;     // rows (ranks), E
     uint32_t* off;      // n + 1
@@ -88,8 +88,9 @@ __device__ Work carve(uint8_t* base, uint32_t maxn, uint64_t maxe) {
         p = align_up(p + bytes);
         return r;
     };
-    w.k1 = (uint32_t*)take(maxe * 4);
-    w.k2 = (uint32_t*)take(maxe * 4);
+    const uint64_t keys = maxe > maxn ? maxe : (uint64_t)maxn;   // an entry, or a vertex
+    w.k1 = (uint32_t*)take(keys * 4);
+    w.k2 = (uint32_t*)take(keys * 4);
     w.adj = (uint32_t*)take(maxe * 4);
     w.radj = (uint32_t*)take(maxe * 4);
     w.off = (uint32_t*)take(((size_t)maxn + 1) * 4);

@@ -301,3 +301,33 @@ def test_narrow_rounds(L, orc, h, w, count, length):
                 assert np.array_equal(np.asarray(a, np.uint64), np.asarray(b, np.uint64))
             if nn == n and 2 * count <= 64 and 2 * w <= 16 and length > 100 and limit == 0:
                 assert st["barriers"] < st["rounds"] // 2 + 20
+
+
+@pytest.mark.parametrize("kind", ["empty", "sparse", "one_large"])
+def test_batch_more_vertices_than_entries(L, orc, kind):
+    """A batch whose largest graph has more vertices than any has row entries:
+    the (round, id) keys have room (they ran over the rows behind them)."""
+    e = np.zeros(0, np.uint32)
+    rng = np.random.default_rng(5)
+    if kind == "empty":
+        graphs = [(100, e, e, 2 + i % 3) for i in range(9)] + [(1, e, e, 3), (65535, e, e, 4)]
+    elif kind == "sparse":
+        graphs = []
+        for i in range(12):
+            n, k = 300 + 117 * i, 6 + i
+            at = rng.choice(n, k, replace=False).astype(np.uint32)
+            a, b = np.triu_indices(k, 1)
+            graphs.append((n, at[a], at[b], 2 + i % 3))
+    else:
+        _, s, d = gg.er(120, 0.2, 1)
+        graphs = [(120, s, d, h) for h in (2, 3, 4)]
+        graphs += [(60_000, np.array([7, 7, 9], np.uint32), np.array([9, 59_999, 59_999], np.uint32), h)
+                   for h in (3, 4)]
+    b = L.Batch(graphs, want_cores=True)
+    b.run()
+    res = b.results()
+    for (n, s, d, h), r in zip(graphs, res):
+        og = orc.csr(n, s, d)
+        core, k = orc.core_decompose(og, h)
+        assert r["status"] == 0 and r["kmax"] == k and np.array_equal(r["core"], core)
+    b.close()
