@@ -18,10 +18,17 @@ constexpr uint32_t kWarpRow = 256;              // a warp's sort buffer
 constexpr uint32_t kBlockRow = NW * kWarpRow;   // 8192: all of them together
 static_assert(kBlockRow >= kTinyN, "a row without repeats fits the block's buffer");
 
+// Rows above kWarpRow are sorted one after another by the whole block, each
+// some 2 (4 + N / 128) us, padded to N entries (50 rows of 300 entries: the
+// CSR 0.49 ms, 0.21 by the general path; 20 of 1,600: 0.41 and 0.23; 4 of
+// 2,900: 0.28 and 0.39 before its pool): above this sum of 4 + N / 128 the
+// general path sorts them side by side.
+constexpr uint32_t kLongBudget = 192;
+
 struct TinyOut {
     unsigned long long total;   // entries of the cleaned CSR
     uint32_t err;               // an endpoint out of range
-    uint32_t big;               // a row (with repeats) beyond the block's buffer
+    uint32_t big;               // rows (with repeats) too long, or too many long ones
     uint32_t dmax;              // largest |N+(v)|
 };
 
@@ -182,11 +189,16 @@ __global__ void __launch_bounds__(NT, 1) k_tiny_csr(uint32_t n, uint32_t m, cons
         atomicAdd(&pos[v], 1u);
     }
     __syncthreads();
-    for (uint32_t v = threadIdx.x; v < n; v += NT)
-        if (pos[v] > kBlockRow) s_big = 1;
+    for (uint32_t v = threadIdx.x; v < n; v += NT) {
+        const uint32_t l = pos[v];
+        if (l <= kWarpRow) continue;
+        uint32_t N = 512;
+        while (N < l) N <<= 1;
+        atomicAdd(&s_big, l > kBlockRow ? kLongBudget + 1u : 4u + N / 128u);
+    }
     __syncthreads();
-    if (s_err || s_big) {
-        if (threadIdx.x == 0) *out = TinyOut{0, s_err, s_big, 0};
+    if (s_err || s_big > kLongBudget) {
+        if (threadIdx.x == 0) *out = TinyOut{0, s_err, 1, 0};
         return;
     }
     (void)prefix(pos, n, s_w);

@@ -12,7 +12,8 @@ constexpr uint32_t kTinyN = 3072;    // vertices
 constexpr uint32_t kTinyM = 16384;   // edge-list entries
 
 // build_csr's result for n <= kTinyN, m <= kTinyM; *done = false (nothing kept)
-// when a row with its repeats exceeds the block's buffer.
+// when a row with its repeats exceeds the block's buffer, or there are too many
+// long ones.
 dsd_status tiny_csr(dsd_graph* g, uint32_t m, const uint32_t* src, const uint32_t* dst,
                     bool* done);
 // Ranks, relabelled rows and N+ starts from g->rnd; every array allocated.

@@ -331,3 +331,27 @@ def test_batch_more_vertices_than_entries(L, orc, kind):
         core, k = orc.core_decompose(og, h)
         assert r["status"] == 0 and r["kmax"] == k and np.array_equal(r["core"], core)
     b.close()
+
+
+@pytest.mark.parametrize("rows,length,general", [(50, 300, True), (3, 300, False),
+                                                 (20, 1600, True), (1, 3000, False),
+                                                 (16, 1000, False), (17, 1000, True)])
+def test_small_csr_long_rows(L, orc, rows, length, general):
+    """The one-block CSR build leaves graphs with many long rows, which it sorts
+    one after another, to the general path (more than its one launch)."""
+    rng = np.random.default_rng(rows)
+    n = 3050
+    s = np.repeat(np.arange(rows), length)
+    d = np.concatenate([rows + rng.permutation(n - rows)[:length] if length < 1600 or rows == 1
+                        else rng.integers(rows, n, length) for _ in range(rows)])
+    keep = rng.permutation(s.size)[:16384]
+    s, d = s[keep].astype(np.uint32), d[keep].astype(np.uint32)
+    og = orc.csr(n, s, d)
+    with L.Graph.from_edges(n, s, d) as g:
+        off, adj = g.csr()
+        launches = int(L.dsd_phase_stats(g.handle)[2][0])
+        core, _, _ = g.degeneracy_order()
+    assert np.array_equal(off, og.off) and np.array_equal(adj, og.adj)
+    wcore, _ = orc.core_decompose(og, 2)
+    assert np.array_equal(core, wcore)
+    assert (launches > 1) == general
