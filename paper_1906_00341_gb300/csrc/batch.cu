@@ -383,6 +383,7 @@ struct BPeel {
     uint32_t* alive;
     uint32_t* fa;
     uint32_t* fb;
+    uint32_t* tmp;           // n words
     unsigned long long* lk;
     unsigned long long* lm;
     uint32_t* ls;
@@ -469,6 +470,9 @@ __device__ unsigned long long bitem(const BPeel& B, uint32_t v, uint32_t w, unsi
     return tot;
 }
 
+// Rows above this are shared by the block's warps in any round.
+constexpr uint32_t kBatchSharedRow = 128;
+
 // Level-synchronous peel of one graph by one CTA; returns k_max and writes
 // the level records; *nl receives their number.
 template <int NT, int LPR>
@@ -537,17 +541,23 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
             nf = S.cnt1;
         }
         for (uint32_t i = threadIdx.x; i < nf; i += NT) B.st[F[i]] = kFr;
-        if (threadIdx.x == 0) S.cnt2 = 0;   // next frontier size
+        if (threadIdx.x == 0) {
+            S.cnt2 = 0;   // next frontier size
+            S.flag = 0;   // listed rows
+        }
         __syncthreads();
         unsigned long long destroyed = 0;
+        const bool many = nf >= 2 * NW;
         // a frontier vertex of count 0 lies in no clique of the current set:
         // nothing to enumerate (frontier counts do not change here), and at
-        // level 0 that is every one of them
+        // level 0 that is every one of them; asking costs a load that a round of
+        // few vertices would wait for (strips of 300 to 3,000 vertices, h = 2..4:
+        // 9.1 ms, 10.5 when every round asks)
         if (k == 0) {
         } else if (B.h == 2) {
             for (uint32_t i = wid; i < nf; i += NW) {
                 uint32_t v = F[i];
-                if (B.deg[v] == 0) continue;
+                if (many && B.deg[v] == 0) continue;
                 for (uint32_t p = B.off[v] + lane; p < B.off[v + 1]; p += 32) {
                     uint32_t u = B.adj[p];
                     uint32_t s = B.st[u];
@@ -562,17 +572,31 @@ __device__ unsigned long long block_peel(const BPeel& B, Smem<NT>& S, uint32_t* 
         } else {
             uint32_t* C = S.wbuf[wid];
             uint32_t* cnt = C + kBatchMaxDplus;
-            // many frontier vertices: a warp each; few: the block's warps share
-            // the neighbours of one after another
-            const bool each = nf >= 2 * NW;
-            for (uint32_t i = each ? wid : 0; i < nf; i += each ? NW : 1) {
-                uint32_t v = F[i];
-                if (B.deg[v] == 0) continue;
-                for (uint32_t p = B.off[v] + (each ? 0 : wid); p < B.off[v + 1];
-                     p += each ? 1 : NW) {
-                    unsigned long long t = bitem<LPR>(B, v, B.adj[p], k, G, &S.cnt2, C, cnt);
-                    if (lane == 0) destroyed += t;
+            // many frontier vertices: a warp each, those with long rows listed
+            // for after; few, or listed: the block's warps share the neighbours of
+            // one after another (a warp a vertex alone: 16 graphs G(600, 0.4),
+            // h = 4, 665 ms against 536)
+            const uint32_t* list = F;
+            uint32_t nv = nf;
+            for (bool each = many;; each = false) {
+                for (uint32_t i = each ? wid : 0; i < nv; i += each ? NW : 1) {
+                    const uint32_t v = list[i], b = B.off[v], e = B.off[v + 1];
+                    if (each) {
+                        if (B.deg[v] == 0) continue;
+                        if (e - b > kBatchSharedRow) {
+                            if (lane == 0) B.tmp[atomicAdd(&S.flag, 1u)] = v;
+                            continue;
+                        }
+                    }
+                    for (uint32_t p = b + (each ? 0 : wid); p < e; p += each ? 1 : NW) {
+                        unsigned long long t = bitem<LPR>(B, v, B.adj[p], k, G, &S.cnt2, C, cnt);
+                        if (lane == 0) destroyed += t;
+                    }
                 }
+                if (!each) break;
+                __syncthreads();
+                list = B.tmp;
+                nv = S.flag;
             }
         }
         destroyed = bsum<NT>(destroyed, S.red);
@@ -752,6 +776,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
         B2.alive = W.alive;
         B2.fa = W.fa;
         B2.fb = W.fb;
+        B2.tmp = W.k2;
         B2.lk = W.lk;
         B2.lm = W.lm;
         B2.ls = W.ls;
@@ -903,6 +928,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs A) {
             B.alive = W.alive;
             B.fa = W.fa;
             B.fb = W.fb;
+            B.tmp = W.k2;
             B.lk = W.lk;
             B.lm = W.lm;
             B.ls = W.ls;

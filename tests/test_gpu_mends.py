@@ -355,3 +355,27 @@ def test_small_csr_long_rows(L, orc, rows, length, general):
     wcore, _ = orc.core_decompose(og, 2)
     assert np.array_equal(core, wcore)
     assert (launches > 1) == general
+
+
+def test_batch_long_rows(L, orc):
+    """The batch kernel's frontiers: many vertices with rows on both sides of
+    128 entries (a warp each, or listed and shared by the block), few vertices
+    (shared) and hubs beside short rows."""
+    graphs = []
+    for h in (2, 3, 4):
+        graphs += [(400, *gg.er(400, 0.32, h)[1:], h), (300, *gg.er(300, 0.6, h)[1:], h),
+                   (*strip(700, 3), h)]
+        _, s, d = gg.er(900, 0.02, h)
+        hub = np.arange(1, 900, dtype=np.uint32)
+        graphs.append((900, np.concatenate([s, np.zeros(899, np.uint32)]),
+                       np.concatenate([d, hub]), h))
+    b = L.Batch(graphs, want_cores=True)
+    b.run()
+    for (n, s, d, h), r in zip(graphs, b.results()):
+        og = orc.csr(n, s, d)
+        core, k = orc.core_decompose(og, h)
+        lk, ls, lm = orc.level_stats(og, h, core)
+        assert r["status"] == 0 and r["kmax"] == k and np.array_equal(r["core"], core)
+        assert r["nlevels"] == len(lk) and r["kmax_core_size"] == ls[-1]
+        assert r["kmax_core_mu"] == lm[-1]
+    b.close()
