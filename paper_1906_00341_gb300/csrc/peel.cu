@@ -95,10 +95,14 @@ constexpr uint32_t kMaxSlices = 8;      // blocks sharing one such vertex
 // are spread, and those above kHubRow get bitmaps.
 // h >= 3, phase 1: runs of rounds whose frontiers are at most kSoloFront
 // vertices, all with rows of at most kSoloRow entries, go to block 0 alone
-// (solo_rounds), at most kSoloRounds of them between two grid barriers.
+// (solo_rounds), at most kSoloRounds of them between two grid barriers, once a
+// level or cascade has lasted kSoloAfter rounds: the last, narrow rounds of a
+// power law's cascades (2-5 rounds) are as fast on the grid (cl50k, h = 3: 8.02
+// ms; 8.12 with their narrow rounds in one block, 8.08 from the ninth on).
 constexpr uint32_t kSoloFront = 64;
 constexpr uint32_t kSoloRow = 16;
 constexpr uint32_t kSoloRounds = 256;
+constexpr uint32_t kSoloAfter = 8;
 constexpr uint32_t kLongRow = 128;
 constexpr uint32_t kHubRow = 512;
 constexpr uint32_t kMidWords = 3 + kWarpCand;    // a mid item: v, w, |C|, C
@@ -891,12 +895,13 @@ __device__ __forceinline__ const uint32_t* hub_bm_of(const PeelParams& P, uint32
 // parity's hub list).
 template <int HC>
 __device__ __forceinline__ uint32_t front_word(const PeelParams& P, PeelCtrl* c, uint32_t v,
-                                               uint32_t par, uint32_t slot, uint32_t& cls) {
+                                               uint32_t par, uint32_t& cls, bool& lrow) {
     cls = 0;
+    lrow = false;
     if (P.deg[v] == 0) return kGone;
     if (HC == 2) return kFront;
     const uint64_t d = P.wend[v] - P.off[v];
-    if (d > kSoloRow) c->lrow[slot] = 1;
+    lrow = d > kSoloRow;
     if (HC != 4) cls = d > kLongRow ? 2u : 0u;
     else cls = d > kBitmapMax ? 2u : (d > kTinyRow ? 1u : 0u);
     uint32_t w = kFront | (cls ? kListedBit : 0u);
@@ -1582,14 +1587,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
         for (uint64_t base = gwarp * 32; base < fcur && !undo; base += gwarps * 32) {
             uint64_t i = base + lane;
             uint32_t v = 0, cls = 0;
+            bool lrow = false;
             if (i < fcur) {
                 v = Fcur[i];
-                P.sl[v] = front_word<HC>(P, c, v, r & 1, r % 3, cls);
+                P.sl[v] = front_word<HC>(P, c, v, r & 1, cls, lrow);
                 bytes += 4 + 4 + 8 + (HC > 2 ? 16 : 0);
             }
             if (HC > 2) {
                 warp_append(cls == 2, v, &c->hcnt[r % 3], P.heavy);
                 warp_append(cls == 1, v, &c->vcnt[r % 3], P.vlist);
+                if (fcur <= kSoloFront && __any_sync(0xffffffffu, lrow) && lane == 0)
+                    c->lrow[r % 3] = 1;
             }
         }
         if (lead) {
@@ -1729,14 +1737,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
             }
             for (uint64_t base = gwarp * 32; base < left; base += gwarps * 32) {
                 uint64_t i = base + lane;
-                bool in = false;
+                bool in = false, lrow = false;
                 uint32_t v = 0, cls = 0;
                 if (i < left) {
                     v = Aout[i];
                     bytes += 4 + 8;
                     if (P.deg[v] <= k) {
                         in = true;
-                        P.sl[v] = front_word<HC>(P, c, v, r & 1, r % 3, cls);
+                        P.sl[v] = front_word<HC>(P, c, v, r & 1, cls, lrow);
                         bytes += 4 + 4 + (HC > 2 ? 16 : 0);
                     }
                 }
@@ -1744,6 +1752,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
                 if (HC > 2) {
                     warp_append(cls == 2, v, &c->hcnt[r % 3], P.heavy);
                     warp_append(cls == 1, v, &c->vcnt[r % 3], P.vlist);
+                    if (__any_sync(0xffffffffu, lrow) && lane == 0) c->lrow[r % 3] = 1;
                 }
             }
             BARRIER(2);
@@ -1759,7 +1768,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
                 BARRIER(3);
             }
         }
-        if (HC > 2 && fcur <= kSoloFront && retired + fcur < P.n && k > 0 && !c->lrow[r % 3]) {
+        if (HC > 2 && r - rjump >= kSoloAfter && fcur <= kSoloFront && retired + fcur < P.n && k > 0 && !c->lrow[r % 3]) {
             if (blockIdx.x == 0)
                 solo_rounds<NT, HC>(P, R1, r, fcur, retired, rs, k, multi,
                                     2u * nb - (multi ? 1u : 0u), seg, rjump + kBandRounds, wC,
