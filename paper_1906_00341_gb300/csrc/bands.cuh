@@ -69,8 +69,6 @@ __device__ __forceinline__ uint32_t block_scan_count(uint32_t v, uint32_t* wtot,
     return before + x - v;
 }
 
-// pre[0] = 0, pre[i+1] = sum of the current row lengths of F[0..i], for
-// f <= kSmallFront entries (each thread owns kSmallFront/NT consecutive ones).
 // Histogram of count offsets at a jump: 16 bins an octave, exact below 32.
 constexpr uint32_t kBins = 1024;
 constexpr uint32_t kLastBin = 975;      // the bin of 2^64 - 1

@@ -9,8 +9,9 @@
 // separated by __syncthreads only: no grid barrier, no host round trip.
 // Per-graph scratch is a private slice of one workspace per CTA.
 //
-// Graph size limits: n <= 65535 vertices (keys u * n + v fit 32 bits) and,
-// for h = 4, at most 512 higher-ranked neighbours per vertex.
+// Graph size limits: n <= 65535 vertices (a vertex's round and id share a
+// 32-bit key, and long rows are sorted by 16 bits) and, for h = 3 and 4, at
+// most 512 higher-ranked neighbours per vertex.
 #include "cliques.cuh"
 #include "graph.cuh"
 

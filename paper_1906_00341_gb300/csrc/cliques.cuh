@@ -531,7 +531,8 @@ __device__ __forceinline__ unsigned long long warp_edges(const BitmapWarp& B, ui
 // most K * K popc.  In the shared rows a node costs its list, its row loads
 // over the whole width of G[C] (with bank conflicts) and its credits, some 570
 // issue slots on R-MAT scale 18 (h = 5, 27 candidates a node).  That listing
-// call: 49.9 -> 24.7 ms.  Bound by popc and the broadcasts of a node.
+// call: 49.9 -> 24.7 ms.  Bound by instruction issue (77 % of the slots; popc
+// takes 22 % of its pipe).
 template <int K>
 __device__ unsigned warp_triangles_reg(const BitmapWarp& B, uint32_t p) {
     const unsigned full = 0xffffffffu, lane = lane_id();

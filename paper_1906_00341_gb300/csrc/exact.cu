@@ -489,8 +489,10 @@ __device__ __forceinline__ void bfs_arc(const PR& P, uint32_t y, uint64_t e, uin
 // kinds overlap; as launches of their own they ran one after the other, the
 // few big nodes of a round leaving most of the GPU idle.  With heights taken
 // over by the collect a round is three launches, not six: the minimum cut of a
-// 300,000-vertex power law, h = 3, 14.4 -> 11.8 ms a call.  Bound by the
-// launches and the host's waits of some hundred rounds and searches.
+// 300,000-vertex power law, h = 3, 14.4 ms a call before and 11.8 after on one
+// GPU, 18.1 and 13.7 on another, where repeated passes spread by a third.
+// Bound by the launches and the host's waits of some hundred rounds and
+// searches.
 __device__ __forceinline__ uint64_t small_warp() {
     return (uint64_t)(gridDim.x - 1 - blockIdx.x) * (blockDim.x >> 5) + warp_id();
 }

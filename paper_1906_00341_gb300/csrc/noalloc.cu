@@ -318,7 +318,7 @@ extern "C" dsd_status dsd_triangle_degrees_noalloc(uint32_t n, const uint64_t* o
     k_na_light<<<sms * 8, 256, 0, s>>>(n, off, adj, (unsigned long long*)deg,
                                        (unsigned long long*)mu, scratch);
     note_launch();
-    // the large rows first: the medium blocks fill the SMs behind them
+    // in one stream: the medium rows wait for the last large one
     kLarge<<<sms, 1024, kLargeBytes, s>>>(off, adj, (unsigned long long*)deg,
                                           (unsigned long long*)mu, scratch);
     note_launch();

@@ -27,8 +27,8 @@ __global__ void k_row_lengths(uint32_t n, const uint64_t* off, unsigned long lon
 // from the lowest: ranks are then ordered by (round, id).  A block takes a
 // tile of consecutive entries, a warp a run of it in steps of 32, so that
 // equal digits keep their order (match masks within a step, running counts a
-// warp, prefix sums over the warps and, by digit, over the blocks).  Two or
-// three passes whatever the sizes of the rounds; scattering and sorting the
+// warp, prefix sums over the warps and, by digit, over the blocks).  One pass
+// for each started 8 bits of the number of rounds; scattering and sorting the
 // rounds one block each, with a flag scan over all vertices for each large
 // one, took most of the orientation (4M vertices, in all: 12.7 -> 7.4 ms).
 constexpr int kRadixNT = 256, kRadixNW = kRadixNT / 32, kRadixItems = 8;
@@ -236,7 +236,7 @@ dsd_status ensure_order(dsd_graph* g) {
     k_fill_rows<<<grid, 256, 0, s>>>(n, g->old_of, g->new_of, g->off, g->adj, g->roff, g->radj); note_launch();
     CUSTEP(cudaGetLastError());
     {
-        // rows have distinct entries; reuse hist as the (ignored) unique counts
+        // rows have distinct entries: the unique counts are ignored
         uint32_t* ulen = nullptr;
         STEP(dalloc(&ulen, (size_t)n + 1, s));
         st = segmented_sort_unique(g->radj, tmp, g->roff, rdeg, ulen, n, 2 * g->m, s);

@@ -52,6 +52,10 @@
 //   P2  enumerate the cliques each v in F_r destroys; decrement   | barrier
 //   P2b (h >= 4) candidate sets above warp_cand: warp groups and   |
 //       blocks                                                    | barrier
+//   or, h >= 3, a narrow frontier from a level's ninth round on:   |
+//       block 0 runs rounds r, r + 1, ... alone (solo_rounds)     | barrier
+// A cascade that grows too large or too long is undone (kBandMax,
+// kBandRounds) and its first level taken alone.
 // Phase 2, round r: each band has one owner block.
 //   A   retire the band's frontier, find its next one (counts <= k, else
 //       k = the least count: a new level), append it to F_r       | barrier
@@ -312,6 +316,8 @@ __device__ __forceinline__ void lower(const PeelParams& P, uint32_t x, uint32_t 
     }
 }
 
+// pre[0] = 0, pre[i+1] = sum of the current row lengths of F[0..i], for
+// f <= kSmallFront entries (each thread owns kSmallFront/NT consecutive ones).
 // ALL: every entry counts; else a frontier vertex marked gone (count 0) has
 // no items.  Rows of at most `skip` entries count as empty.
 template <int NT, bool ALL = false>
@@ -1768,7 +1774,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_peel(PeelParams P) {
                 BARRIER(3);
             }
         }
-        if (HC > 2 && r - rjump >= kSoloAfter && fcur <= kSoloFront && retired + fcur < P.n && k > 0 && !c->lrow[r % 3]) {
+        if (HC > 2 && r - rjump >= kSoloAfter && fcur <= kSoloFront && k > 0 &&
+            retired + fcur < P.n && !c->lrow[r % 3]) {
             if (blockIdx.x == 0)
                 solo_rounds<NT, HC>(P, R1, r, fcur, retired, rs, k, multi,
                                     2u * nb - (multi ? 1u : 0u), seg, rjump + kBandRounds, wC,
